@@ -201,7 +201,7 @@ int ensure_hierarchy(homo_ctx* c) {
     for (int l = 1; l + 1 < c->nlev; ++l)
       KL(c, HOMO_KC_SETUP, 3, launch_galerkin(c->lev[l], c->lev[l + 1], c->z, c->q, c->stream));
   }
-  KL(c, HOMO_KC_SETUP, 3, launch_coarsest_setup(c));
+  KL(c, HOMO_KC_SETUP, coarsest_setup_kernels(c->mc), launch_coarsest_setup(c));
   if (c->opts.smoother == HOMO_SMOOTH_CHEBYSHEV)   // captured Chebyshev coefficients go stale
     for (auto& gr : c->cg_graph)
       if (gr) {
@@ -884,7 +884,7 @@ int homo_create(homo_ctx** out, int n, double E0, double nu, double p, double Em
       if (l + 1 < nlev) A(&L.t, kPlanes * L.N, "level t");
     }
   }
-  if (rc == HOMO_OK) rc = dalloc(c, &c->A, static_cast<size_t>(c->mc) * c->mc, "coarsest A");
+  if (rc == HOMO_OK) rc = dalloc(c, &c->A, coarsest_work_doubles(c->mc), "coarsest A");
   if (rc == HOMO_OK) rc = dalloc(c, &c->G, static_cast<size_t>(c->mc) * c->mc, "coarsest G");
   c->part_cap = std::max(static_cast<size_t>(16 * 152) * 32,
                          static_cast<size_t>(tiled_grid_blocks(n)) * (kCases + kPlanes));
@@ -896,6 +896,7 @@ int homo_create(homo_ctx** out, int n, double E0, double nu, double p, double Em
   }
   if (rc == HOMO_OK) {
     cudaError_t e = tiled_init();
+    if (e == cudaSuccess) e = coarsest_init();
     if (e != cudaSuccess) rc = cuda_err(c, e, "tiled kernel attributes");
   }
   if (rc == HOMO_OK) {

@@ -774,113 +774,244 @@ __global__ void __launch_bounds__(256) k_prolong(const float* __restrict__ coars
   }
 }
 
-// Dense FP64 matrix of the coarsest stencil: A[3v+r][3w+c] = block (v, d)[r][c],
-// w = v + d wrapped (nc >= 3, so the 27 neighbours are distinct).
-__global__ void k_coarsest_dense(const float* __restrict__ st, int nc, bool cb,
-                                 double* __restrict__ A) {
-  const size_t Nc = static_cast<size_t>(nc) * nc * nc;
-  const int m = 3 * static_cast<int>(Nc);
-  for (size_t it = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; it < 27 * Nc;
-       it += static_cast<size_t>(gridDim.x) * blockDim.x) {
-    const int d = static_cast<int>(it / Nc);
-    const size_t v = it - static_cast<size_t>(d) * Nc;
-    const int x = static_cast<int>(v % nc), y = static_cast<int>((v / nc) % nc),
-              z = static_cast<int>(v / (static_cast<size_t>(nc) * nc));
-    const int dx = d % 3 - 1, dy = (d / 3) % 3 - 1, dz = d / 9 - 1;
-    const size_t w = static_cast<size_t>((x + dx + nc) % nc) +
-                     static_cast<size_t>(nc) * (((y + dy + nc) % nc) + static_cast<size_t>(nc) * ((z + dz + nc) % nc));
+// Coarsest operator (Sec. 4.2 "eight corner vertices ... fixed"): the pinned inverse in FP64
+// by Gauss-Jordan elimination without pivoting (SPD pivots are positive), blocked. Step t
+// of the elimination, with c = column t and r = row t before it and ip = 1 / A[t][t], is
+//   A[i][j] -= (c[i] r[j]) ip,  A[t][j] = r[j] ip,  A[i][t] = -c[i] ip,  A[t][t] = ip.
+// A panel of kSw steps needs its columns, rows and diagonal block step by step, but every
+// other entry only the saved c, r and ip of the panel's steps, which it applies in order:
+// the same FP64 operations on the same values as the unblocked elimination, so G is bitwise
+// the inverse it gives (the solution in the void regions follows a change of the
+// preconditioner in its last bits). The m - 3 unknowns are padded to mp, a multiple of kSw,
+// with an identity block. Per panel two launches: the panel's row and column tiles, then
+// every other tile; the tile of the next diagonal block also runs that block's own steps
+// (look-ahead), so no third launch stands in the chain.
+// Bound by the FP64 pipe (2 per clock and SM; 2 m^3 operations) and, for small m, by the chain
+// of 2 m / kSw launches. Against the one-CTA elimination over global memory it replaced
+// (every step a pass over the matrix by one SM): the setup of a 16^3
+// cell (m = 192) 7.1 -> 0.41 ms, of a 96^3 cell (m = 648) 254.6 -> 2.3 ms.
+constexpr int kSw = 16;
+
+__host__ __device__ inline int sweep_size(int m) { return (m - 3 + kSw - 1) / kSw * kSw; }
+
+// Saved values of one panel: the columns' c (mp x kSw, [row][step]) and the rows' r ([column][step])
+// outside the diagonal block, and the block's own c, r and ip per step.
+struct SweepBuf {
+  double* col;
+  double* row;
+  double* dcol;   // [row in block][step]
+  double* drow;   // [step][column in block]
+  double* ip;
+};
+
+// Dense FP64 matrix of the coarsest stencil without the 3 pinned unknowns: entry
+// (3v + r - 3, 3w + c - 3) = block (v, d)[r][c], w = v + d wrapped (nc >= 3, so the 27
+// neighbours are distinct). A is cleared before; the padding gets a unit diagonal.
+__global__ void __launch_bounds__(256) k_coarsest_dense(const float* __restrict__ st, int nc, bool cb, int mp,
+                                                        double* __restrict__ A) {
+  const int Nc = nc * nc * nc, m0 = 3 * Nc - 3;
+  const int gid = blockIdx.x * blockDim.x + threadIdx.x;
+  for (int i = m0 + gid; i < mp; i += gridDim.x * blockDim.x) A[static_cast<size_t>(i) * mp + i] = 1.0;
+  for (int it = gid; it < 27 * Nc; it += gridDim.x * blockDim.x) {
+    const int d = it / Nc;
+    const int v = it - d * Nc;
+    const int x = v % nc, y = (v / nc) % nc, z = v / (nc * nc);
+    const int xw = (x + d % 3 - 1 + nc) % nc, yw = (y + (d / 3) % 3 - 1 + nc) % nc, zw = (z + d / 9 - 1 + nc) % nc;
+    const int w = xw + nc * (yw + nc * zw);
+    if (v == 0 || w == 0) continue;
     const size_t p = stencil_pos(x, y, z, nc, cb);
     for (int r = 0; r < 3; ++r)
       for (int c = 0; c < 3; ++c)
-        A[(3 * v + r) * m + 3 * w + c] = static_cast<double>(st[static_cast<size_t>(9 * d + 3 * r + c) * Nc + p]);
+        A[static_cast<size_t>(3 * v + r - 3) * mp + 3 * w + c - 3] =
+            static_cast<double>(st[static_cast<size_t>(9 * d + 3 * r + c) * Nc + p]);
   }
 }
 
-// In-place Gauss-Jordan inverse of the SPD block A[3:, 3:] (vertex 0 pinned, Sec. 4.2
-// "eight corner vertices ... fixed"), no pivoting (SPD pivots are positive). One CTA.
-// Row and column 0..2 are zeroed, giving the pinned inverse embedded in m x m.
-__global__ void __launch_bounds__(1024) k_coarsest_invert(double* __restrict__ A, int m,
-                                                          int* __restrict__ status) {
-  __shared__ double piv_row[1536];
-  __shared__ double piv_col[1536];
-  for (int k = 3; k < m; ++k) {
-    const double piv = A[static_cast<size_t>(k) * m + k];
-    if (!(piv > 0.0)) {
-      if (threadIdx.x == 0) *status = 1;
-      return;
-    }
-    const double ip = 1.0 / piv;
-    for (int j = threadIdx.x; j < m; j += blockDim.x) {
-      piv_row[j] = A[static_cast<size_t>(k) * m + j];
-      piv_col[j] = A[static_cast<size_t>(j) * m + k];
-    }
-    __syncthreads();
-    for (size_t e = threadIdx.x; e < static_cast<size_t>(m) * m; e += blockDim.x) {
-      const int i = static_cast<int>(e / m), j = static_cast<int>(e % m);
-      if (i < 3 || j < 3) continue;
-      double val;
-      if (i == k && j == k) val = ip;
-      else if (i == k) val = piv_row[j] * ip;
-      else if (j == k) val = -piv_col[i] * ip;
-      else val = A[e] - piv_col[i] * piv_row[j] * ip;
-      A[e] = val;
-    }
-    __syncthreads();
-  }
-  for (size_t e = threadIdx.x; e < static_cast<size_t>(m) * m; e += blockDim.x) {
-    const int i = static_cast<int>(e / m), j = static_cast<int>(e % m);
-    if (i < 3 || j < 3) A[e] = 0.0;
-  }
+// a - (c r) ip with the product rounded first, as in the elimination step above.
+__device__ __forceinline__ double sweep_update(double a, double c, double r, double ip) {
+  return fma(-__dmul_rn(c, r), ip, a);
 }
 
-// G = P X P with P the projector removing the 3 rigid translations (per-component means):
-// the centred pseudo-inverse of the coarsest operator (Sec. 4.2 null-space removal).
-__global__ void __launch_bounds__(1024) k_coarsest_centre(const double* __restrict__ X, int m,
-                                                          double* __restrict__ G) {
-  extern __shared__ double sh[];          // rowmean[m*3] + tot[9]
-  double* rmean = sh;                     // rmean[i*3 + b] = mean_w X[i][3w+b]
-  double* tot = sh + 3 * m;
+// The kSw steps of diagonal block D (256 threads, one entry each); leaves its final values in
+// D and saves the steps' c, r and ip. A pivot that is not positive sets *status.
+__device__ __forceinline__ void sweep_diagonal(double (&D)[kSw][kSw + 1], double& ip_s, const SweepBuf& b,
+                                               int* status) {
+  const int r = threadIdx.x / kSw, c = threadIdx.x % kSw;
+  for (int t = 0; t < kSw; ++t) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      const double piv = D[t][t];
+      if (!(piv > 0.0)) *status = 1;
+      ip_s = 1.0 / piv;
+      b.ip[t] = ip_s;
+    }
+    __syncthreads();
+    const double ip = ip_s, cv = D[r][t], rv = D[t][c], av = D[r][c];
+    if (c == t) b.dcol[r * kSw + t] = cv;
+    if (r == t) b.drow[t * kSw + c] = rv;
+    double val;
+    if (r == t && c == t) val = ip;
+    else if (r == t) val = rv * ip;
+    else if (c == t) val = -cv * ip;
+    else val = sweep_update(av, cv, rv, ip);
+    __syncthreads();
+    D[r][c] = val;
+  }
+  __syncthreads();
+}
+
+// Diagonal block 0 (one CTA), before the first panel.
+__global__ void __launch_bounds__(kSw * kSw) k_coarsest_first(double* __restrict__ A, int mp, SweepBuf b,
+                                                             int* __restrict__ status) {
+  __shared__ double D[kSw][kSw + 1];
+  __shared__ double ip_s;
+  const int r = threadIdx.x / kSw, c = threadIdx.x % kSw;
+  D[r][c] = A[static_cast<size_t>(r) * mp + c];
+  sweep_diagonal(D, ip_s, b, status);
+  A[static_cast<size_t>(r) * mp + c] = D[r][c];
+}
+
+// Panel k: block b < nb the column tile (b, k), block nb + b the row tile (k, b); b = k skipped
+// (its own steps ran before). Half a warp holds a tile row (column) of kSw values, lane s its
+// value s; step t broadcasts value t within the half warp.
+__global__ void __launch_bounds__(kSw * kSw) k_coarsest_panel(double* __restrict__ A, int mp, int k, SweepBuf b) {
+  const int nb = mp / kSw;
+  const bool is_row = static_cast<int>(blockIdx.x) >= nb;
+  const int tile = is_row ? static_cast<int>(blockIdx.x) - nb : static_cast<int>(blockIdx.x);
+  if (tile == k) return;
+  __shared__ double dv[kSw][kSw + 1], ips[kSw], T[kSw][kSw + 1];
+  const int i = threadIdx.x / kSw, s = threadIdx.x % kSw;
+  // dv[t][s]: what step t multiplies value t with to update value s
+  dv[is_row ? s : i][is_row ? i : s] = is_row ? b.dcol[i * kSw + s] : b.drow[i * kSw + s];
+  if (threadIdx.x < kSw) ips[threadIdx.x] = b.ip[threadIdx.x];
+  const size_t at = is_row ? static_cast<size_t>(kSw * k + i) * mp + kSw * tile + s
+                           : static_cast<size_t>(kSw * tile + i) * mp + kSw * k + s;
+  double v = A[at];
+  if (is_row) {   // lane s of half warp i takes row s of column i
+    T[i][s] = v;
+    __syncthreads();
+    v = T[s][i];
+  } else {
+    __syncthreads();
+  }
+  double save = 0.0;
+#pragma unroll
+  for (int t = 0; t < kSw; ++t) {
+    const double x = __shfl_sync(0xffffffffu, v, t, kSw);
+    if (s == t) {
+      save = x;
+      v = is_row ? x * ips[t] : -x * ips[t];
+    } else {
+      v = sweep_update(v, x, dv[t][s], ips[t]);
+    }
+  }
+  (is_row ? b.row : b.col)[static_cast<size_t>(kSw * tile + i) * kSw + s] = save;
+  if (is_row) {
+    __syncthreads();
+    T[s][i] = v;
+    __syncthreads();
+    v = T[i][s];
+  }
+  A[at] = v;
+}
+
+// Every tile outside panel k's rows and columns: the panel's kSw steps in order. The tile of
+// the next diagonal block then runs that block's own steps into nb.
+__global__ void __launch_bounds__(kSw * kSw) k_coarsest_rest(double* __restrict__ A, int mp, int k, SweepBuf b,
+                                                            SweepBuf next, int* __restrict__ status) {
+  const int bi = blockIdx.y, bj = blockIdx.x;
+  if (bi == k || bj == k) return;
+  __shared__ double cs[kSw][kSw + 1], rs[kSw][kSw + 1], ips[kSw];
+  __shared__ double ip_s;
+  const int r = threadIdx.x / kSw, c = threadIdx.x % kSw;
+  const size_t at = static_cast<size_t>(kSw * bi + r) * mp + kSw * bj + c;
+  cs[r][c] = b.col[static_cast<size_t>(kSw * bi + r) * kSw + c];
+  rs[r][c] = b.row[static_cast<size_t>(kSw * bj + r) * kSw + c];
+  if (threadIdx.x < kSw) ips[threadIdx.x] = b.ip[threadIdx.x];
+  double a = A[at];
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < kSw; ++t) a = sweep_update(a, cs[r][t], rs[c][t], ips[t]);
+  if (bi == k + 1 && bj == k + 1) {
+    __syncthreads();
+    cs[r][c] = a;
+    sweep_diagonal(cs, ip_s, next, status);
+    a = cs[r][c];
+  }
+  A[at] = a;
+}
+
+// The three component means of row i of the embedded inverse X (rows and columns 0..2 zero),
+// rmean[3 i + b], summed in column order; a thread per (row, component).
+__global__ void __launch_bounds__(128) k_coarsest_means(const double* __restrict__ A, int m, int mp,
+                                                        double* __restrict__ rmean) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = t / 3, b = t - 3 * i;
+  if (i >= m) return;
+  double s = 0.0;
+  if (i >= 3) {
+    const double* row = A + static_cast<size_t>(i - 3) * mp + b;
+#pragma unroll 8
+    for (int w = 1; w < m / 3; ++w) s += row[3 * w - 3];
+  }
+  rmean[t] = s / (m / 3);
+}
+
+// G = P X P with P the projector removing the 3 rigid translations (per-component means): the
+// centred pseudo-inverse of the coarsest operator (Sec. 4.2 null-space removal).
+__global__ void __launch_bounds__(256) k_coarsest_centre(const double* __restrict__ A, int m, int mp,
+                                                         const double* __restrict__ rmean, double* __restrict__ G) {
+  extern __shared__ double rms[];   // the 3 m row means: every block sums them in the same order
+  __shared__ double tot[9];
   const int nv = m / 3;
-  for (int i = threadIdx.x; i < m; i += blockDim.x)
-    for (int b = 0; b < 3; ++b) {
-      double s = 0.0;
-      for (int w = 0; w < nv; ++w) s += X[static_cast<size_t>(i) * m + 3 * w + b];
-      rmean[i * 3 + b] = s / nv;
-    }
+  for (int t = threadIdx.x; t < 3 * m; t += blockDim.x) rms[t] = rmean[t];
   __syncthreads();
   if (threadIdx.x < 9) {
     const int a = threadIdx.x / 3, b = threadIdx.x % 3;
     double s = 0.0;
-    for (int v = 0; v < nv; ++v) s += rmean[(3 * v + a) * 3 + b];
+    for (int v = 0; v < nv; ++v) s += rms[(3 * v + a) * 3 + b];
     tot[threadIdx.x] = s / nv;
   }
   __syncthreads();
-  for (size_t e = threadIdx.x; e < static_cast<size_t>(m) * m; e += blockDim.x) {
-    const int i = static_cast<int>(e / m), j = static_cast<int>(e % m);
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < m * m; e += gridDim.x * blockDim.x) {
+    const int i = e / m, j = e - i * m;
     const int a = i % 3, b = j % 3;
-    // X symmetric: column mean of column j over rows of component a = rmean[j][a]
-    G[e] = X[e] - rmean[i * 3 + b] - rmean[j * 3 + a] + tot[a * 3 + b];
+    const double x = i < 3 || j < 3 ? 0.0 : A[static_cast<size_t>(i - 3) * mp + j - 3];
+    // X symmetric: column mean of column j over rows of component a = rms[j][a]
+    G[e] = x - rms[3 * i + b] - rms[3 * j + a] + tot[3 * a + b];
   }
 }
 
-// x = G b for the 6 cases (FP64 dot products), one warp per output row.
-__global__ void __launch_bounds__(256) k_coarsest_apply(const double* __restrict__ G, int m,
+// x = G b for the 6 cases (FP64 dot products), one warp per output row for all cases: G is
+// read once and the right-hand sides are converted to FP64 once per CTA (a conversion
+// costs as much of the narrow FP64 pipe as a multiply-add). Two rows per CTA spread the
+// FP64 work (2 operations per clock and SM) over more SMs.
+constexpr int kApplyBlock = 64;
+
+__global__ void __launch_bounds__(kApplyBlock) k_coarsest_apply(const double* __restrict__ G, int m,
                                                         const float* __restrict__ b,
                                                         float* __restrict__ x) {
+  extern __shared__ double bs[];   // [case][j]
   const int nv = m / 3;
+  for (int t = threadIdx.x; t < kCases * m; t += blockDim.x) {
+    const int c = t / m, j = t - c * m;
+    bs[t] = static_cast<double>(b[static_cast<size_t>(3 * c + j % 3) * nv + j / 3]);
+  }
+  __syncthreads();
   const int lane = threadIdx.x & 31;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nwarps = (gridDim.x * blockDim.x) >> 5;
-  for (int row = warp; row < kCases * m; row += nwarps) {
-    const int c = row / m, i = row % m;
-    double s = 0.0;
-    for (int j = lane; j < m; j += 32) {
-      const int w = j / 3, k = j % 3;
-      s += G[static_cast<size_t>(i) * m + j] * static_cast<double>(b[static_cast<size_t>(3 * c + k) * nv + w]);
-    }
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (i >= m) return;
+  double s[kCases] = {};
+  for (int j = lane; j < m; j += 32) {
+    const double g = G[static_cast<size_t>(i) * m + j];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) x[static_cast<size_t>(3 * c + i % 3) * nv + i / 3] = static_cast<float>(s);
+    for (int c = 0; c < kCases; ++c) s[c] = fma(g, bs[c * m + j], s[c]);
+  }
+#pragma unroll
+  for (int c = 0; c < kCases; ++c) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s[c] += __shfl_down_sync(0xffffffffu, s[c], o);
+    if (lane == 0) x[static_cast<size_t>(3 * c + i % 3) * nv + i / 3] = static_cast<float>(s[c]);
   }
 }
 
@@ -1136,28 +1267,48 @@ cudaError_t launch_prolong_add(int nf, const float* coarse, float* fine, int ove
   return cudaGetLastError();
 }
 
+size_t coarsest_work_doubles(int m) {   // A, two sets of saved panel values, row means
+  const size_t mp = static_cast<size_t>(sweep_size(m));
+  return mp * mp + 2 * (2 * mp * kSw + 2 * kSw * kSw + kSw) + 3 * static_cast<size_t>(m);
+}
+
+int coarsest_setup_kernels(int m) { return 4 + 2 * (sweep_size(m) / kSw); }
+
 cudaError_t launch_coarsest_setup(homo_ctx* c) {
   const Level& L = c->lev[c->nlev - 1];
-  const int m = c->mc;
-  cudaError_t e = cudaMemsetAsync(c->A, 0, sizeof(double) * m * m, c->stream);
+  const int m = c->mc, mp = sweep_size(m), np = mp / kSw;
+  double* at = c->A + static_cast<size_t>(mp) * mp;
+  SweepBuf buf[2];
+  for (SweepBuf& b : buf) {
+    b = {at, at + mp * kSw, at + 2 * mp * kSw, at + 2 * mp * kSw + kSw * kSw, at + 2 * mp * kSw + 2 * kSw * kSw};
+    at = b.ip + kSw;
+  }
+  double* rmean = at;
+  cudaError_t e = cudaMemsetAsync(c->A, 0, sizeof(double) * mp * mp, c->stream);
   if (e != cudaSuccess) return e;
-  k_coarsest_dense<<<grid_for(27 * L.N, 256), 256, 0, c->stream>>>(L.st, L.n, L.colour_blocked, c->A);
   int* status = reinterpret_cast<int*>(c->scal + S_OC + 63);
   e = cudaMemsetAsync(status, 0, sizeof(int), c->stream);
   if (e != cudaSuccess) return e;
-  k_coarsest_invert<<<1, 1024, 0, c->stream>>>(c->A, m, status);
-  const size_t shm = sizeof(double) * (3 * m + 9);
-  e = cudaFuncSetAttribute(k_coarsest_centre, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(shm));
-  if (e != cudaSuccess) return e;
-  k_coarsest_centre<<<1, 1024, shm, c->stream>>>(c->A, m, c->G);
+  k_coarsest_dense<<<grid_for(27 * L.N, 256), 256, 0, c->stream>>>(L.st, L.n, L.colour_blocked, mp, c->A);
+  k_coarsest_first<<<1, kSw * kSw, 0, c->stream>>>(c->A, mp, buf[0], status);
+  for (int k = 0; k < np; ++k) {
+    k_coarsest_panel<<<2 * np, kSw * kSw, 0, c->stream>>>(c->A, mp, k, buf[k & 1]);
+    k_coarsest_rest<<<dim3(np, np), kSw * kSw, 0, c->stream>>>(c->A, mp, k, buf[k & 1], buf[(k + 1) & 1], status);
+  }
+  k_coarsest_means<<<(3 * m + 127) / 128, 128, 0, c->stream>>>(c->A, m, mp, rmean);
+  k_coarsest_centre<<<std::min(grid_for(static_cast<size_t>(m) * m, 256), 304), 256, sizeof(double) * 3 * m, c->stream>>>(
+      c->A, m, mp, rmean, c->G);
   return cudaGetLastError();
 }
 
+cudaError_t coarsest_init() {   // shared-memory limit, before any capture
+  return cudaFuncSetAttribute(k_coarsest_apply, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(sizeof(double) * kCases * 1536));
+}
+
 cudaError_t launch_coarsest_apply(const homo_ctx* c, const float* b, float* x) {
-  const int rows = kCases * c->mc;
-  const int blocks = (rows * 32 + 255) / 256;
-  k_coarsest_apply<<<blocks < 1216 ? blocks : 1216, 256, 0, c->stream>>>(c->G, c->mc, b, x);
+  const int m = c->mc;
+  k_coarsest_apply<<<(m * 32 + kApplyBlock - 1) / kApplyBlock, kApplyBlock, sizeof(double) * kCases * m, c->stream>>>(c->G, m, b, x);
   return cudaGetLastError();
 }
 

@@ -138,7 +138,7 @@ struct homo_ctx {
   homo::Level lev[homo::kMaxLevels];
   std::vector<float> hBf;    // level-1 Galerkin tables (host), 8 * 576 floats
   int nc = 0, mc = 0;        // coarsest cells per axis, 3*nc^3
-  double* A = nullptr;       // mc*mc FP64 work (coarsest)
+  double* A = nullptr;       // FP64 work of the coarsest inverse (coarsest_work_doubles(mc))
   double* G = nullptr;       // mc*mc FP64 centred pseudo-inverse of the coarsest operator
 
   double* part = nullptr;    // reduction partials
@@ -283,6 +283,10 @@ int coarse_cluster_size();
 cudaError_t launch_restrict(int nf, const float* fine, float* coarse, cudaStream_t s);
 cudaError_t launch_prolong_add(int nf, const float* coarse, float* fine, int overwrite,
                                cudaStream_t s);
+// doubles of homo_ctx::A and kernels launched for a coarsest matrix of m unknowns
+size_t coarsest_work_doubles(int m);
+int coarsest_setup_kernels(int m);
+cudaError_t coarsest_init();   // kernel attributes on the current device (before any capture)
 cudaError_t launch_coarsest_setup(homo_ctx* c);
 cudaError_t launch_coarsest_apply(const homo_ctx* c, const float* b, float* x);
 cudaError_t launch_stencil_export(const Level& L, float* out, cudaStream_t s);
