@@ -382,14 +382,14 @@ int homo_autotune(homo_ctx* ctx, int flags, int* gs_cases, int* gs_block, double
 
 /* Coarse-level Gauss-Seidel kernels (Eq. 15-16 on levels >= 1). All four forms compute
  * bitwise the same iterates; they differ in how the work reaches the GPU:
- *  - levels with at most resident_max_n cells per axis (FP32 stencils, and only where the
- *    shared memory suffices: up to 16^3 with 16-CTA clusters): every sweep of one
- *    smoothing phase (the pre- or post-smoothing sweeps of a V-cycle, or the single sweep
- *    of homo_smooth) is one launch of six thread-block clusters, one per load case. Each
- *    CTA holds a copy of its case's displacement in shared memory, writes the updates of
- *    its own vertices into every copy of the cluster, and streams the stencil rows of its
- *    vertices for the next colour while the current one computes; the colour passes are
- *    separated by the cluster's hardware barrier (default 16);
+ *  - levels with at most resident_max_n cells per axis (up to 16^3, where the device launches
+ *    clusters large enough): every sweep of one smoothing phase (the pre- or post-smoothing
+ *    sweeps of a V-cycle, or the single sweep of homo_smooth) is one launch of six
+ *    thread-block clusters, one per load case. Each CTA holds a copy of its case's
+ *    displacement in shared memory and the stencil rows of its own vertices in registers
+ *    (half of them in shared memory at 14^3 and 16^3), and writes each update into the copies
+ *    of the CTAs that read it; the colour passes are separated by the cluster's hardware
+ *    barrier (default 16);
  *  - other levels with at most cluster_max_n cells per axis: the same per-case cluster
  *    launch, reading the displacement and stencils through L2 (default 32);
  *  - larger levels with at most split_max_n cells per axis: one launch per colour pass with

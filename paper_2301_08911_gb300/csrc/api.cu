@@ -232,8 +232,8 @@ int smooth_level(homo_ctx* c, int l, bool reverse, const float* f, float* x, boo
 }
 
 // sweeps 8-colour sweeps on level l; first: the first sweep starts from x = 0. A small
-// coarse level runs them all as one launch of per-case clusters (its displacement resident
-// in shared memory up to gs_res_n cells per axis, read through L2 up to gs_fuse_n), larger
+// coarse level runs them all as one launch of per-case clusters (displacement and stencil on
+// the chip up to gs_res_n cells per axis, read through L2 up to gs_fuse_n), larger
 // levels one launch per colour (the per-colour launches of the small levels are mostly
 // launch and load latency).
 int smooth_level_sweeps(homo_ctx* c, int l, bool reverse, const float* f, float* x, int sweeps,

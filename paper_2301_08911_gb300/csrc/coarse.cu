@@ -401,184 +401,237 @@ __global__ void __launch_bounds__(kClusterBlock) k_coarse_gs_cluster(const T* __
   }
 }
 
-// ---- shared-memory-resident form of the small-level smoother
-// Six clusters again, one per load case; the CTAs of a cluster split each colour's
-// vertices into ranges of at most kResVerts (CTA r owns positions [r Mper, (r+1) Mper) of
-// every colour, three threads per vertex, one per block row). Every CTA keeps a full copy of its case's
-// displacement in shared memory, so all neighbour reads of a pass are shared-memory
-// loads; the owner of a vertex writes its new value into every CTA's copy (distributed
-// shared memory) before the cluster barrier that ends the pass. Each CTA streams the
-// stencil rows of its own vertices for the next colour pass into a second buffer with
-// asynchronous copies while the current pass computes, and keeps the right-hand side of
-// its vertices for all colours. The arithmetic per vertex is gs_item's, on the same
-// values in the same order: bitwise the iterates of the other forms.
-constexpr int kResVerts = 64;     // vertices per colour per CTA, at most
-constexpr int kResThreads = 256;  // threads per CTA: all stage, 3 x kResVerts compute (a row each)
+// ---- on-chip form of the small-level smoother
+// Six clusters again, one per load case; CTA `rank` of a cluster owns positions
+// [rank Mper, (rank + 1) Mper) of every colour. Everything a phase reads twice stays on the
+// chip: each CTA keeps a copy of its case's displacement in shared memory (16 bytes per
+// vertex, colour by colour, so that a quarter warp's neighbour loads are one conflict-free
+// 128-byte line), and the stencil rows of its own vertices in registers, one block row of
+// one vertex (26 x 3 values) per thread and colour. A pass is then the 78-FMA chain of a
+// row on register and shared-memory operands, three shuffles that gather the vertex's
+// rows, the solve with factors made once per phase, one 16-byte store per CTA that reads
+// the vertex, and the cluster barrier: bound by that chain and the barrier, not by loads.
+// kRegColours colour groups of threads: with 8 (Mper <= 16) a group serves one colour; with
+// 4 (Mper <= 32) it serves colours g and g + 4, the second one's rows in shared memory (the
+// registers hold 512 x 78 values, half of what 32 vertices of 8 colours need).
+// Warps of a group: 8 vertices each, lane = 8 row + vertex (lanes 24..31 idle).
+// The arithmetic per vertex is gs_item's, on the same values in the same order (the first
+// sweep from zero multiplies the zeros it skips elsewhere): bitwise the same iterates.
+// Against streaming each pass's rows through shared memory (three threads per vertex, one pass
+// 3.0 / 3.7 us at 8^3 / 16^3, the copies' issue and waits): one
+// sweep at 16^3 / 8^3, launch and setup included, 45.2 / 30.9 -> 22.7 / 16.9 us,
+// the coarse smoothing of a 64^3 V-cycle 810 -> 340 us, of a mixed 256^3 one 16.1 -> 5.3 ms.
+constexpr int kResThreads = 512;
+constexpr int kResRow = 84;       // floats per stored row: 78 rounded up, quarter warps on distinct banks
+constexpr int kResTargets = 6;    // a lane's share (a third) of at most 16 CTAs
 
 __device__ __forceinline__ unsigned smem_addr(const void* p) {
   return static_cast<unsigned>(__cvta_generic_to_shared(p));
 }
 
-__device__ __forceinline__ void cp_async_f4(float* dst, const float* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
-__device__ __forceinline__ void cp_async_f16(float* dst, const float* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-}
-
-// value into the same shared-memory offset of CTA `rank` of the cluster
-__device__ __forceinline__ void st_cluster_f32(const float* local, unsigned rank, float v) {
+// address of the same shared-memory location in CTA `rank` of the cluster
+__device__ __forceinline__ unsigned map_rank(unsigned local, unsigned rank) {
   unsigned remote;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_addr(local)), "r"(rank));
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(v) : "memory");
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
+  return remote;
 }
 
-// Shared memory of k_coarse_gs_resident in floats: the case's displacement (3N), two
-// stencil buffers (2 x 243 x Mper) and the owned right-hand sides (8 x 3 x Mper).
-__host__ __device__ inline size_t resident_smem_floats(size_t N, int Mper) {
-  return 3 * N + 2 * static_cast<size_t>(kStencil) * Mper + 24 * static_cast<size_t>(Mper);
+// Dynamic shared memory: displacement (4 N floats), factors (8 colours x Mper x 8 floats) and,
+// with 4 colour groups, the rows of colours 4..7.
+__host__ __device__ inline size_t resident_smem_bytes(size_t N, int Mper, int groups) {
+  return sizeof(float) * (4 * N + 64 * static_cast<size_t>(Mper) +
+                          (groups == 4 ? static_cast<size_t>(4) * Mper * 3 * kResRow : 0));
 }
 
-// Stage the stencil rows of positions colour*Nh + m0 .. + mcount of every plane: 16-byte
-// copies when every segment is 16-byte aligned (vec), 4-byte copies otherwise. Thread t
-// copies chunk t % per of planes t / per, t / per + blockDim / per, ... (per = chunks per
-// plane; the quotient is taken once per launch, not per copy).
-struct StageMap {
-  int per, plane0, step, chunk;   // step 0: the thread copies nothing
+// Index parts of the neighbours of half-grid position (i, j, k) of a colour in the
+// colour-blocked displacement: neighbour d sits at X[dx + 1] + Y[dy + 1] + Z[dz + 1].
+struct ResNb {
+  int X[3], Y[3], Z[3];
 };
 
-__device__ __forceinline__ StageMap stage_map(int mcount, bool vec) {
-  StageMap m;
-  m.per = vec ? (mcount >> 2) : mcount;
-  const int planes_per_pass = m.per > 0 ? static_cast<int>(blockDim.x) / m.per : 0;
-  if (planes_per_pass == 0 || static_cast<int>(threadIdx.x) >= planes_per_pass * m.per) {
-    m.plane0 = 0;
-    m.step = 0;
-    m.chunk = 0;
-    return m;
-  }
-  m.plane0 = static_cast<int>(threadIdx.x) / m.per;
-  m.chunk = static_cast<int>(threadIdx.x) - m.plane0 * m.per;
-  m.step = planes_per_pass;
-  return m;
+__device__ __forceinline__ ResNb res_nb(unsigned m, int colour, int h, int Nh) {
+  int i, j, k;
+  decode3(m, static_cast<unsigned>(h), i, j, k);
+  const int cx = colour & 1, cy = (colour >> 1) & 1, cz = colour >> 2;
+  ResNb nb;
+  // an even coordinate 2i has neighbours 2(i-1)+1 and 2i+1, an odd one 2i+1 has 2i and 2(i+1)
+  auto lo = [h](int a, int odd) { return odd ? a : (a == 0 ? h - 1 : a - 1); };
+  auto hi = [h](int a, int odd) { return odd ? (a == h - 1 ? 0 : a + 1) : a; };
+  nb.X[1] = cx * Nh + i;
+  nb.X[0] = (1 - cx) * Nh + lo(i, cx);
+  nb.X[2] = (1 - cx) * Nh + hi(i, cx);
+  nb.Y[1] = 2 * cy * Nh + h * j;
+  nb.Y[0] = 2 * (1 - cy) * Nh + h * lo(j, cy);
+  nb.Y[2] = 2 * (1 - cy) * Nh + h * hi(j, cy);
+  nb.Z[1] = 4 * cz * Nh + h * h * k;
+  nb.Z[0] = 4 * (1 - cz) * Nh + h * h * lo(k, cz);
+  nb.Z[2] = 4 * (1 - cz) * Nh + h * h * hi(k, cz);
+  return nb;
 }
 
-__device__ __forceinline__ void stage_rows(const float* __restrict__ st, size_t N, unsigned Nh, int colour,
-                                           unsigned m0, int Mper, bool vec, const StageMap& sm_, float* buf) {
-  if (sm_.step > 0) {
-    const int j = vec ? (sm_.chunk << 2) : sm_.chunk;
-    const float* src = st + static_cast<size_t>(colour) * Nh + m0 + j + static_cast<size_t>(sm_.plane0) * N;
-    float* dst = buf + sm_.plane0 * Mper + j;
-    const size_t src_step = static_cast<size_t>(sm_.step) * N;
-    const int dst_step = sm_.step * Mper;
-    for (int plane = sm_.plane0; plane < kStencil; plane += sm_.step, src += src_step, dst += dst_step) {
-      if (vec) cp_async_f16(dst, src);
-      else cp_async_f4(dst, src);
-    }
+// b minus the off-diagonal part of one block row: the FMA chain of the row, in the order of
+// every other form. row(e) is neighbour e's three values (e = 0..25, the diagonal skipped).
+template <typename Row>
+__device__ __forceinline__ float res_chain(float b, const float4* us, const ResNb& nb, Row row) {
+#pragma unroll
+  for (int d = 0; d < 27; ++d) {
+    if (d == 13) continue;
+    const int e = d < 13 ? d : d - 1;
+    const float4 u = us[nb.X[d % 3] + nb.Y[(d / 3) % 3] + nb.Z[d / 9]];
+    b = fmaf(-row(3 * e + 2), u.z, fmaf(-row(3 * e + 1), u.y, fmaf(-row(3 * e), u.x, b)));
   }
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
+  return b;
 }
 
-__global__ void __launch_bounds__(kResThreads) k_coarse_gs_resident(const float* __restrict__ st,
-                                                                  const float* __restrict__ f, float* x,
-                                                                  int n, int sweeps, int reverse, int first,
-                                                                  int csize, int Mper, int vec16) {
-  extern __shared__ float sm[];
-  const size_t N = static_cast<size_t>(n) * n * n;
-  const int h = n >> 1;
-  const unsigned Nh = static_cast<unsigned>(h) * h * h;
-  const int c = static_cast<int>(blockIdx.x) / csize;   // load case of this cluster
-  const unsigned rank = blockIdx.x - static_cast<unsigned>(c * csize);
-  const unsigned m0 = rank * static_cast<unsigned>(Mper);
-  const int mcount = m0 >= Nh ? 0 : static_cast<int>(min(static_cast<unsigned>(Mper), Nh - m0));
-  const bool vec = vec16 && (mcount % 4 == 0);   // vec16: st, N, Nh and Mper allow 16-byte segments
-  float* us = sm;                                          // [3][N]
-  float* sb[2] = {us + 3 * N, us + 3 * N + kStencil * Mper};
-  float* fs = sb[1] + kStencil * Mper;                     // [8][3][Mper]
-  const float* xc = x + static_cast<size_t>(3 * c) * N;
+template <typename T, int kGroups>
+__global__ void __launch_bounds__(kResThreads, 1) k_coarse_gs_resident(const T* __restrict__ st,
+                                                                     const float* __restrict__ f, float* x,
+                                                                     int n, int sweeps, int reverse, int first,
+                                                                     int csize, int Mper) {
+  extern __shared__ __align__(16) float sm[];
+  __shared__ unsigned need_s;
+  constexpr int kWarps = kResThreads / 32 / kGroups;       // warps (8 vertices each) per group
+  const int N = n * n * n, h = n >> 1, Nh = h * h * h;
+  const int c = static_cast<int>(blockIdx.x) / csize;      // load case of this cluster
+  const int rank = static_cast<int>(blockIdx.x) - c * csize;
+  const int m0 = rank * Mper;
+  const int mcount = m0 >= Nh ? 0 : min(Mper, Nh - m0);
+  float4* us = reinterpret_cast<float4*>(sm);
+  float4* fac = us + N;                                    // [8][Mper][2]: l10 l20 l21 i0 | i1 i2
+  float* rows = sm + 4 * N + 64 * Mper;                    // [4][Mper][3][kResRow]
   const float* fc = f + static_cast<size_t>(3 * c) * N;
-  const int r = static_cast<int>(threadIdx.x) / kResVerts;   // row of the vertex's block rows (3: stage only)
-  const int j = static_cast<int>(threadIdx.x) - r * kResVerts;
-  __shared__ float rows_s[3][kResVerts];
+  float* xc = x + static_cast<size_t>(3 * c) * N;
+  const int warp = static_cast<int>(threadIdx.x) >> 5, lane = static_cast<int>(threadIdx.x) & 31;
+  const int group = warp / kWarps;
+  const int r = lane >> 3, jj = lane & 7;                  // block row (3: idle) and vertex in the warp
+  const int j = (warp - group * kWarps) * 8 + jj;
+  const bool own = r < 3 && j < mcount;
 
-  for (size_t i = threadIdx.x; i < 3 * N; i += blockDim.x) us[i] = __ldcg(xc + i);
-  for (int i = threadIdx.x; i < 8 * mcount; i += blockDim.x) {
-    const int colour = i / mcount, jj = i - colour * mcount;
-    int a, b, cc;
-    decode3(m0 + jj, static_cast<unsigned>(h), a, b, cc);
-    const size_t v = static_cast<size_t>(2 * a + (colour & 1)) +
-                     static_cast<size_t>(n) * ((2 * b + ((colour >> 1) & 1)) + static_cast<size_t>(n) * (2 * cc + (colour >> 2)));
-#pragma unroll
-    for (int k = 0; k < 3; ++k) fs[(colour * 3 + k) * Mper + jj] = __ldg(fc + k * N + v);
+  // displacement, colour by colour (zero where the first sweep starts from zero)
+  if (threadIdx.x == 0) need_s = 0u;
+  const bool from_zero = first && !reverse;
+  for (int v = threadIdx.x; v < N; v += kResThreads) {
+    int a, b, d;
+    decode3(static_cast<unsigned>(v), static_cast<unsigned>(n), a, b, d);
+    const int pos = ((a & 1) + 2 * (b & 1) + 4 * (d & 1)) * Nh + (a >> 1) + h * ((b >> 1) + h * (d >> 1));
+    us[pos] = from_zero ? make_float4(0.f, 0.f, 0.f, 0.f)
+                        : make_float4(__ldcg(xc + v), __ldcg(xc + N + v), __ldcg(xc + 2 * static_cast<size_t>(N) + v), 0.f);
   }
-  const int total = sweeps * 8;
-  const StageMap smap = stage_map(mcount, vec);
-  stage_rows(st, N, Nh, reverse ? 7 : 0, m0, Mper, vec, smap, sb[0]);
-  cluster_barrier();   // every copy of the displacement is loaded before any owner writes into it
-
-  for (int pass = 0; pass < total; ++pass) {
-    const int k = pass & 7;
-    const int colour = reverse ? 7 - k : k;
-    const int fz = first && pass < 8 && !reverse ? 1 : 0;
-    if (pass + 1 < total) {
-      const int kn = (pass + 1) & 7;
-      stage_rows(st, N, Nh, reverse ? 7 - kn : kn, m0, Mper, vec, smap, sb[(pass + 1) & 1]);
-    } else {
-      asm volatile("cp.async.commit_group;\n" ::: "memory");
-    }
-    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-    __syncthreads();
-    // thread (row r, vertex j): the FMA chain of row r of the vertex's three rows (the
-    // rows are independent chains); the solve gathers the three rows through rows_s
-    const int cx = colour & 1, cy = (colour >> 1) & 1, cz = colour >> 2;
-    size_t v = 0;
-    if (r < 3 && j < mcount) {
-      const float* S_ = sb[pass & 1];
-      int a, b, cc;
-      decode3(m0 + j, static_cast<unsigned>(h), a, b, cc);
-      const int X = 2 * a + cx, Y = 2 * b + cy, Z = 2 * cc + cz;
-      v = static_cast<size_t>(X) + static_cast<size_t>(n) * (Y + static_cast<size_t>(n) * Z);
-      const Nb nb = make_nb(X, Y, Z, n);
-      float br = fs[(colour * 3 + r) * Mper + j];
+  // this thread's stencil rows and right-hand sides
+  float A[78], rhs[8 / kGroups];
 #pragma unroll
-      for (int d = 0; d < 27; ++d) {
-        if (d == 13) continue;
-        const int dx = d % 3 - 1, dy = (d / 3) % 3 - 1, dz = d / 9 - 1;
-        const int odd = (dx != 0) | ((dy != 0) << 1) | ((dz != 0) << 2);
-        if (fz && (colour ^ odd) > colour) continue;
-        const float* Ad = S_ + (9 * d + 3 * r) * Mper + j;
-        const size_t w = static_cast<size_t>(nb.X[dx + 1] + nb.Y[dy + 1] + nb.Z[dz + 1]);
-        br = fmaf(-Ad[2 * Mper], us[2 * N + w], fmaf(-Ad[Mper], us[N + w], fmaf(-Ad[0], us[w], br)));
+  for (int q = 0; q < 8 / kGroups; ++q) rhs[q] = 0.f;
+#pragma unroll
+  for (int e = 0; e < 78; ++e) A[e] = 0.f;
+  if (own) {
+    int a, b, d;
+    decode3(static_cast<unsigned>(m0 + j), static_cast<unsigned>(h), a, b, d);
+#pragma unroll
+    for (int q = 0; q < 8 / kGroups; ++q) {
+      const int colour = group + 4 * q;
+      const size_t p = static_cast<size_t>(colour) * Nh + m0 + j;
+      const size_t v = static_cast<size_t>(2 * a + (colour & 1)) +
+                       static_cast<size_t>(n) * ((2 * b + ((colour >> 1) & 1)) + static_cast<size_t>(n) * (2 * d + (colour >> 2)));
+      rhs[q] = __ldg(fc + static_cast<size_t>(r) * N + v);
+      float* dst = rows + ((static_cast<size_t>(group) * Mper + j) * 3 + r) * kResRow;
+#pragma unroll
+      for (int e = 0; e < 26; ++e)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const float val = ld_st(st + static_cast<size_t>(9 * (e < 13 ? e : e + 1) + 3 * r + k) * N + p);
+          if (q == 0) A[3 * e + k] = val;
+          else dst[3 * e + k] = val;
+        }
+      if (r == 0) {
+        float S[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) S[k] = ld_st(st + static_cast<size_t>(9 * 13 + k) * N + p);
+        const Factor3 F = factor3(S);
+        fac[2 * (colour * Mper + j)] = make_float4(F.l10, F.l20, F.l21, F.i0);
+        fac[2 * (colour * Mper + j) + 1] = make_float4(F.i1, F.i2, 0.f, 0.f);
       }
-      rows_s[r][j] = br;
     }
-    __syncthreads();
-    if (r < 3 && j < mcount) {
-      const float* S_ = sb[pass & 1];
-      float S[9];
-#pragma unroll
-      for (int q = 0; q < 9; ++q) S[q] = S_[(9 * 13 + q) * Mper + j];
-      float y0 = rows_s[0][j], y1 = rows_s[1][j], y2 = rows_s[2][j];
-      solve3(factor3(S), y0, y1, y2);
-      const float val = r == 0 ? y0 : (r == 1 ? y1 : y2);
-      float* dst = us + static_cast<size_t>(r) * N + v;
-      *dst = val;
-      for (unsigned t = 0; t < static_cast<unsigned>(csize); ++t)
-        if (t != rank) st_cluster_f32(dst, t, val);
-    }
-    cluster_barrier();
   }
-  // every vertex is owned by one CTA: write the owned values back
-  for (int i = threadIdx.x; i < 8 * mcount; i += blockDim.x) {
-    const int colour = i / mcount, jj = i - colour * mcount;
-    int a, b, cc;
-    decode3(m0 + jj, static_cast<unsigned>(h), a, b, cc);
-    const size_t v = static_cast<size_t>(2 * a + (colour & 1)) +
-                     static_cast<size_t>(n) * ((2 * b + ((colour >> 1) & 1)) + static_cast<size_t>(n) * (2 * cc + (colour >> 2)));
-    float* xo = x + static_cast<size_t>(3 * c) * N + v;
+  __syncthreads();
+  // the CTAs that read this one's vertices: owners of positions at most one half-grid step away
+  for (int t = threadIdx.x; t < 27 * mcount; t += kResThreads) {
+    const int d = t / mcount;
+    int a, b, k;
+    decode3(static_cast<unsigned>(m0 + t - d * mcount), static_cast<unsigned>(h), a, b, k);
+    a = (a + d % 3 - 1 + h) % h;
+    b = (b + (d / 3) % 3 - 1 + h) % h;
+    k = (k + d / 9 - 1 + h) % h;
+    atomicOr(&need_s, 1u << ((a + h * (b + h * k)) / Mper));
+  }
+  __syncthreads();
+  unsigned target[kResTargets];   // displacement copies this lane writes (rows split them), 0: none
 #pragma unroll
-    for (int k = 0; k < 3; ++k) __stcg(xo + k * N, us[k * N + v]);
+  for (int q = 0; q < kResTargets; ++q) target[q] = 0u;
+  {
+    const unsigned need = need_s;
+    const unsigned base = smem_addr(us);
+    int seen = 0;
+    for (int t = 0; t < csize; ++t) {
+      if (!((need >> t) & 1u)) continue;
+#pragma unroll
+      for (int q = 0; q < kResTargets; ++q)
+        if (seen == 3 * q + r) target[q] = map_rank(base, static_cast<unsigned>(t));
+      ++seen;
+    }
+  }
+  cluster_arrive();   // every copy of the displacement is complete before any owner writes into it
+
+  const int total = sweeps * 8;
+  for (int pass = 0; pass < total; ++pass) {
+    const int colour = reverse ? 7 - (pass & 7) : pass & 7;
+    if (colour % kGroups == group) {
+      const ResNb nb = res_nb(static_cast<unsigned>(own ? m0 + j : 0), colour, h, Nh);
+      const float4 f0 = fac[2 * (colour * Mper + (own ? j : 0))], f1 = fac[2 * (colour * Mper + (own ? j : 0)) + 1];
+      const Factor3 F = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y};
+      cluster_wait();
+      float br;
+      if (kGroups == 8 || colour < 4) {
+        br = res_chain(rhs[0], us, nb, [&](int e) { return A[e]; });
+      } else {
+        const float4* row = reinterpret_cast<const float4*>(
+            rows + ((static_cast<size_t>(group) * Mper + (own ? j : 0)) * 3 + (r < 3 ? r : 0)) * kResRow);
+        br = res_chain(rhs[8 / kGroups - 1], us, nb, [&](int e) {
+          const float4 q4 = row[e / 4];   // the compiler merges the loads of one float4
+          return e % 4 == 0 ? q4.x : e % 4 == 1 ? q4.y : e % 4 == 2 ? q4.z : q4.w;
+        });
+      }
+      float y0 = __shfl_sync(0xffffffffu, br, jj), y1 = __shfl_sync(0xffffffffu, br, 8 + jj),
+            y2 = __shfl_sync(0xffffffffu, br, 16 + jj);
+      solve3(F, y0, y1, y2);
+      if (own) {
+        const unsigned off = 16u * static_cast<unsigned>(colour * Nh + m0 + j);
+#pragma unroll
+        for (int q = 0; q < kResTargets; ++q)
+          if (target[q])
+            asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(target[q] + off), "f"(y0),
+                         "f"(y1), "f"(y2), "f"(0.f)
+                         : "memory");
+      }
+    } else {
+      cluster_wait();
+    }
+    cluster_arrive();
+  }
+  cluster_wait();
+  // every vertex is owned by one CTA: write the owned values back
+  for (int i = threadIdx.x; i < 8 * mcount; i += kResThreads) {
+    const int colour = i / mcount, q = i - colour * mcount;
+    int a, b, d;
+    decode3(static_cast<unsigned>(m0 + q), static_cast<unsigned>(h), a, b, d);
+    const size_t v = static_cast<size_t>(2 * a + (colour & 1)) +
+                     static_cast<size_t>(n) * ((2 * b + ((colour >> 1) & 1)) + static_cast<size_t>(n) * (2 * d + (colour >> 2)));
+    const float4 u = us[colour * Nh + m0 + q];
+    __stcg(xc + v, u.x);
+    __stcg(xc + N + v, u.y);
+    __stcg(xc + 2 * static_cast<size_t>(N) + v, u.z);
   }
 }
 
@@ -1090,10 +1143,11 @@ int cluster_fits(int size) {
 std::mutex g_cluster_mu;
 int g_cluster_size[256] = {};    // per device: 0 = not queried, -1 = no cluster launch
 int g_resident_size[256] = {};   // per device: largest resident-form cluster, -1 = none
-constexpr int kResidentSmemMax = 200 * 1024;   // dynamic; the static row scratch comes on top
+constexpr int kResidentSmemMax = 216 * 1024;   // dynamic shared memory of the resident form, at most
 
+template <typename T, int kGroups>
 int resident_fits(int size) {
-  const void* fn = reinterpret_cast<const void*>(k_coarse_gs_resident);
+  const void* fn = reinterpret_cast<const void*>(k_coarse_gs_resident<T, kGroups>);
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, size > 8 ? 1 : 0) != cudaSuccess ||
       cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kResidentSmemMax) != cudaSuccess)
     return 0;
@@ -1113,18 +1167,20 @@ int resident_fits(int size) {
   return count;
 }
 
-// Cluster size and per-CTA vertex count of the resident form on level L, or false when
-// the level does not qualify (BF16 stencil, too many vertices, too much shared memory).
-bool resident_shape(const Level& L, int cluster_max, int& csize, int& Mper, size_t& smem) {
-  if (L.sth || cluster_max < 1 || L.n % 2) return false;
-  const size_t h = static_cast<size_t>(L.n / 2), Nh = h * h * h;
-  const size_t need = (Nh + kResVerts - 1) / kResVerts;
+// Cluster size, vertices per colour and CTA, and colour groups of the resident form on level
+// L, or false when the level does not qualify. 8 groups (every row in registers) wherever
+// at most cluster_max CTAs of 16 vertices hold a colour, else 4 groups of 32.
+bool resident_shape(const Level& L, int cluster_max, int& csize, int& Mper, int& groups, size_t& smem) {
+  if (cluster_max < 1 || L.n % 2 || L.n > 16) return false;
+  const int h = L.n / 2, Nh = h * h * h;
+  groups = Nh <= 16 * cluster_max ? 8 : 4;
+  const int verts = groups == 8 ? 16 : 32;
   int size = 1;
-  while (size < cluster_max && static_cast<size_t>(size) < need) size *= 2;
-  if (static_cast<size_t>(size) < need) return false;
+  while (size < cluster_max && size * verts < Nh) size *= 2;
+  if (size * verts < Nh) return false;
   csize = size;
-  Mper = static_cast<int>((Nh + size - 1) / size);
-  smem = resident_smem_floats(L.N, Mper) * sizeof(float);
+  Mper = (Nh + size - 1) / size;
+  smem = resident_smem_bytes(L.N, Mper, groups);
   return smem <= static_cast<size_t>(kResidentSmemMax);
 }
 
@@ -1147,7 +1203,8 @@ int coarse_cluster_size() {
     }
     int res = -1;
     for (int size : {16, 8, 4, 2, 1}) {
-      if (resident_fits(size) > 0) {
+      if (resident_fits<float, 8>(size) > 0 && resident_fits<float, 4>(size) > 0 &&
+          resident_fits<__nv_bfloat16, 8>(size) > 0 && resident_fits<__nv_bfloat16, 4>(size) > 0) {
         res = size;
         break;
       }
@@ -1171,19 +1228,18 @@ int coarse_resident_size() {
 }
 
 bool coarse_resident_ok(const Level& L, int cluster_max) {
-  int csize, Mper;
+  int csize, Mper, groups;
   size_t smem;
-  return resident_shape(L, cluster_max, csize, Mper, smem);
+  return resident_shape(L, cluster_max, csize, Mper, groups, smem);
 }
 
-cudaError_t launch_coarse_gs_resident(const Level& L, int sweeps, int reverse, int first, const float* f,
-                                      float* x, int cluster_max, cudaStream_t s) {
-  int csize, Mper;
+namespace {
+template <typename T>
+cudaError_t resident_launch(const Level& L, const T* st, int sweeps, int reverse, int first, const float* f, float* x,
+                            int cluster_max, cudaStream_t s) {
+  int csize, Mper, groups;
   size_t smem;
-  if (!resident_shape(L, cluster_max, csize, Mper, smem)) return cudaErrorInvalidValue;
-  const size_t h = static_cast<size_t>(L.n / 2), Nh = h * h * h;
-  const int vec16 = (L.N % 4 == 0) && (Nh % 4 == 0) && (Mper % 4 == 0) &&
-                    (reinterpret_cast<uintptr_t>(L.st) % 16 == 0);
+  if (!resident_shape(L, cluster_max, csize, Mper, groups, smem)) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kCases * csize);
   cfg.blockDim = dim3(kResThreads);
@@ -1196,8 +1252,15 @@ cudaError_t launch_coarse_gs_resident(const Level& L, int sweeps, int reverse, i
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_coarse_gs_resident, L.st, f, x, L.n, sweeps, reverse, first, csize, Mper,
-                            vec16);
+  return cudaLaunchKernelEx(&cfg, groups == 8 ? k_coarse_gs_resident<T, 8> : k_coarse_gs_resident<T, 4>, st, f, x, L.n,
+                            sweeps, reverse, first, csize, Mper);
+}
+}  // namespace
+
+cudaError_t launch_coarse_gs_resident(const Level& L, int sweeps, int reverse, int first, const float* f,
+                                      float* x, int cluster_max, cudaStream_t s) {
+  return L.sth ? resident_launch(L, static_cast<const __nv_bfloat16*>(L.sth), sweeps, reverse, first, f, x, cluster_max, s)
+               : resident_launch(L, static_cast<const float*>(L.st), sweeps, reverse, first, f, x, cluster_max, s);
 }
 
 cudaError_t launch_coarse_gs_sweeps(const Level& L, int sweeps, int reverse, int first, const float* f,

@@ -178,8 +178,8 @@ struct homo_ctx {
   // larger levels one launch per colour with a thread per vertex; gs_cluster: the largest
   // cluster the device launches (-1: none, per-colour launches everywhere)
   int gs_fuse_n = 32, gs_split_n = 32, gs_cluster = -1;
-  // levels with at most gs_res_n cells per axis (FP32 stencils, shared memory permitting)
-  // keep each case's displacement resident in the clusters' shared memory instead;
+  // levels with at most gs_res_n cells per axis (16 at most) keep each case's displacement
+  // in the clusters' shared memory and its stencil rows in their registers instead;
   // gs_resident: the largest cluster of that form the device launches (-1: none)
   int gs_res_n = 16, gs_resident = -1;
 
@@ -269,8 +269,8 @@ cudaError_t launch_coarse_gs_sweeps(const Level& L, int sweeps, int reverse, int
 // One colour pass of level L with a thread per (vertex, case); bitwise launch_coarse_gs.
 cudaError_t launch_coarse_gs_item(const Level& L, int colour, const float* f, float* x, int first,
                                   cudaStream_t s);
-// Every sweep of one smoothing phase of level L with each case's displacement resident in
-// shared memory (FP32 stencils only; coarse_resident_ok says whether L qualifies with
+// Every sweep of one smoothing phase of level L with each case's displacement in shared
+// memory and its stencil rows in registers (coarse_resident_ok says whether L qualifies with
 // clusters of at most cluster_max CTAs); bitwise the iterates of the per-colour launches.
 cudaError_t launch_coarse_gs_resident(const Level& L, int sweeps, int reverse, int first, const float* f,
                                       float* x, int cluster_max, cudaStream_t s);
