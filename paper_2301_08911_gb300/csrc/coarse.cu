@@ -746,58 +746,64 @@ __global__ void k_fill_hash(float* __restrict__ x, size_t count, unsigned seed) 
 }
 
 // coarse[V] = sum over fine 2V + a, a in {-1,0,1}^3, of w(a) fine[2V + a] (R = I^T).
+// Thread per (coarse vertex, load case; the case is blockIdx.y): six times the threads of one
+// thread for all 18 planes, which left the small levels with a handful of warps waiting on
+// 486 loads each, and a working set of 3 planes that stays in L1 on the large ones.
 __global__ void __launch_bounds__(256) k_restrict(const float* __restrict__ fine, int nf,
                                                   float* __restrict__ coarse) {
   const int nc = nf / 2;
   const size_t Nf = static_cast<size_t>(nf) * nf * nf;
-  const size_t Nc = static_cast<size_t>(nc) * nc * nc;
-  for (size_t V = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; V < Nc;
-       V += static_cast<size_t>(gridDim.x) * blockDim.x) {
-    const int X = static_cast<int>(V % nc), Y = static_cast<int>((V / nc) % nc),
-              Z = static_cast<int>(V / (static_cast<size_t>(nc) * nc));
+  const unsigned Nc = static_cast<unsigned>(nc) * nc * nc;
+  fine += 3 * blockIdx.y * Nf;
+  coarse += 3 * blockIdx.y * static_cast<size_t>(Nc);
+  for (unsigned V = blockIdx.x * blockDim.x + threadIdx.x; V < Nc; V += gridDim.x * blockDim.x) {
+    int X, Y, Z;
+    decode3(V, static_cast<unsigned>(nc), X, Y, Z);
     const Nb nb = make_nb(2 * X, 2 * Y, 2 * Z, nf);
-    float acc[kPlanes];
-#pragma unroll
-    for (int q = 0; q < kPlanes; ++q) acc[q] = 0.f;
+    float acc[3] = {0.f, 0.f, 0.f};
 #pragma unroll
     for (int d = 0; d < 27; ++d) {
       const int dx = d % 3 - 1, dy = (d / 3) % 3 - 1, dz = d / 9 - 1;
       const float w = (dx ? 0.5f : 1.f) * (dy ? 0.5f : 1.f) * (dz ? 0.5f : 1.f);
       const size_t o = static_cast<size_t>(nb.X[dx + 1] + nb.Y[dy + 1] + nb.Z[dz + 1]);
 #pragma unroll
-      for (int q = 0; q < kPlanes; ++q) acc[q] = fmaf(w, __ldg(fine + q * Nf + o), acc[q]);
+      for (int q = 0; q < 3; ++q) acc[q] = fmaf(w, __ldg(fine + q * Nf + o), acc[q]);
     }
 #pragma unroll
-    for (int q = 0; q < kPlanes; ++q) coarse[q * Nc + V] = acc[q];
+    for (int q = 0; q < 3; ++q) coarse[q * static_cast<size_t>(Nc) + V] = acc[q];
   }
 }
 
-// fine (+)= I coarse. One thread per coarse cell (X..X+1, Y..Y+1, Z..Z+1): its 8 corner
-// values give the 8 fine vertices (2X+a, 2Y+b, 2Z+c), a,b,c in {0,1}, by trilinear
-// weights (1 on an even fine coordinate, 1/2 to each neighbour on an odd one).
+// fine (+)= I coarse. One thread per coarse cell (X..X+1, Y..Y+1, Z..Z+1) and load case
+// (blockIdx.y): its 8 corner values give the 8 fine vertices (2X+a, 2Y+b, 2Z+c), a,b,c in
+// {0,1}, by trilinear weights (1 on an even fine coordinate, 1/2 to each neighbour on an
+// odd one). PAIRS: the two fine vertices of an x pair move as one 8-byte access (fine is
+// 8-byte aligned and nf even, so every pair is); otherwise one by one.
+template <bool PAIRS>
 __global__ void __launch_bounds__(256) k_prolong(const float* __restrict__ coarse, int nf,
                                                  float* __restrict__ fine, int overwrite) {
   const int nc = nf / 2;
   const size_t Nf = static_cast<size_t>(nf) * nf * nf;
-  const size_t Nc = static_cast<size_t>(nc) * nc * nc;
-  for (size_t V = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; V < Nc;
-       V += static_cast<size_t>(gridDim.x) * blockDim.x) {
-    const int X = static_cast<int>(V % nc), Y = static_cast<int>((V / nc) % nc),
-              Z = static_cast<int>(V / (static_cast<size_t>(nc) * nc));
+  const unsigned Nc = static_cast<unsigned>(nc) * nc * nc;
+  coarse += 3 * blockIdx.y * static_cast<size_t>(Nc);
+  fine += 3 * blockIdx.y * Nf;
+  for (unsigned V = blockIdx.x * blockDim.x + threadIdx.x; V < Nc; V += gridDim.x * blockDim.x) {
+    int X, Y, Z;
+    decode3(V, static_cast<unsigned>(nc), X, Y, Z);
     const int X1 = X + 1 == nc ? 0 : X + 1, Y1 = Y + 1 == nc ? 0 : Y + 1, Z1 = Z + 1 == nc ? 0 : Z + 1;
     size_t cidx[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k)
       cidx[k] = static_cast<size_t>((k & 1) ? X1 : X) +
                 static_cast<size_t>(nc) * (((k >> 1) & 1 ? Y1 : Y) + static_cast<size_t>(nc) * ((k >> 2) ? Z1 : Z));
-    size_t fidx[8];
+    size_t fidx[4];
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-      fidx[k] = static_cast<size_t>(2 * X + (k & 1)) +
-                static_cast<size_t>(nf) * ((2 * Y + ((k >> 1) & 1)) + static_cast<size_t>(nf) * (2 * Z + (k >> 2)));
-#pragma unroll 1
-    for (int q = 0; q < kPlanes; ++q) {
-      const float* cq = coarse + q * Nc;
+    for (int k = 0; k < 4; ++k)
+      fidx[k] = static_cast<size_t>(2 * X) +
+                static_cast<size_t>(nf) * ((2 * Y + (k & 1)) + static_cast<size_t>(nf) * (2 * Z + (k >> 1)));
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const float* cq = coarse + q * static_cast<size_t>(Nc);
       float c[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) c[k] = __ldg(cq + cidx[k]);
@@ -819,9 +825,20 @@ __global__ void __launch_bounds__(256) k_prolong(const float* __restrict__ coars
         }
       float* fq = fine + q * Nf;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const float val = (k >> 2) ? 0.5f * (ay[k & 3] + ay[4 + (k & 3)]) : ay[k];
-        fq[fidx[k]] = overwrite ? val : fq[fidx[k]] + val;
+      for (int k = 0; k < 4; ++k) {
+        const int e = 2 * k;
+        const float v0 = (e >> 2) ? 0.5f * (ay[e & 3] + ay[4 + (e & 3)]) : ay[e];
+        const float v1 = (e >> 2) ? 0.5f * (ay[(e & 3) + 1] + ay[5 + (e & 3)]) : ay[e + 1];
+        float* o = fq + fidx[k];
+        if (PAIRS) {
+          float2 t = overwrite ? make_float2(0.f, 0.f) : *reinterpret_cast<const float2*>(o);
+          t.x = overwrite ? v0 : t.x + v0;
+          t.y = overwrite ? v1 : t.y + v1;
+          *reinterpret_cast<float2*>(o) = t;
+        } else {
+          o[0] = overwrite ? v0 : o[0] + v0;
+          o[1] = overwrite ? v1 : o[1] + v1;
+        }
       }
     }
   }
@@ -1319,14 +1336,16 @@ cudaError_t launch_fill_hash(float* x, size_t count, unsigned seed, cudaStream_t
 
 cudaError_t launch_restrict(int nf, const float* fine, float* coarse, cudaStream_t s) {
   const size_t nc = static_cast<size_t>(nf / 2);
-  k_restrict<<<grid_for(nc * nc * nc, 256), 256, 0, s>>>(fine, nf, coarse);
+  k_restrict<<<dim3(grid_for(nc * nc * nc, 256), kCases), 256, 0, s>>>(fine, nf, coarse);
   return cudaGetLastError();
 }
 
 cudaError_t launch_prolong_add(int nf, const float* coarse, float* fine, int overwrite,
                                cudaStream_t s) {
   const size_t Nf = static_cast<size_t>(nf) * nf * nf;
-  k_prolong<<<grid_for(Nf / 8, 256), 256, 0, s>>>(coarse, nf, fine, overwrite);
+  const dim3 grid(grid_for(Nf / 8, 256), kCases);
+  if (reinterpret_cast<uintptr_t>(fine) % 8 == 0) k_prolong<true><<<grid, 256, 0, s>>>(coarse, nf, fine, overwrite);
+  else k_prolong<false><<<grid, 256, 0, s>>>(coarse, nf, fine, overwrite);
   return cudaGetLastError();
 }
 
