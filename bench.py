@@ -213,11 +213,12 @@ SOLVE_FLOP = 6 * 15 + 30                # 3x3 LDL^T and 6 solves
 def algorithmic_work(kc: str, n: int, sweeps: int = 1):
     N = n ** 3
     if kc == "fine_gs":
-        # colour pass: E 4N, the other colours' u 63N, f_c 9N, u_c 9N (85N); in the first
-        # sweep from zero only lower colours are read (half: 53.5N). 1 of 2*sweeps sweeps.
-        full_b, first_b = 85 * N, 53.5 * N
-        full_f = (576 + 26 * 54 + SOLVE_FLOP) * 2 * N / 8
-        first_f = (288 + 13 * 54 + SOLVE_FLOP) * 2 * N / 8
+        # pass of two colours (the x pairs of the rows of one parity): E 4N, u 72N, f 18N and
+        # 18N written (112N); in the first sweep from zero only the rows of earlier passes are
+        # read (27N on average: 67N). 1 of 2*sweeps sweeps.
+        full_b, first_b = 112 * N, 67 * N
+        full_f = (576 + 26 * 54 + SOLVE_FLOP) * 2 * N / 4
+        first_f = (288 + 13 * 54 + SOLVE_FLOP) * 2 * N / 4
         w = 1.0 / (2 * sweeps)
         return w * first_b + (1 - w) * full_b, w * first_f + (1 - w) * full_f
     if kc == "fine_cheb":
@@ -916,7 +917,7 @@ def run_ours(args, rank, world, local):
 
 def record_traffic(args) -> int:
     """Average DRAM bytes per launch of the fine Gauss-Seidel pass from an ncu CSV (the
-    captured launches should be one V-cycle's 16 passes, first sweep included, which the
+    captured launches should be one V-cycle's 8 passes, first sweep included, which the
     roofline's algorithmic bytes average over too)."""
     import csv
     rows = list(csv.reader(open(args.record_traffic)))

@@ -221,10 +221,14 @@ int ensure_hierarchy(homo_ctx* c) {
 int smooth_level(homo_ctx* c, int l, bool reverse, const float* f, float* x, bool first = false,
                  const double* fmean = nullptr) {
   const int fz = first && !reverse ? 1 : 0;
+  if (l == 0) {
+    for (int k = 0; k < 4; ++k)
+      KL(c, HOMO_KC_FINE_GS, 1, launch_fine_gs(c, reverse ? 3 - k : k, reverse, f, x, fz, fmean));
+    return HOMO_OK;
+  }
   for (int k = 0; k < 8; ++k) {
     const int col = reverse ? 7 - k : k;
-    if (l == 0) KL(c, HOMO_KC_FINE_GS, 1, launch_fine_gs(c, col, f, x, fz, fmean));
-    else if (c->lev[l].n <= c->gs_split_n)
+    if (c->lev[l].n <= c->gs_split_n)
       KL(c, HOMO_KC_COARSE_GS, 1, launch_coarse_gs_item(c->lev[l], col, f, x, fz, c->stream));
     else KL(c, HOMO_KC_COARSE_GS, 1, launch_coarse_gs(c->lev[l], col, f, x, fz, c->stream));
   }
@@ -1279,7 +1283,7 @@ int homo_autotune(homo_ctx* ctx, int flags, int* gs_cases, int* gs_block, double
         if (kVar[k][0] == it->second.first && kVar[k][1] == it->second.second) best = k;
   }
   if (best < 0) {
-    // time one symmetric sweep pair (16 colour passes) of each variant on the context's
+    // time one symmetric sweep pair (8 launches of two colours) of each variant on the context's
     // own moduli and loads, into the CG scratch vector z (free between solves)
     RET(ensure_loads(ctx));
     cudaEvent_t a = nullptr, b = nullptr;

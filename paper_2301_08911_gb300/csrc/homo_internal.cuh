@@ -243,9 +243,10 @@ int tiled_grid_blocks(int n);
 cudaError_t launch_fine_residual(const homo_ctx* c, const float* b, const float* u,
                                  const float* ulo, float* out, double* part, int* grid_out,
                                  const double* bmean);
-// first != 0: first sweep from u = 0, colours 0..7 (u need not be cleared); fmean: plane
+// Colours 2 pair and 2 pair + 1 (reverse: the odd one first) of one sweep on the finest level.
+// first != 0: first sweep from u = 0 (colours 0..7; u need not be cleared); fmean: plane
 // means subtracted from f, or null
-cudaError_t launch_fine_gs(const homo_ctx* c, int colour, const float* f, float* u, int first,
+cudaError_t launch_fine_gs(const homo_ctx* c, int pair, int reverse, const float* f, float* u, int first,
                            const double* fmean);
 // (cases, block) is a compiled variant of the fine Gauss-Seidel kernel
 bool gs_variant_ok(int cases, int block);
