@@ -222,6 +222,10 @@ int smooth_level(homo_ctx* c, int l, bool reverse, const float* f, float* x, boo
                  const double* fmean = nullptr) {
   const int fz = first && !reverse ? 1 : 0;
   if (l == 0) {
+    if (c->n <= c->gs_res_n && c->gs_resident > 0 && coarse_resident_ok(c->lev[0], c->gs_resident)) {
+      KL(c, HOMO_KC_FINE_GS, 1, launch_fine_gs_resident(c, reverse, f, x, fz, fmean));
+      return HOMO_OK;
+    }
     for (int k = 0; k < 4; ++k)
       KL(c, HOMO_KC_FINE_GS, 1, launch_fine_gs(c, reverse ? 3 - k : k, reverse, f, x, fz, fmean));
     return HOMO_OK;
@@ -414,8 +418,7 @@ int enq_true_residual(homo_ctx* c, double tol, bool exact) {
   else
     KL(c, HOMO_KC_TRUE_RESIDUAL, 1,
        launch_fine_tiled(c, 2, c->u, c->f, c->r, c->part, &g, nullptr, 0.f, 0.f, c->ulo));
-  KL(c, HOMO_KC_CG_VECTOR, 1, launch_sum_partials(c->part, g, kCases + kPlanes, c->scal + S_RR, c->stream));
-  KL(c, HOMO_KC_CG_VECTOR, 1, launch_cg_active(c->scal, tol, c->N, c->stream));
+  KL(c, HOMO_KC_CG_VECTOR, 1, launch_sum_step(kSumActive, c->part, g, c->scal, 0, tol, c->N, c->stream));
   return enq_read(c, S_RR, 6);
 }
 
@@ -443,8 +446,7 @@ int precondition_and_direction(homo_ctx* c, int first) {
   int g = 0;
   RET(vcycle(c, c->r, c->z, c->scal + S_RMEAN));
   KL(c, HOMO_KC_CG_VECTOR, 1, launch_dot6_zsum(c->r, c->z, c->N, c->scal + S_RMEAN, c->part, &g, c->stream));
-  KL(c, HOMO_KC_CG_VECTOR, 1, launch_sum_partials(c->part, g, kCases + kPlanes, c->scal + S_RZ, c->stream));
-  KL(c, HOMO_KC_CG_VECTOR, 1, launch_cg_beta(c->scal, first, c->stream));
+  KL(c, HOMO_KC_CG_VECTOR, 1, launch_sum_step(kSumBeta, c->part, g, c->scal, first, 0.0, c->N, c->stream));
   KL(c, HOMO_KC_CG_VECTOR, 1, launch_cg_update_p(c->pv, c->z, c->scal, c->N, c->stream));
   return HOMO_OK;
 }
@@ -504,12 +506,10 @@ int enq_iteration(homo_ctx* c, int first, double inner_tol) {
   int g = 0;
   RET(precondition_and_direction(c, first));
   KL(c, HOMO_KC_FINE_MATVEC, 1, launch_fine_apply(c, c->pv, c->q, c->part, &g));
-  KL(c, HOMO_KC_CG_VECTOR, 1, launch_sum_partials(c->part, g, kCases + kPlanes, c->scal + S_PQ, c->stream));
-  KL(c, HOMO_KC_CG_VECTOR, 1, launch_cg_alpha(c->scal, c->stream));
+  KL(c, HOMO_KC_CG_VECTOR, 1, launch_sum_step(kSumAlpha, c->part, g, c->scal, 0, 0.0, c->N, c->stream));
   KL(c, HOMO_KC_CG_VECTOR, 1,
      launch_cg_update_er(c->ecyc, c->ecyclo, c->r, c->pv, c->q, c->scal, c->N, c->part, &g, c->stream));
-  KL(c, HOMO_KC_CG_VECTOR, 1, launch_sum_partials(c->part, g, kCases + kPlanes, c->scal + S_RR, c->stream));
-  KL(c, HOMO_KC_CG_VECTOR, 1, launch_cg_active(c->scal, inner_tol, c->N, c->stream));
+  KL(c, HOMO_KC_CG_VECTOR, 1, launch_sum_step(kSumActive, c->part, g, c->scal, 0, inner_tol, c->N, c->stream));
   return enq_read(c, S_RR, 6);
 }
 

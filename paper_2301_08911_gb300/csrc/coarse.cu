@@ -1,9 +1,10 @@
 // Coarse levels of the multigrid hierarchy (Sec. 3.3, Sec. 4.2): Galerkin stencils,
 // stored-stencil relaxation and residual, trilinear transfers and the direct coarsest
 // solve with the rigid-translation null space projected out.
-#include "dev_common.cuh"
+#include "stencil.cuh"
 
 #include <algorithm>
+#include <iterator>
 #include <mutex>
 
 namespace homo {
@@ -486,11 +487,56 @@ __device__ __forceinline__ float res_chain(float b, const float4* us, const ResN
   return b;
 }
 
-template <typename T, int kGroups>
-__global__ void __launch_bounds__(kResThreads, 1) k_coarse_gs_resident(const T* __restrict__ st,
-                                                                     const float* __restrict__ f, float* x,
-                                                                     int n, int sweeps, int reverse, int first,
-                                                                     int csize, int Mper) {
+// Where a resident smoother's rows come from: load(colour, position m, r, row, S) gives block row
+// r of the 26 neighbour blocks (78 values, diagonal skipped) and, if S, the diagonal block.
+template <typename T>
+struct StoredRows {   // a coarse level's stencil
+  const T* st;
+  __device__ __forceinline__ float mean(int) const { return 0.f; }
+  template <typename Put>
+  __device__ __forceinline__ void load(int colour, unsigned m, int n, int r, Put put, float (&S)[9]) const {
+    const size_t N = static_cast<size_t>(n) * n * n;
+    const int h = n >> 1;
+    const size_t p = static_cast<size_t>(colour) * h * h * h + m;
+#pragma unroll
+    for (int e = 0; e < 26; ++e)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) put(3 * e + k, ld_st(st + static_cast<size_t>(9 * (e < 13 ? e : e + 1) + 3 * r + k) * N + p));
+#pragma unroll
+    for (int k = 0; k < 9; ++k) S[k] = ld_st(st + static_cast<size_t>(9 * 13 + k) * N + p);
+  }
+};
+
+struct FineRows {   // the finest level: built from the moduli, as its other kernels do
+  const KeParam& K;
+  const float* E;
+  const double* fmean;
+  __device__ __forceinline__ float mean(int q) const { return fmean ? static_cast<float>(fmean[q]) : 0.f; }
+  template <typename Put>
+  __device__ __forceinline__ void load(int colour, unsigned m, int n, int r, Put put, float (&S)[9]) const {
+    int i, j, k;
+    decode3(m, static_cast<unsigned>(n >> 1), i, j, k);
+    const Nb nb = make_nb(2 * i + (colour & 1), 2 * j + ((colour >> 1) & 1), 2 * k + (colour >> 2), n);
+    float Et[8];
+    load_E8(E, nb, Et);
+#pragma unroll
+    for (int d = 0; d < 27; ++d) {
+      float A[9];
+      nb_block(K, Et, d % 3 - 1, (d / 3) % 3 - 1, d / 9 - 1, A);
+      if (d == 13) {
+#pragma unroll
+        for (int q = 0; q < 9; ++q) S[q] = A[q];
+        continue;
+      }
+#pragma unroll
+      for (int q = 0; q < 3; ++q) put(3 * (d < 13 ? d : d - 1) + q, r == 0 ? A[q] : (r == 1 ? A[3 + q] : A[6 + q]));
+    }
+  }
+};
+
+template <int kGroups, typename Rows>
+__device__ __forceinline__ void gs_resident(const Rows& src, const float* __restrict__ f, float* x, int n,
+                                            int sweeps, int reverse, int first, int csize, int Mper) {
   extern __shared__ __align__(16) float sm[];
   __shared__ unsigned need_s;
   constexpr int kWarps = kResThreads / 32 / kGroups;       // warps (8 vertices each) per group
@@ -532,23 +578,16 @@ __global__ void __launch_bounds__(kResThreads, 1) k_coarse_gs_resident(const T* 
 #pragma unroll
     for (int q = 0; q < 8 / kGroups; ++q) {
       const int colour = group + 4 * q;
-      const size_t p = static_cast<size_t>(colour) * Nh + m0 + j;
       const size_t v = static_cast<size_t>(2 * a + (colour & 1)) +
                        static_cast<size_t>(n) * ((2 * b + ((colour >> 1) & 1)) + static_cast<size_t>(n) * (2 * d + (colour >> 2)));
-      rhs[q] = __ldg(fc + static_cast<size_t>(r) * N + v);
+      rhs[q] = __ldg(fc + static_cast<size_t>(r) * N + v) - src.mean(3 * c + r);
       float* dst = rows + ((static_cast<size_t>(group) * Mper + j) * 3 + r) * kResRow;
-#pragma unroll
-      for (int e = 0; e < 26; ++e)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          const float val = ld_st(st + static_cast<size_t>(9 * (e < 13 ? e : e + 1) + 3 * r + k) * N + p);
-          if (q == 0) A[3 * e + k] = val;
-          else dst[3 * e + k] = val;
-        }
+      float S[9];
+      src.load(colour, static_cast<unsigned>(m0 + j), n, r, [&](int e, float val) {
+        if (q == 0) A[e] = val;
+        else dst[e] = val;
+      }, S);
       if (r == 0) {
-        float S[9];
-#pragma unroll
-        for (int k = 0; k < 9; ++k) S[k] = ld_st(st + static_cast<size_t>(9 * 13 + k) * N + p);
         const Factor3 F = factor3(S);
         fac[2 * (colour * Mper + j)] = make_float4(F.l10, F.l20, F.l21, F.i0);
         fac[2 * (colour * Mper + j) + 1] = make_float4(F.i1, F.i2, 0.f, 0.f);
@@ -633,6 +672,26 @@ __global__ void __launch_bounds__(kResThreads, 1) k_coarse_gs_resident(const T* 
     __stcg(xc + N + v, u.y);
     __stcg(xc + 2 * static_cast<size_t>(N) + v, u.z);
   }
+}
+
+template <typename T, int kGroups>
+__global__ void __launch_bounds__(kResThreads, 1) k_coarse_gs_resident(const T* __restrict__ st,
+                                                                     const float* __restrict__ f, float* x,
+                                                                     int n, int sweeps, int reverse, int first,
+                                                                     int csize, int Mper) {
+  gs_resident<kGroups>(StoredRows<T>{st}, f, x, n, sweeps, reverse, first, csize, Mper);
+}
+
+// One sweep of the finest level of a cell of at most 16^3 in one launch: as many launches of
+// colour pairs are all launch and load latency there (16^3: 11 us each, four a sweep).
+template <int kGroups>
+__global__ void __launch_bounds__(kResThreads, 1) k_fine_gs_resident(const __grid_constant__ KeParam K,
+                                                                    const float* __restrict__ E,
+                                                                    const float* __restrict__ f, float* x, int n,
+                                                                    int reverse, int first,
+                                                                    const double* __restrict__ fmean, int csize,
+                                                                    int Mper) {
+  gs_resident<kGroups>(FineRows{K, E, fmean}, f, x, n, 1, reverse, first, csize, Mper);
 }
 
 // out = b - K x with the stored stencil; threads walk stencil positions (coalesced).
@@ -1162,9 +1221,7 @@ int g_cluster_size[256] = {};    // per device: 0 = not queried, -1 = no cluster
 int g_resident_size[256] = {};   // per device: largest resident-form cluster, -1 = none
 constexpr int kResidentSmemMax = 216 * 1024;   // dynamic shared memory of the resident form, at most
 
-template <typename T, int kGroups>
-int resident_fits(int size) {
-  const void* fn = reinterpret_cast<const void*>(k_coarse_gs_resident<T, kGroups>);
+int resident_fits(int size, const void* fn) {
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, size > 8 ? 1 : 0) != cudaSuccess ||
       cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kResidentSmemMax) != cudaSuccess)
     return 0;
@@ -1220,8 +1277,13 @@ int coarse_cluster_size() {
     }
     int res = -1;
     for (int size : {16, 8, 4, 2, 1}) {
-      if (resident_fits<float, 8>(size) > 0 && resident_fits<float, 4>(size) > 0 &&
-          resident_fits<__nv_bfloat16, 8>(size) > 0 && resident_fits<__nv_bfloat16, 4>(size) > 0) {
+      const void* forms[] = {reinterpret_cast<const void*>(k_coarse_gs_resident<float, 8>),
+                             reinterpret_cast<const void*>(k_coarse_gs_resident<float, 4>),
+                             reinterpret_cast<const void*>(k_coarse_gs_resident<__nv_bfloat16, 8>),
+                             reinterpret_cast<const void*>(k_coarse_gs_resident<__nv_bfloat16, 4>),
+                             reinterpret_cast<const void*>(k_fine_gs_resident<8>),
+                             reinterpret_cast<const void*>(k_fine_gs_resident<4>)};
+      if (std::all_of(std::begin(forms), std::end(forms), [size](const void* fn) { return resident_fits(size, fn) > 0; })) {
         res = size;
         break;
       }
@@ -1251,28 +1313,46 @@ bool coarse_resident_ok(const Level& L, int cluster_max) {
 }
 
 namespace {
+// Launch configuration of a resident smoother on level L.
+struct ResidentLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  int csize = 0, Mper = 0, groups = 0;
+  bool set(const Level& L, int cluster_max, cudaStream_t s) {
+    size_t smem;
+    if (!resident_shape(L, cluster_max, csize, Mper, groups, smem)) return false;
+    cfg.gridDim = dim3(kCases * csize);
+    cfg.blockDim = dim3(kResThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = csize;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return true;
+  }
+};
+
 template <typename T>
 cudaError_t resident_launch(const Level& L, const T* st, int sweeps, int reverse, int first, const float* f, float* x,
                             int cluster_max, cudaStream_t s) {
-  int csize, Mper, groups;
-  size_t smem;
-  if (!resident_shape(L, cluster_max, csize, Mper, groups, smem)) return cudaErrorInvalidValue;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(kCases * csize);
-  cfg.blockDim = dim3(kResThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = csize;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, groups == 8 ? k_coarse_gs_resident<T, 8> : k_coarse_gs_resident<T, 4>, st, f, x, L.n,
-                            sweeps, reverse, first, csize, Mper);
+  ResidentLaunch r;
+  if (!r.set(L, cluster_max, s)) return cudaErrorInvalidValue;
+  return cudaLaunchKernelEx(&r.cfg, r.groups == 8 ? k_coarse_gs_resident<T, 8> : k_coarse_gs_resident<T, 4>, st, f, x,
+                            L.n, sweeps, reverse, first, r.csize, r.Mper);
 }
 }  // namespace
+
+cudaError_t launch_fine_gs_resident(const homo_ctx* c, int reverse, const float* f, float* u, int first,
+                                    const double* fmean) {
+  ResidentLaunch r;
+  if (!r.set(c->lev[0], c->gs_resident, c->stream)) return cudaErrorInvalidValue;
+  const float* E = c->E;
+  return cudaLaunchKernelEx(&r.cfg, r.groups == 8 ? k_fine_gs_resident<8> : k_fine_gs_resident<4>, c->ke, E, f, u,
+                            c->n, reverse, first, fmean, r.csize, r.Mper);
+}
 
 cudaError_t launch_coarse_gs_resident(const Level& L, int sweeps, int reverse, int first, const float* f,
                                       float* x, int cluster_max, cudaStream_t s) {

@@ -248,6 +248,10 @@ cudaError_t launch_fine_residual(const homo_ctx* c, const float* b, const float*
 // means subtracted from f, or null
 cudaError_t launch_fine_gs(const homo_ctx* c, int pair, int reverse, const float* f, float* u, int first,
                            const double* fmean);
+// The whole sweep in one launch (coarse.cu, the resident form with rows built from E and K0);
+// the finest level must satisfy coarse_resident_ok. Bitwise the sweep of launch_fine_gs.
+cudaError_t launch_fine_gs_resident(const homo_ctx* c, int reverse, const float* f, float* u, int first,
+                                    const double* fmean);
 // (cases, block) is a compiled variant of the fine Gauss-Seidel kernel
 bool gs_variant_ok(int cases, int block);
 cudaError_t launch_fine_elem(const homo_ctx* c, int mode, const double* g36, float* sens,
@@ -314,15 +318,17 @@ cudaError_t nn_pool(int n, int f, const float* rho, float* out, cudaStream_t s);
 int reduce_grid(size_t n_items);
 cudaError_t launch_sum_partials(const double* part, int nblk, int nv, double* out,
                                 cudaStream_t s);
+// The 24 sums (6 dots, 18 plane sums) of one CG reduction into their slots and the scalar step
+// they are for: alpha (sums at S_PQ), beta (S_RZ; first: of a cycle) or the centred norms, plane
+// means and active flags of r (S_RR; tol, N)
+enum SumStep { kSumOnly, kSumAlpha, kSumBeta, kSumActive };
+cudaError_t launch_sum_step(int step, const double* part, int nblk, double* scal, int first, double tol, size_t N,
+                            cudaStream_t s);
 cudaError_t launch_dot6(const float* a, const float* b, size_t N, double* part, int* grid_out,
                         cudaStream_t s);
 // (r - rmean, z) per case and plane sums of z; rmean: 18 doubles or null
 cudaError_t launch_dot6_zsum(const float* r, const float* z, size_t N, const double* rmean,
                              double* part, int* grid_out, cudaStream_t s);
-cudaError_t launch_cg_alpha(double* scal, cudaStream_t s);
-cudaError_t launch_cg_beta(double* scal, int first, cudaStream_t s);
-// centred norms and plane means of r from its raw sums, active flags
-cudaError_t launch_cg_active(double* scal, double tol, size_t N, cudaStream_t s);
 // e += alpha p, r -= alpha (q - mean q), partials of ||r||^2 and plane sums of r
 cudaError_t launch_cg_update_er(float* e, float* elo, float* r, const float* p, const float* q,
                                 const double* scal, size_t N, double* part, int* grid_out,

@@ -58,8 +58,48 @@ __device__ __forceinline__ void df_add(float& hi, float& lo, float d, float dlo)
   hi = s2;
 }
 
+// CG scalar steps (thread c < 6 of a block that has just written the sums they read).
+__device__ __forceinline__ void cg_alpha(double* s, int c) {
+  const double pq = s[S_PQ + c];
+  double a = 0.0;
+  if (s[S_ACTIVE + c] != 0.0 && pq > 0.0 && isfinite(pq)) a = s[S_RZ + c] / pq;
+  s[S_ALPHA + c] = a;
+}
+
+// beta = rz_new / rz_old (0 on the first step or for finished cases); rz_old <- rz_new.
+__device__ __forceinline__ void cg_beta(double* s, int c, int first) {
+  const double rz = s[S_RZ + c], old = s[S_RZ_OLD + c];
+  double b = 0.0;
+  if (!first && s[S_ACTIVE + c] != 0.0 && old != 0.0 && isfinite(rz)) b = rz / old;
+  s[S_BETA + c] = b;
+  s[S_RZ_OLD + c] = rz;
+}
+
+// The stored residual keeps the plane means it had when it was last recomputed (the
+// rigid translations, outside the range of K); every consumer subtracts them. This
+// step turns the raw sums into the centred norms ||r_c - mean||^2 = sum r^2 - sum^2/N
+// and the plane means, and marks case c active while ||r_c||^2 > tol^2 ||f_c||^2.
+__device__ __forceinline__ void cg_active(double* s, int c, double tol2, double N) {
+  double rr = s[S_RR + c];
+  for (int k = 0; k < 3; ++k) {
+    const double sum = s[S_RSUM + 3 * c + k];
+    rr -= sum * sum / N;
+    s[S_RMEAN + 3 * c + k] = sum / N;
+  }
+  rr = fmax(rr, 0.0);
+  s[S_RR + c] = rr;
+  const double ff = s[S_FF + c];
+  s[S_ACTIVE + c] = (ff > 0.0 && rr > tol2 * ff) ? 1.0 : 0.0;
+}
+
+// out[k] = sum over the nblk rows of part, then the CG step the sums are for (STEP: SumStep;
+// scal: the slots, out one of them). One block: the step needs no launch of its own, which
+// cost a small cell's iteration three of its launches. 16 loads of a thread in flight: with 4 the
+// one block took 33 us over 2432 x 24 partials.
+template <int STEP>
 __global__ void __launch_bounds__(256) k_sum_partials(const double* __restrict__ part, int nblk,
-                                                      int nv, double* __restrict__ out) {
+                                                      int nv, double* out, double* scal, int first,
+                                                      double tol2, double N) {
   // thread t owns value k = t % nv of rows r0, r0 + per, r0 + 2 per, ... (r0 = t / nv):
   // the block reads the row-major partials contiguously, with four independent sums
   __shared__ double sh[256];
@@ -71,13 +111,14 @@ __global__ void __launch_bounds__(256) k_sum_partials(const double* __restrict__
     const size_t stride = static_cast<size_t>(per) * nv;
     const size_t total = static_cast<size_t>(nblk) * nv;
     size_t i = static_cast<size_t>(r0) * nv + k;
+#pragma unroll 4
     for (; i + 3 * stride < total; i += 4 * stride) {
-      s0 += part[i];
-      s1 += part[i + stride];
-      s2 += part[i + 2 * stride];
-      s3 += part[i + 3 * stride];
+      s0 += __ldg(part + i);
+      s1 += __ldg(part + i + stride);
+      s2 += __ldg(part + i + 2 * stride);
+      s3 += __ldg(part + i + 3 * stride);
     }
-    for (; i < total; i += stride) s0 += part[i];
+    for (; i < total; i += stride) s0 += __ldg(part + i);
   }
   sh[t] = (s0 + s1) + (s2 + s3);
   __syncthreads();
@@ -86,6 +127,12 @@ __global__ void __launch_bounds__(256) k_sum_partials(const double* __restrict__
     for (int r = 0; r < per; ++r) acc += sh[r * nv + t];
     out[t] = acc;
   }
+  if (STEP == kSumOnly) return;
+  __syncthreads();
+  if (t >= kCases) return;
+  if (STEP == kSumAlpha) cg_alpha(scal, t);
+  if (STEP == kSumBeta) cg_beta(scal, t, first);
+  if (STEP == kSumActive) cg_active(scal, t, tol2, N);
 }
 
 // Per case c: sum over the 3 planes of case c of a*b. Each thread takes W consecutive
@@ -136,45 +183,6 @@ __global__ void __launch_bounds__(256) k_dot6_zsum(const float* __restrict__ r,
     }
   }
   block_sum_store<kCases + kPlanes>(red, part);
-}
-
-__global__ void k_cg_alpha(double* __restrict__ s) {
-  const int c = threadIdx.x;
-  if (c >= kCases) return;
-  const double pq = s[S_PQ + c];
-  double a = 0.0;
-  if (s[S_ACTIVE + c] != 0.0 && pq > 0.0 && isfinite(pq)) a = s[S_RZ + c] / pq;
-  s[S_ALPHA + c] = a;
-}
-
-// beta = rz_new / rz_old (0 on the first step or for finished cases); rz_old <- rz_new.
-__global__ void k_cg_beta(double* __restrict__ s, int first) {
-  const int c = threadIdx.x;
-  if (c >= kCases) return;
-  const double rz = s[S_RZ + c], old = s[S_RZ_OLD + c];
-  double b = 0.0;
-  if (!first && s[S_ACTIVE + c] != 0.0 && old != 0.0 && isfinite(rz)) b = rz / old;
-  s[S_BETA + c] = b;
-  s[S_RZ_OLD + c] = rz;
-}
-
-// The stored residual keeps the plane means it had when it was last recomputed (the
-// rigid translations, outside the range of K); every consumer subtracts them. This
-// kernel turns the raw sums into the centred norms ||r_c - mean||^2 = sum r^2 - sum^2/N
-// and the plane means, and marks case c active while ||r_c||^2 > tol^2 ||f_c||^2.
-__global__ void k_cg_active(double* __restrict__ s, double tol2, double N) {
-  const int c = threadIdx.x;
-  if (c >= kCases) return;
-  double rr = s[S_RR + c];
-  for (int k = 0; k < 3; ++k) {
-    const double sum = s[S_RSUM + 3 * c + k];
-    rr -= sum * sum / N;
-    s[S_RMEAN + 3 * c + k] = sum / N;
-  }
-  rr = fmax(rr, 0.0);
-  s[S_RR + c] = rr;
-  const double ff = s[S_FF + c];
-  s[S_ACTIVE + c] = (ff > 0.0 && rr > tol2 * ff) ? 1.0 : 0.0;
 }
 
 // e += alpha p, e kept in double-float (e + elo): the product is split exactly (its
@@ -595,7 +603,21 @@ int reduce_grid(size_t n_items) { return grid_for(n_items, 256); }
 cudaError_t launch_sum_partials(const double* part, int nblk, int nv, double* out,
                                 cudaStream_t s) {
   if (nv < 1 || nv > 256) return cudaErrorInvalidValue;
-  k_sum_partials<<<1, 256, 0, s>>>(part, nblk, nv, out);
+  k_sum_partials<kSumOnly><<<1, 256, 0, s>>>(part, nblk, nv, out, nullptr, 0, 0.0, 0.0);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_sum_step(int step, const double* part, int nblk, double* scal, int first, double tol, size_t N,
+                            cudaStream_t s) {
+  const int nv = kCases + kPlanes;
+  if (step == kSumAlpha)
+    k_sum_partials<kSumAlpha><<<1, 256, 0, s>>>(part, nblk, nv, scal + S_PQ, scal, 0, 0.0, 0.0);
+  else if (step == kSumBeta)
+    k_sum_partials<kSumBeta><<<1, 256, 0, s>>>(part, nblk, nv, scal + S_RZ, scal, first, 0.0, 0.0);
+  else if (step == kSumActive)
+    k_sum_partials<kSumActive><<<1, 256, 0, s>>>(part, nblk, nv, scal + S_RR, scal, 0, tol * tol, static_cast<double>(N));
+  else
+    return cudaErrorInvalidValue;
   return cudaGetLastError();
 }
 
@@ -614,21 +636,6 @@ cudaError_t launch_dot6_zsum(const float* r, const float* z, size_t N, const dou
   *grid_out = g;
   if (N % 4 == 0) k_dot6_zsum<4><<<g, 256, 0, s>>>(r, z, N, rmean, part);
   else k_dot6_zsum<1><<<g, 256, 0, s>>>(r, z, N, rmean, part);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_cg_alpha(double* scal, cudaStream_t s) {
-  k_cg_alpha<<<1, 32, 0, s>>>(scal);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_cg_beta(double* scal, int first, cudaStream_t s) {
-  k_cg_beta<<<1, 32, 0, s>>>(scal, first);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_cg_active(double* scal, double tol, size_t N, cudaStream_t s) {
-  k_cg_active<<<1, 32, 0, s>>>(scal, tol * tol, static_cast<double>(N));
   return cudaGetLastError();
 }
 
@@ -735,7 +742,7 @@ cudaError_t launch_oc(homo_ctx* c, const float* dc, float* rho, double volfrac, 
   for (int it = 0; it < kOcPasses; ++it) {
     k_oc_pass<<<g, 256, 0, s>>>(rho, c->tmp, N, static_cast<float>(move), static_cast<float>(rho_min), oc,
                                 c->part);
-    k_sum_partials<<<1, 256, 0, s>>>(c->part, g, kOcCand, oc + OC_SUMS);
+    k_sum_partials<kSumOnly><<<1, 256, 0, s>>>(c->part, g, kOcCand, oc + OC_SUMS, nullptr, 0, 0.0, 0.0);
     k_oc_pass_final<<<1, 32, 0, s>>>(oc + OC_SUMS, N, volfrac, oc);
   }
   k_oc_apply<<<g, 256, 0, s>>>(rho, c->tmp, N, static_cast<float>(move), static_cast<float>(rho_min), oc,
