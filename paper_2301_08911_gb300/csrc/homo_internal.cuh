@@ -28,7 +28,7 @@ constexpr int kStencil = 243;
 constexpr int kMaxLevels = 16;
 constexpr int kRedBlock = 256;          // threads per block of every reduction kernel
 constexpr int kOcPasses = 8;            // OC multiplier search passes (15 candidates each)
-constexpr int kOcKernels = 4 + 3 * kOcPasses;   // kernels one OC update launches
+constexpr int kOcKernels = 2 + kOcPasses;   // kernels one OC update launches
 
 // Element matrix of a unit-modulus voxel (side 1), row-major 24x24, dof 3j + comp.
 struct KeParam {

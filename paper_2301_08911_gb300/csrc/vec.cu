@@ -1,6 +1,7 @@
 // Vector kernels of the CG driver, reductions, the periodic density filter and the OC
 // update. All reductions are two-stage and deterministic: per-block partials in FP64,
 // then one block sums them in a fixed order.
+#include <algorithm>
 #include <cmath>
 
 #include "dev_common.cuh"
@@ -336,173 +337,313 @@ __global__ void __launch_bounds__(256) k_filter(const __grid_constant__ FilterPa
   }
 }
 
+// The same for a radius in (sqrt 3, 2]: exactly the 27 offsets of the unit cube, in k_filter's
+// order with its weights (w[k]: k nonzero components), so the result is bitwise k_filter's.
+// The general loop spends about 20 integer instructions per offset on wrapping and on
+// indexing its offset table; with the neighbour indices taken once per element the pass
+// is bound by its 27 loads through L1 (192^3: 265 -> 58 us).
+struct Filter27 {
+  float w[4];
+  float inv_wsum;
+};
+
+template <bool kSens>
+__global__ void __launch_bounds__(256) k_filter27(Filter27 F, int n, const float* __restrict__ in,
+                                                  const float* __restrict__ rho, float gamma,
+                                                  float* __restrict__ out) {
+  const unsigned N = static_cast<unsigned>(n) * n * n;
+  for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < N; e += gridDim.x * blockDim.x) {
+    int x, y, z;
+    decode3(e, static_cast<unsigned>(n), x, y, z);
+    const Nb nb = make_nb(x, y, z, n);
+    float s = 0.f;
+#pragma unroll
+    for (int k = 0; k < 27; ++k) {
+      const int a = k % 3, b = (k / 3) % 3, c = k / 9;
+      const unsigned f = static_cast<unsigned>(nb.X[a] + nb.Y[b] + nb.Z[c]);
+      const float v = kSens ? __ldg(in + f) * __ldg(rho + f) : __ldg(in + f);
+      s = fmaf(F.w[(a != 1) + (b != 1) + (c != 1)], v, s);
+    }
+    out[e] = kSens ? s * F.inv_wsum / fmaxf(gamma, __ldg(rho + e)) : s * F.inv_wsum;
+  }
+}
+
 // ---------------------------------------------------------------- OC update
 // rho_new(s) = clamp(base_e * s, lo_e, hi_e), base_e = rho_e max(-dc_e, 0)^eta,
 // s = lambda^(-eta); mean(rho_new) increases with s. OC scratch (doubles at S_OC):
 constexpr int kOcCand = 15;      // candidate multipliers per pass
 // kOcPasses passes (homo_internal.cuh): the bracket shrinks 16x per pass in log scale
-enum { OC_SLO = 0, OC_SHI = 1, OC_MODE = 2, OC_CAND = 8, OC_CHANGE = 32, OC_SUMS = 40 };
+enum { OC_SLO = 0, OC_SHI = 1, OC_MODE = 2, OC_CAND = 8, OC_CHANGE = 32, OC_TICKET = 56 };
+
+// One launch per pass: the block that finishes last (a ticket counter, taken after its partials
+// are fenced; no block waits) sums the partials in a fixed order and takes the pass's host-free
+// decision. Sums: an FP32 pair per thread and through the warp (TwoSum), FP64 across warps:
+// an FP64 warp reduction of 15 values by every thread cost 80 of the 90 us of a 192^3
+// pass (2 FP64 operations per clock and SM). What is summed are the FP32 sums of the up to 8
+// terms e, e + stride, ... e + 7 stride of a run (stride: the grid of one thread per element, at most 16 blocks per SM), which decide the last
+// bits of the multiplier and with it the density: they keep their grouping whatever the grid.
+// 192^3 update: 2600 -> 440 us in 10 launches instead of 28.
+constexpr int kOcBlock = 256;
+constexpr int kOcGrid = 152 * 4;
 
 __device__ __forceinline__ float oc_lo(float r, float move, float rmin) { return fmaxf(rmin, r - move); }
 __device__ __forceinline__ float oc_hi(float r, float move) { return fminf(1.f, r + move); }
 
-// base -> tmp; block partials [min lo/base, max hi/base, sum lo, sum hi] over base > 0.
-__global__ void __launch_bounds__(256) k_oc_setup(const float* __restrict__ rho,
-                                                  const float* __restrict__ dc,
-                                                  float* __restrict__ base, size_t N, float eta,
-                                                  float move, float rmin,
-                                                  double* __restrict__ part) {
-  float mn = INFINITY, mx = 0.f;
-  double slo = 0.0, shi = 0.0;
-  for (size_t e = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < N;
-       e += static_cast<size_t>(gridDim.x) * blockDim.x) {
-    const float r = rho[e];
-    const float D = fmaxf(-dc[e], 0.f);
-    const float bs = D > 0.f ? r * powf(D, eta) : 0.f;
-    base[e] = bs;
-    const float lo = oc_lo(r, move, rmin), hi = oc_hi(r, move);
-    slo += lo;
-    shi += hi;
-    if (bs > 0.f) {
-      mn = fminf(mn, lo / bs);
-      mx = fmaxf(mx, hi / bs);
+// hi + lo += v with TwoSum, lo collecting the rounding errors
+__device__ __forceinline__ void pair_add(float& hi, float& lo, float v) {
+  const float s = __fadd_rn(hi, v);
+  const float bb = __fadd_rn(s, -hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -bb)), __fadd_rn(v, -bb)));
+  hi = s;
+}
+
+// Block sums of NV FP32 pairs into part[blockIdx.x * NV + k] (FP64 across the warps).
+template <int NV>
+__device__ __forceinline__ void pair_block_sum(float (&hi)[NV], float (&lo)[NV], double* part) {
+  __shared__ double sh[kOcBlock / 32][NV];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float h = __shfl_down_sync(0xffffffffu, hi[k], o), l = __shfl_down_sync(0xffffffffu, lo[k], o);
+      pair_add(hi[k], lo[k], h);
+      lo[k] = __fadd_rn(lo[k], l);
     }
+    if (lane == 0) sh[wid][k] = static_cast<double>(hi[k]) + static_cast<double>(lo[k]);
   }
-  __shared__ float smn[256], smx[256];
-  __shared__ double ssl[256], ssh[256];
-  smn[threadIdx.x] = mn;
-  smx[threadIdx.x] = mx;
-  ssl[threadIdx.x] = slo;
-  ssh[threadIdx.x] = shi;
   __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) {
-      smn[threadIdx.x] = fminf(smn[threadIdx.x], smn[threadIdx.x + o]);
-      smx[threadIdx.x] = fmaxf(smx[threadIdx.x], smx[threadIdx.x + o]);
-      ssl[threadIdx.x] += ssl[threadIdx.x + o];
-      ssh[threadIdx.x] += ssh[threadIdx.x + o];
-    }
-    __syncthreads();
+  if (threadIdx.x < NV) {
+    double s = 0.0;
+#pragma unroll
+    for (int w = 0; w < kOcBlock / 32; ++w) s += sh[w][threadIdx.x];
+    part[static_cast<size_t>(blockIdx.x) * NV + threadIdx.x] = s;
   }
+}
+
+// True in every thread of the block that arrives last; its view of part is then complete.
+__device__ __forceinline__ bool oc_last_block(double* oc) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
   if (threadIdx.x == 0) {
-    double* o = part + 4 * static_cast<size_t>(blockIdx.x);
-    o[0] = smn[0];
-    o[1] = smx[0];
-    o[2] = ssl[0];
-    o[3] = ssh[0];
+    unsigned* ticket = reinterpret_cast<unsigned*>(oc + OC_TICKET);
+    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    if (last) *ticket = 0u;
+  }
+  __syncthreads();
+  if (last) __threadfence();
+  return last;
+}
+
+// Sums over blocks of the NV partials (thread t: value t % NV, rows t / NV + i * per; then the
+// rows' sums in order), valid in thread k < NV.
+template <int NV>
+__device__ __forceinline__ double oc_total(const double* part, int nblk) {
+  __shared__ double sh[kOcBlock];
+  constexpr int per = kOcBlock / NV;
+  const int k = threadIdx.x % NV, r0 = threadIdx.x / NV;
+  double s = 0.0;
+  if (r0 < per)
+#pragma unroll 8
+    for (int r = r0; r < nblk; r += per) s += __ldcg(part + static_cast<size_t>(r) * NV + k);
+  sh[threadIdx.x] = s;
+  __syncthreads();
+  double acc = 0.0;
+  if (threadIdx.x < NV)
+    for (int r = 0; r < per; ++r) acc += sh[r * NV + threadIdx.x];
+  return acc;
+}
+
+// Thread k < kOcCand: candidate k of the bracket (log-uniform).
+__device__ __forceinline__ void oc_make_candidates(double* oc, double lo, double hi) {
+  if (threadIdx.x < kOcCand) {
+    const double lr = log(hi / lo);
+    oc[OC_CAND + threadIdx.x] = lo * exp(lr * (threadIdx.x + 1) / (kOcCand + 1));
   }
 }
 
-__device__ void oc_make_candidates(double* oc) {
-  const double lo = oc[OC_SLO], hi = oc[OC_SHI];
-  const double lr = log(hi / lo);
-  for (int k = 0; k < kOcCand; ++k) oc[OC_CAND + k] = lo * exp(lr * (k + 1) / (kOcCand + 1));
-}
-
-__global__ void k_oc_setup_final(const double* __restrict__ part, int nblk, size_t N, double V,
-                                 double* __restrict__ oc) {
-  if (threadIdx.x != 0) return;
-  double mn = INFINITY, mx = 0.0, sl = 0.0, sh = 0.0;
-  for (int b = 0; b < nblk; ++b) {
-    mn = fmin(mn, part[4 * b]);
-    mx = fmax(mx, part[4 * b + 1]);
-    sl += part[4 * b + 2];
-    sh += part[4 * b + 3];
+// W consecutive elements per step (4: 16-byte accesses; the launcher checks the alignment).
+// base -> tmp; min lo/base, max hi/base over base > 0, sum lo, sum hi: the bracket of s.
+template <int W>
+__global__ void __launch_bounds__(kOcBlock) k_oc_setup(const float* __restrict__ rho,
+                                                       const float* __restrict__ dc,
+                                                       float* __restrict__ base, size_t N, float eta,
+                                                       float move, float rmin, double V,
+                                                       double* __restrict__ part, double* __restrict__ oc) {
+  float mn = INFINITY, mx = 0.f;
+  float hi2[2] = {0.f, 0.f}, lo2[2] = {0.f, 0.f};
+  for (size_t i = static_cast<size_t>(blockIdx.x) * kOcBlock + threadIdx.x; i < N / W;
+       i += static_cast<size_t>(gridDim.x) * kOcBlock) {
+    const Pk<W> r = ldg_pk<W>(rho + i * W), d = ldg_pk<W>(dc + i * W);
+    Pk<W> bs;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      const float D = fmaxf(-d.v[w], 0.f);
+      bs.v[w] = D > 0.f ? r.v[w] * powf(D, eta) : 0.f;
+      const float lo = oc_lo(r.v[w], move, rmin), hi = oc_hi(r.v[w], move);
+      pair_add(hi2[0], lo2[0], lo);
+      pair_add(hi2[1], lo2[1], hi);
+      if (bs.v[w] > 0.f) {
+        mn = fminf(mn, lo / bs.v[w]);
+        mx = fmaxf(mx, hi / bs.v[w]);
+      }
+    }
+    st_pk<W>(base + i * W, bs);
   }
-  const double vlo = sl / static_cast<double>(N), vhi = sh / static_cast<double>(N);
-  oc[OC_SLO] = mn;
-  oc[OC_SHI] = mx;
-  if (!(mx > 0.0) || !isfinite(mn) || vlo >= V) oc[OC_MODE] = 2;     // everything at its lower bound
-  else if (vhi <= V) oc[OC_MODE] = 1;                                // everything at its upper bound
-  else oc[OC_MODE] = 0;
-  if (oc[OC_MODE] == 0) oc_make_candidates(oc);
+  __shared__ float smn[kOcBlock / 32], smx[kOcBlock / 32];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    mn = fminf(mn, __shfl_down_sync(0xffffffffu, mn, o));
+    mx = fmaxf(mx, __shfl_down_sync(0xffffffffu, mx, o));
+  }
+  if ((threadIdx.x & 31) == 0) {
+    smn[threadIdx.x >> 5] = mn;
+    smx[threadIdx.x >> 5] = mx;
+  }
+  pair_block_sum<2>(hi2, lo2, part);   // its barrier also publishes smn and smx
+  double* ext = part + 2 * static_cast<size_t>(gridDim.x);
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kOcBlock / 32; ++w) {
+      smn[0] = fminf(smn[0], smn[w]);
+      smx[0] = fmaxf(smx[0], smx[w]);
+    }
+    ext[2 * blockIdx.x] = smn[0];
+    ext[2 * blockIdx.x + 1] = smx[0];
+  }
+  if (!oc_last_block(oc)) return;
+  __shared__ double tot[4];
+  const double t = oc_total<2>(part, gridDim.x);
+  if (threadIdx.x < 2) tot[threadIdx.x] = t;
+  if (threadIdx.x >= 32 && threadIdx.x < 64) {
+    double a = INFINITY, b = 0.0;
+    for (int i = threadIdx.x - 32; i < static_cast<int>(gridDim.x); i += 32) {
+      a = fmin(a, __ldcg(ext + 2 * i));
+      b = fmax(b, __ldcg(ext + 2 * i + 1));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      a = fmin(a, __shfl_down_sync(0xffffffffu, a, o));
+      b = fmax(b, __shfl_down_sync(0xffffffffu, b, o));
+    }
+    if (threadIdx.x == 32) {
+      tot[2] = a;
+      tot[3] = b;
+    }
+  }
+  __syncthreads();
+  const double lo = tot[2], hi = tot[3];
+  const double vlo = tot[0] / static_cast<double>(N), vhi = tot[1] / static_cast<double>(N);
+  int mode = 0;
+  if (!(hi > 0.0) || !isfinite(lo) || vlo >= V) mode = 2;     // everything at its lower bound
+  else if (vhi <= V) mode = 1;                                // everything at its upper bound
+  if (threadIdx.x == 0) {
+    oc[OC_SLO] = lo;
+    oc[OC_SHI] = hi;
+    oc[OC_MODE] = mode;
+  }
+  if (mode == 0) oc_make_candidates(oc, lo, hi);
 }
 
-__global__ void __launch_bounds__(256) k_oc_pass(const float* __restrict__ rho,
-                                                 const float* __restrict__ base, size_t N,
-                                                 float move, float rmin,
-                                                 const double* __restrict__ oc,
-                                                 double* __restrict__ part) {
+// Volumes of the 15 candidates; the last block narrows the bracket to the two they straddle V
+// with and makes the next candidates. stride: distance of a run's terms (a run: 8 of the
+// elements v, v + stride, v + 2 stride, ... of one v < stride).
+__global__ void __launch_bounds__(kOcBlock) k_oc_pass(const float* __restrict__ rho,
+                                                      const float* __restrict__ base, size_t N,
+                                                      size_t stride, float move, float rmin, double V,
+                                                      double* oc, double* __restrict__ part) {
   if (oc[OC_MODE] != 0) return;
-  float cand[kOcCand], acc[kOcCand];
-  double accd[kOcCand];
+  float cand[kOcCand], hi[kOcCand], lo[kOcCand];
 #pragma unroll
   for (int k = 0; k < kOcCand; ++k) {
     cand[k] = static_cast<float>(oc[OC_CAND + k]);
-    acc[k] = 0.f;
-    accd[k] = 0.0;
+    hi[k] = lo[k] = 0.f;
   }
-  int cnt = 0;
-  for (size_t e = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < N;
-       e += static_cast<size_t>(gridDim.x) * blockDim.x) {
-    const float r = __ldg(rho + e), bs = __ldg(base + e);
-    const float lo = oc_lo(r, move, rmin), hi = oc_hi(r, move);
+  const size_t runs = (N + 8 * stride - 1) / (8 * stride);
+  for (size_t run = 0; run < runs; ++run)
+    for (size_t v = static_cast<size_t>(blockIdx.x) * kOcBlock + threadIdx.x; v < stride;
+         v += static_cast<size_t>(gridDim.x) * kOcBlock) {
+      const size_t e0 = v + 8 * stride * run;
+      if (e0 >= N) continue;
+      float r[8], bs[8];
 #pragma unroll
-    for (int k = 0; k < kOcCand; ++k) acc[k] += fminf(fmaxf(bs * cand[k], lo), hi);
-    if (++cnt == 8) {   // FP32 over at most 8 terms, FP64 beyond
-#pragma unroll
-      for (int k = 0; k < kOcCand; ++k) {
-        accd[k] += acc[k];
-        acc[k] = 0.f;
+      for (int t = 0; t < 8; ++t) {
+        const size_t e = e0 + t * stride;
+        r[t] = e < N ? __ldg(rho + e) : -1.f;
+        bs[t] = e < N ? __ldg(base + e) : 0.f;
       }
-      cnt = 0;
-    }
-  }
+      float acc[kOcCand];
 #pragma unroll
-  for (int k = 0; k < kOcCand; ++k) accd[k] += acc[k];
-  block_sum_store_d<kOcCand>(accd, part);
-}
-
-// sums: the kOcCand volume sums already reduced over blocks.
-__global__ void k_oc_pass_final(const double* __restrict__ sums, size_t N, double V,
-                                double* __restrict__ oc) {
-  if (threadIdx.x != 0 || oc[OC_MODE] != 0) return;
-  double lo = oc[OC_SLO], hi = oc[OC_SHI];
-  for (int k = 0; k < kOcCand; ++k) {
-    const double vol = sums[k] / static_cast<double>(N);
-    if (vol <= V) {
-      lo = oc[OC_CAND + k];
-    } else {
-      hi = oc[OC_CAND + k];
-      break;
+      for (int k = 0; k < kOcCand; ++k) acc[k] = 0.f;
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        if (e0 + t * stride >= N) break;
+        const float l = oc_lo(r[t], move, rmin), h = oc_hi(r[t], move);
+#pragma unroll
+        for (int k = 0; k < kOcCand; ++k) acc[k] += fminf(fmaxf(bs[t] * cand[k], l), h);
+      }
+#pragma unroll
+      for (int k = 0; k < kOcCand; ++k) pair_add(hi[k], lo[k], acc[k]);
     }
+  pair_block_sum<kOcCand>(hi, lo, part);
+  if (!oc_last_block(oc)) return;
+  __shared__ double vol[kOcCand], br[2];
+  const double t = oc_total<kOcCand>(part, gridDim.x);
+  if (threadIdx.x < kOcCand) vol[threadIdx.x] = t / static_cast<double>(N);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double a = oc[OC_SLO], b = oc[OC_SHI];
+    for (int k = 0; k < kOcCand; ++k) {
+      if (vol[k] <= V) {
+        a = oc[OC_CAND + k];
+      } else {
+        b = oc[OC_CAND + k];
+        break;
+      }
+    }
+    oc[OC_SLO] = br[0] = a;
+    oc[OC_SHI] = br[1] = b;
   }
-  oc[OC_SLO] = lo;
-  oc[OC_SHI] = hi;
-  oc_make_candidates(oc);
+  __syncthreads();
+  oc_make_candidates(oc, br[0], br[1]);
 }
 
-__global__ void __launch_bounds__(256) k_oc_apply(float* __restrict__ rho,
-                                                  const float* __restrict__ base, size_t N,
-                                                  float move, float rmin,
-                                                  const double* __restrict__ oc,
-                                                  double* __restrict__ part) {
+template <int W>
+__global__ void __launch_bounds__(kOcBlock) k_oc_apply(float* __restrict__ rho,
+                                                       const float* __restrict__ base, size_t N,
+                                                       float move, float rmin, double* __restrict__ oc,
+                                                       double* __restrict__ part) {
   const int mode = static_cast<int>(oc[OC_MODE]);
   const float s = mode == 2 ? 0.f : static_cast<float>(mode == 1 ? oc[OC_SHI] : oc[OC_SLO]);
   float ch = 0.f;
-  for (size_t e = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < N;
-       e += static_cast<size_t>(gridDim.x) * blockDim.x) {
-    const float r = rho[e];
-    const float lo = oc_lo(r, move, rmin), hi = oc_hi(r, move);
-    const float nr = fminf(fmaxf(base[e] * s, lo), hi);
-    ch = fmaxf(ch, fabsf(nr - r));
-    rho[e] = nr;
+  for (size_t i = static_cast<size_t>(blockIdx.x) * kOcBlock + threadIdx.x; i < N / W;
+       i += static_cast<size_t>(gridDim.x) * kOcBlock) {
+    const Pk<W> r = ld_pk<W>(rho + i * W), bs = ldg_pk<W>(base + i * W);
+    Pk<W> nr;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      nr.v[w] = fminf(fmaxf(bs.v[w] * s, oc_lo(r.v[w], move, rmin)), oc_hi(r.v[w], move));
+      ch = fmaxf(ch, fabsf(nr.v[w] - r.v[w]));
+    }
+    st_pk<W>(rho + i * W, nr);
   }
-  __shared__ float sm[256];
-  sm[threadIdx.x] = ch;
+  __shared__ float sm[kOcBlock / 32];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) ch = fmaxf(ch, __shfl_down_sync(0xffffffffu, ch, o));
+  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = ch;
   __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) sm[threadIdx.x] = fmaxf(sm[threadIdx.x], sm[threadIdx.x + o]);
-    __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kOcBlock / 32; ++w) ch = fmaxf(ch, sm[w]);
+    part[blockIdx.x] = ch;
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = sm[0];
-}
-
-__global__ void k_max_partials(const double* __restrict__ part, int nblk, double* __restrict__ out) {
-  if (threadIdx.x != 0) return;
-  double m = 0.0;
-  for (int b = 0; b < nblk; ++b) m = fmax(m, part[b]);
-  *out = m;
+  if (!oc_last_block(oc)) return;
+  if (threadIdx.x < 32) {
+    double m = 0.0;
+    for (int i = threadIdx.x; i < static_cast<int>(gridDim.x); i += 32) m = fmax(m, __ldcg(part + i));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
+    if (threadIdx.x == 0) oc[OC_CHANGE] = m;
+  }
 }
 
 // Orbit averages under a cube symmetry group (Sec. 6.1). Thread per element: it forms
@@ -716,39 +857,59 @@ cudaError_t launch_symmetrize(const SymParam& sp, int n, const float* in, float*
   return cudaGetLastError();
 }
 
+namespace {
+// The 27-offset form's weights, or false when fp is another stencil (27 offsets are exactly the
+// unit cube: the next ones, at distance 2, come six at a time with 33).
+bool filter27(const FilterParam& fp, Filter27& F) {
+  if (fp.count != 27) return false;
+  F = {{fp.w[13], fp.w[14], fp.w[17], fp.w[26]}, fp.inv_wsum};   // centre, +x, +x+y, +x+y+z
+  return true;
+}
+}  // namespace
+
 cudaError_t launch_filter(const FilterParam& fp, int n, const float* in, float* out,
                           cudaStream_t s) {
   const size_t N = static_cast<size_t>(n) * n * n;
-  k_filter<false><<<grid_for(N, 256), 256, 0, s>>>(fp, n, in, nullptr, 0.f, out);
+  Filter27 F;
+  if (filter27(fp, F)) k_filter27<false><<<grid_for(N, 256), 256, 0, s>>>(F, n, in, nullptr, 0.f, out);
+  else k_filter<false><<<grid_for(N, 256), 256, 0, s>>>(fp, n, in, nullptr, 0.f, out);
   return cudaGetLastError();
 }
 
 cudaError_t launch_sensitivity_filter(const FilterParam& fp, int n, const float* rho, const float* dc,
                                       float gamma, float* out, cudaStream_t s) {
   const size_t N = static_cast<size_t>(n) * n * n;
-  k_filter<true><<<grid_for(N, 256), 256, 0, s>>>(fp, n, dc, rho, gamma, out);
+  Filter27 F;
+  if (filter27(fp, F)) k_filter27<true><<<grid_for(N, 256), 256, 0, s>>>(F, n, dc, rho, gamma, out);
+  else k_filter<true><<<grid_for(N, 256), 256, 0, s>>>(fp, n, dc, rho, gamma, out);
   return cudaGetLastError();
 }
 
-cudaError_t launch_oc(homo_ctx* c, const float* dc, float* rho, double volfrac, double move,
-                      double eta, double rho_min, double* change) {
+namespace {
+template <int W>
+cudaError_t oc_run(homo_ctx* c, const float* dc, float* rho, double volfrac, double move, double eta, double rho_min) {
   const size_t N = c->N;
-  const int g = grid_for(N, 256);
+  const int g = static_cast<int>(std::min<size_t>((N / W + kOcBlock - 1) / kOcBlock, kOcGrid));
+  const size_t stride = static_cast<size_t>(grid_for(N, kOcBlock)) * kOcBlock;
+  const int gp = std::min(grid_for(N, kOcBlock), kOcGrid);
   double* oc = c->scal + S_OC;
   cudaStream_t s = c->stream;
-  k_oc_setup<<<g, 256, 0, s>>>(rho, dc, c->tmp, N, static_cast<float>(eta), static_cast<float>(move),
-                               static_cast<float>(rho_min), c->part);
-  k_oc_setup_final<<<1, 32, 0, s>>>(c->part, g, N, volfrac, oc);
-  for (int it = 0; it < kOcPasses; ++it) {
-    k_oc_pass<<<g, 256, 0, s>>>(rho, c->tmp, N, static_cast<float>(move), static_cast<float>(rho_min), oc,
-                                c->part);
-    k_sum_partials<kSumOnly><<<1, 256, 0, s>>>(c->part, g, kOcCand, oc + OC_SUMS, nullptr, 0, 0.0, 0.0);
-    k_oc_pass_final<<<1, 32, 0, s>>>(oc + OC_SUMS, N, volfrac, oc);
-  }
-  k_oc_apply<<<g, 256, 0, s>>>(rho, c->tmp, N, static_cast<float>(move), static_cast<float>(rho_min), oc,
-                               c->part);
-  k_max_partials<<<1, 32, 0, s>>>(c->part, g, oc + OC_CHANGE);
-  cudaError_t e = cudaGetLastError();
+  const float mv = static_cast<float>(move), rm = static_cast<float>(rho_min);
+  k_oc_setup<W><<<g, kOcBlock, 0, s>>>(rho, dc, c->tmp, N, static_cast<float>(eta), mv, rm, volfrac, c->part, oc);
+  for (int it = 0; it < kOcPasses; ++it)
+    k_oc_pass<<<gp, kOcBlock, 0, s>>>(rho, c->tmp, N, stride, mv, rm, volfrac, oc, c->part);
+  k_oc_apply<W><<<g, kOcBlock, 0, s>>>(rho, c->tmp, N, mv, rm, oc, c->part);
+  return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_oc(homo_ctx* c, const float* dc, float* rho, double volfrac, double move,
+                      double eta, double rho_min, double* change) {
+  double* oc = c->scal + S_OC;
+  cudaStream_t s = c->stream;
+  const bool vec = c->N % 4 == 0 && (reinterpret_cast<uintptr_t>(dc) | reinterpret_cast<uintptr_t>(rho)) % 16 == 0;
+  cudaError_t e = vec ? oc_run<4>(c, dc, rho, volfrac, move, eta, rho_min)
+                      : oc_run<1>(c, dc, rho, volfrac, move, eta, rho_min);
   if (e != cudaSuccess) return e;
   if (change) {
     e = cudaMemcpyAsync(c->hscal + S_OC + OC_CHANGE, oc + OC_CHANGE, sizeof(double),
