@@ -2,21 +2,28 @@
 // (tcgen05.mma, accumulators in tensor memory). Implicit GEMM: M = 128 voxels, N = 32
 // output channels, K = 27 taps x c_in, BF16 operands, FP32 accumulation.
 //
-// A persistent CTA (4 warps) keeps the layer's weights in shared memory and walks tiles of
-// 30 x 4 x 2 output voxels. Each tile's periodic halo box (32 x 6 x 4 voxels, all input
-// channels) is staged with 16-byte asynchronous copies into a K-major, non-swizzled
-// operand layout whose rows are 16 bytes apart along the box's (z, y, x) order: channel
-// chunk c (8 channels) of box row r sits at plane c, row r. For a tap with offset d, the
-// 128 rows of the A operand are then the output rows shifted by the constant row offset of
-// d, so every tap's operand is the same staged box seen through a shifted descriptor, with
-// no per-tap copy. Output rows 0 and 31 of each 32-row run are halo positions: computed and
-// discarded (30 of every 32 rows are outputs).
+// A persistent CTA keeps the layer's weights in shared memory and walks tiles of 30 x 4 x 2
+// output voxels. Each tile's periodic halo box (32 x 6 x 4 voxels, all input channels) is
+// staged with 16-byte asynchronous copies into a K-major, non-swizzled operand layout whose
+// rows are 16 bytes apart along the box's (z, y, x) order: channel chunk c (8 channels) of
+// box row r sits at plane c, row r. For a tap with offset d, the 128 rows of the A operand
+// are then the output rows shifted by the constant row offset of d, so every tap's operand
+// is the same staged box seen through a shifted descriptor, with no per-tap copy. Output
+// rows 0 and 31 of each 32-row run are halo positions: computed and discarded (30 of every
+// 32 rows are outputs).
 //
-// One thread issues the tile's 27 x c_in/16 MMAs per output plane into two 32-column TMEM
-// accumulators and commits them to an mbarrier; after a bounded wait every warp reads its
-// 32 TMEM lanes (one voxel per thread, 32 channels) and applies the same epilogues as the
-// other layers: bias, residual, ReLU or a backward ReLU mask, BF16 voxel-major output or
-// scaled FP32 displacement planes.
+// Nine warps in three roles, handing tiles on through mbarriers, so that the copies of the
+// next tiles, the MMAs of one and the epilogue of the one before run at the same time:
+//   warps 4..7  copy boxes into a ring of kStages buffers;
+//   warp 8      issues (one elected lane) the tile's 27 x c_in/16 MMAs per output plane into one of
+//               two pairs of 32-column TMEM accumulators and commits them to the barriers
+//               that free the box and publish the accumulators;
+//   warps 0..3  read their 32 TMEM lanes (one voxel per thread, 32 channels), free the
+//               accumulators and apply the epilogue: bias, residual, ReLU or a backward ReLU
+//               mask, BF16 voxel-major output or scaled FP32 displacement planes.
+// Every wait is bounded. Bound: an MMA of 128 x 32 x 16 reads 5 KB of operands for 16 cycles
+// of math, so about 40 cycles of shared-memory bandwidth each. 64^3, 32 -> 32 channels: 70 -> 39 us
+// (four warps did all three in turn, two CTAs per SM: tensor pipe 14 % busy).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -36,19 +43,22 @@ constexpr int kBoxRows = BXr * BYr * BZr;                  // 768
 constexpr int kRowPad = 1;                                 // row 0: guard below the box
 constexpr int kRows = 776;                                 // >= kRowPad + kBoxRows + 1, multiple of 8
 constexpr int kPlaneBytes = kRows * 16;                    // one 8-channel chunk of every row
-constexpr int kThreads = 128;
-constexpr int kTmemCols = 64;                              // two 128 x 32 FP32 accumulators
+constexpr int kThreads = 9 * 32;                           // epilogue, copy and MMA warps
+constexpr int kRole = 128;                                 // threads of the epilogue and of the copy role
+constexpr int kStages = 3;                                 // boxes in flight
+constexpr int kTmemCols = 128;                             // two pairs of 128 x 32 FP32 accumulators
 constexpr long long kWaitLimit = 1LL << 18;                // bounded mbarrier polls (~1 s on a GB300)
 
 static_assert(kRowPad + kBoxRows + 1 <= kRows, "guard rows");
-static_assert(kThreads == 4 * 32 && TYo == 4, "warp w owns output row y = w of each plane");
+static_assert(kRole == 4 * 32 && TYo == 4, "epilogue warp w owns output row y = w of each plane");
 
 template <int CIN>
 struct TcShape {
   static constexpr int kChunks = CIN / 8;
   static constexpr int kBoxBytes = kChunks * kPlaneBytes;
   static constexpr int kWBytes = kTaps * kChunks * kC * 16;
-  static constexpr int kBytes = kBoxBytes + kWBytes + 64;   // + mbarrier and TMEM address
+  static constexpr int kBarriers = 2 * kStages + 4;
+  static constexpr int kBytes = kStages * kBoxBytes + kWBytes + 8 * kBarriers + 16;   // + mbarriers, TMEM address
 };
 
 struct TcScale {
@@ -70,6 +80,9 @@ __device__ __forceinline__ int wrapc(int a, int n) {
   return a < 0 ? a + n : a;
 }
 
+// the same for -n <= a < 2 n
+__device__ __forceinline__ int wrap1(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
+
 // Shared-memory matrix descriptor of a K-major, non-swizzled operand: core matrices of
 // 8 rows x 16 bytes with rows 16 bytes apart, 8-row groups SBO bytes apart along M/N and
 // 16-byte K chunks LBO bytes apart; descriptor version 1 (bits 46-47), no base offset.
@@ -86,17 +99,24 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
 // N = 32, M = 128.
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((kC >> 3) << 17) | ((128 >> 4) << 24);
 
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t accumulate) {
+// One MMA, issued by the lane whose leader flag is set. The whole warp runs the issue loop: a
+// descriptor derived by one lane alone would have to be moved to the uniform registers the
+// instruction reads it from, four moves an MMA.
+__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t accumulate, uint32_t leader) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p, q;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
-      "l"(a), "l"(b), "r"(kIdesc), "r"(accumulate));
+      "setp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
+      "l"(a), "l"(b), "r"(kIdesc), "r"(accumulate), "r"(leader));
 }
 
-__device__ __forceinline__ void mma_commit(uint32_t mbar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(mbar)
-               : "memory");
+__device__ __forceinline__ void mma_commit(uint32_t mbar, uint32_t leader) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(mbar), "r"(leader)
+      : "memory");
 }
 
 // Poll the mbarrier for phase `parity` at most kWaitLimit times; true once it completed.
@@ -144,8 +164,58 @@ __device__ __forceinline__ float2 unbf2(uint32_t u) {
   return __bfloat1622float2(h);
 }
 
+__device__ __forceinline__ void mbar_init(uint32_t mbar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(mbar), "r"(count) : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(mbar) : "memory");
+}
+
+// The epilogue of one output voxel: acc[32] of the MMA.
+template <int EPI>
+__device__ __forceinline__ void conv_epilogue(const float (&acc)[32], const float (&bo)[32], const float (&so)[6],
+                                              size_t v, size_t N, const uint4 (&rr)[4], const uint4 (&mm)[4], bool has_res,
+                                              __nv_bfloat16* __restrict__ out, float* __restrict__ outf) {
+  if (EPI == HOMO_NN_PLANES || EPI == HOMO_NN_PLANES_ADD) {
+#pragma unroll
+    for (int o = 0; o < 18; ++o) {
+      float* d = outf + static_cast<size_t>(o) * N + v;
+      const float val = so[o / 3] * (acc[o] + bo[o]);
+      *d = EPI == HOMO_NN_PLANES_ADD ? *d + val : val;
+    }
+    return;
+  }
+  uint4* dst = reinterpret_cast<uint4*>(out + v * kC);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const uint32_t r4[4] = {rr[q].x, rr[q].y, rr[q].z, rr[q].w}, m4[4] = {mm[q].x, mm[q].y, mm[q].z, mm[q].w};
+    uint32_t pk[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int o = 8 * q + 2 * j;
+      float v0 = acc[o] + bo[o], v1 = acc[o + 1] + bo[o + 1];
+      if (has_res) {
+        const float2 r = unbf2(r4[j]);
+        v0 += r.x;
+        v1 += r.y;
+      }
+      if (EPI == HOMO_NN_RELU) {
+        v0 = fmaxf(v0, 0.f);
+        v1 = fmaxf(v1, 0.f);
+      } else {
+        const float2 m = unbf2(m4[j]);
+        v0 = m.x > 0.f ? v0 : 0.f;
+        v1 = m.y > 0.f ? v1 : 0.f;
+      }
+      pk[j] = bf2(v0, v1);
+    }
+    dst[q] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+  }
+}
+
 template <int CIN, int EPI>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kThreads, 1)
     k_conv3d_tc(int n, int tiles_x, int tiles_y, int ntiles, const __nv_bfloat16* __restrict__ x,
                 const __nv_bfloat16* __restrict__ w, const float* __restrict__ bias,
                 const __nv_bfloat16* __restrict__ res, const __nv_bfloat16* __restrict__ mask,
@@ -153,13 +223,17 @@ __global__ void __launch_bounds__(kThreads, 2)
   using S = TcShape<CIN>;
   constexpr int kCh = S::kChunks;
   extern __shared__ __align__(128) unsigned char smem[];
-  unsigned char* box = smem;                              // kCh planes x kRows x 16 B
-  unsigned char* wsm = smem + S::kBoxBytes;               // [tap][chunk][o][16 B]
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(smem + S::kBoxBytes + S::kWBytes);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mbar + 1);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  unsigned char* wsm = smem + kStages * S::kBoxBytes;     // [tap][chunk][o][16 B]
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(wsm + S::kWBytes);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mbar + S::kBarriers);
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const size_t N = static_cast<size_t>(n) * n * n;
-  const uint32_t box_s = smem_u32(box), w_s = smem_u32(wsm), mbar_s = smem_u32(mbar);
+  const uint32_t box_s = smem_u32(smem), w_s = smem_u32(wsm), bar_s = smem_u32(mbar);
+  // barriers: box filled / box free per stage, accumulators filled / free per pair
+  auto full = [&](int s) { return bar_s + 8u * s; };
+  auto empty = [&](int s) { return bar_s + 8u * (kStages + s); };
+  auto tfull = [&](int t) { return bar_s + 8u * (2 * kStages + t); };
+  auto tempty = [&](int t) { return bar_s + 8u * (2 * kStages + 2 + t); };
 
   // weights once per CTA; guard rows of every plane zeroed once (never loaded)
   for (int c = tid; c < kTaps * kC * kCh; c += kThreads) {
@@ -167,13 +241,20 @@ __global__ void __launch_bounds__(kThreads, 2)
     cp_async16(w_s + ((tap * kCh + ch) * kC + o) * 16, w + (static_cast<size_t>(tap) * kC + o) * CIN + ch * 8);
   }
   asm volatile("cp.async.commit_group;\n" ::: "memory");
-  for (int c = tid; c < kCh * (kRows - kBoxRows); c += kThreads) {
-    const int ch = c / (kRows - kBoxRows), r = c % (kRows - kBoxRows);
+  for (int c = tid; c < kStages * kCh * (kRows - kBoxRows); c += kThreads) {
+    const int p = c / (kRows - kBoxRows), r = c % (kRows - kBoxRows);   // plane p of all stages
     const int row = r < kRowPad ? r : kRowPad + kBoxRows + (r - kRowPad);
-    *reinterpret_cast<uint4*>(box + ch * kPlaneBytes + row * 16) = make_uint4(0u, 0u, 0u, 0u);
+    *reinterpret_cast<uint4*>(smem + p * kPlaneBytes + row * 16) = make_uint4(0u, 0u, 0u, 0u);
   }
   if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(mbar_s) : "memory");
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(full(s), kRole);
+      mbar_init(empty(s), 1);
+    }
+    for (int t = 0; t < 2; ++t) {
+      mbar_init(tfull(t), 1);
+      mbar_init(tempty(t), kRole);
+    }
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   if (warp == 0) {
@@ -182,125 +263,127 @@ __global__ void __launch_bounds__(kThreads, 2)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
   }
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // weights and guard rows visible to the tensor core
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   const uint32_t tmem = *tmem_slot;
 
-  // this thread's TMEM lane (warp w reads lanes 32 w .. 32 w + 31) and output position
-  const uint32_t tlane = tmem + (static_cast<uint32_t>(32 * warp) << 16);
-  const bool xout = lane >= 1 && lane <= TXo;             // rows 0 and 31 of a run are halo
-  float bo[kC], so[18];
+  if (warp >= 4 && warp < 8) {
+    // ---- copies: box row br = t + 128 k (k < 6) and all its chunks per thread
+    const int t = tid - kRole;
+    int k = 0;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++k) {
+      const int st = k % kStages;
+      if (!mbar_wait(empty(st), ((k / kStages) & 1) ^ 1)) break;   // a fresh barrier passes parity 1
+      const int tx = tile % tiles_x, rest = tile / tiles_x;
+      const int x0 = tx * TXo, y0 = (rest % tiles_y) * TYo, z0 = (rest / tiles_y) * TZo;
+      const uint32_t dst = box_s + st * S::kBoxBytes + kRowPad * 16;
 #pragma unroll
-  for (int o = 0; o < kC; ++o) bo[o] = (EPI != HOMO_NN_MASK && bias) ? bias[o] : 0.f;
+      for (int q = 0; q < kBoxRows / kRole; ++q) {
+        const int br = t + kRole * q;
+        const int bx = br % BXr, by = (br / BXr) % BYr, bz = br / (BXr * BYr);
+        // a box spans at most x0 - 1 .. x0 + 30: past one period only on grids below 32
+        const int gx = x0 - 1 + bx, gy = y0 - 1 + by, gz = z0 - 1 + bz;
+        const size_t gv = n >= BXr ? static_cast<size_t>(wrap1(gx, n)) +
+                                         static_cast<size_t>(n) * (wrap1(gy, n) + static_cast<size_t>(n) * wrap1(gz, n))
+                                   : static_cast<size_t>(wrapc(gx, n)) +
+                                         static_cast<size_t>(n) * (wrapc(gy, n) + static_cast<size_t>(n) * wrapc(gz, n));
+        const __nv_bfloat16* src = x + gv * CIN;
 #pragma unroll
-  for (int o = 0; o < 18; ++o) so[o] = sc.s[o / 3];
-
-  uint32_t phase = 0;
-  bool timed_out = false;
-  for (int tile = blockIdx.x; tile < ntiles && !timed_out; tile += gridDim.x) {
-    const int tx = tile % tiles_x, rest = tile / tiles_x;
-    const int ty = rest % tiles_y, tz = rest / tiles_y;
-    const int x0 = tx * TXo, y0 = ty * TYo, z0 = tz * TZo;
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();   // the previous tile's TMEM reads and box reads are finished
-    for (int c = tid; c < kBoxRows * kCh; c += kThreads) {
-      const int ch = c % kCh, br = c / kCh;
-      const int bx = br % BXr, by = (br / BXr) % BYr, bz = br / (BXr * BYr);
-      const size_t gv = static_cast<size_t>(wrapc(x0 - 1 + bx, n)) +
-                        static_cast<size_t>(n) * (wrapc(y0 - 1 + by, n) + static_cast<size_t>(n) * wrapc(z0 - 1 + bz, n));
-      cp_async16(box_s + ch * kPlaneBytes + (kRowPad + br) * 16, x + gv * CIN + ch * 8);
+        for (int ch = 0; ch < kCh; ++ch) cp_async16(dst + ch * kPlaneBytes + br * 16, src + ch * 8);
+      }
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+      if (k > 0) {   // the previous tile's copies have landed: hand it on
+        asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        mbar_arrive(full((k - 1) % kStages));
+      }
     }
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // copies visible to the tensor core
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    if (tid == 0) {
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    if (k > 0) mbar_arrive(full((k - 1) % kStages));
+  } else if (warp == 8) {
+    // ---- MMAs: the warp runs the loop, one elected lane issues
+    uint32_t leader;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(leader));
+    const uint64_t a0 = smem_desc(box_s, kPlaneBytes, 128), b0 = smem_desc(w_s, kC * 16, 128);
+    int k = 0;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++k) {
+      const int st = k % kStages, ac = k & 1;
+      const bool ok = mbar_wait(tempty(ac), ((k >> 1) & 1) ^ 1) && mbar_wait(full(st), (k / kStages) & 1);
+      if (!__all_sync(0xffffffffu, ok)) break;
+      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 #pragma unroll 1
       for (int zo = 0; zo < TZo; ++zo) {
-        const int r0 = ((zo + 1) * BYr + 1) * BXr;     // box row of output (x = -1, y = 0, z = zo)
-#pragma unroll 1
-        for (int tap = 0; tap < kTaps; ++tap) {
-          const int dx = tap % 3 - 1, dy = (tap / 3) % 3 - 1, dz = tap / 9 - 1;
-          const int row = kRowPad + r0 + (dz * BYr + dy) * BXr + dx;
+        // box row of output (x = -1, y = 0, z = zo); descriptor addresses count 16-byte rows
+        const uint64_t az = a0 + static_cast<uint32_t>(st * (S::kBoxBytes / 16) + kRowPad + ((zo + 1) * BYr + 1) * BXr);
+        const uint32_t d = tmem + (ac * TZo + zo) * kC;
 #pragma unroll
-          for (int ks = 0; ks < CIN / 16; ++ks) {
-            const uint64_t a = smem_desc(box_s + (2 * ks) * kPlaneBytes + row * 16, kPlaneBytes, 128);
-            const uint64_t b = smem_desc(w_s + (tap * kCh + 2 * ks) * kC * 16, kC * 16, 128);
-            mma_bf16(tmem + zo * kC, a, b, (tap | ks) != 0 ? 1u : 0u);
-          }
+        for (int tap = 0; tap < kTaps; ++tap) {
+          const int row = ((tap / 9 - 1) * BYr + (tap / 3) % 3 - 1) * BXr + tap % 3 - 1;
+#pragma unroll
+          for (int ks = 0; ks < CIN / 16; ++ks)
+            mma_bf16(d, az + static_cast<int64_t>(row + 2 * ks * kRows), b0 + (tap * kCh + 2 * ks) * kC,
+                     (tap | ks) != 0 ? 1u : 0u, leader);
         }
       }
-      mma_commit(mbar_s);
+      mma_commit(empty(st), leader);
+      mma_commit(tfull(ac), leader);
     }
     __syncwarp();
-    const bool ok = mbar_wait(mbar_s, phase);
-    phase ^= 1u;
-    if (__syncthreads_or(!ok)) {         // every thread takes the same decision
-      if (tid == 0) atomicAdd(&g_conv_tc_timeouts, 1);
-      timed_out = true;
-      break;
-    }
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-#pragma unroll 1
-    for (int zo = 0; zo < TZo; ++zo) {
-      float acc[32];
-      tmem_ld32(tlane + zo * kC, acc);
-      const int gx = x0 + lane - 1, gy = y0 + warp, gz = z0 + zo;
-      if (!xout || gx >= n || gy >= n || gz >= n) continue;
-      const size_t v = static_cast<size_t>(gx) + static_cast<size_t>(n) * (gy + static_cast<size_t>(n) * gz);
-      if (EPI == HOMO_NN_PLANES || EPI == HOMO_NN_PLANES_ADD) {
+  } else {
+    // ---- epilogue: this thread's TMEM lane (warp w reads lanes 32 w .. 32 w + 31) and output position
+    const uint32_t tlane = tmem + (static_cast<uint32_t>(32 * warp) << 16);
+    const bool xout = lane >= 1 && lane <= TXo;             // rows 0 and 31 of a run are halo
+    float bo[kC], so[6];
 #pragma unroll
-        for (int o = 0; o < 18; ++o) {
-          float* d = outf + static_cast<size_t>(o) * N + v;
-          const float val = so[o] * (acc[o] + bo[o]);
-          *d = EPI == HOMO_NN_PLANES_ADD ? *d + val : val;
-        }
-        continue;
-      }
-      uint32_t pk[16];
-      const uint4* rp = res ? reinterpret_cast<const uint4*>(res + v * kC) : nullptr;
-      const uint4* mp = EPI == HOMO_NN_MASK ? reinterpret_cast<const uint4*>(mask + v * kC) : nullptr;
+    for (int o = 0; o < kC; ++o) bo[o] = (EPI != HOMO_NN_MASK && bias) ? bias[o] : 0.f;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        uint32_t rr[4] = {0u, 0u, 0u, 0u}, mm[4] = {0u, 0u, 0u, 0u};
-        if (rp) {
-          const uint4 t = rp[q];
-          rr[0] = t.x; rr[1] = t.y; rr[2] = t.z; rr[3] = t.w;
-        }
-        if (mp) {
-          const uint4 t = mp[q];
-          mm[0] = t.x; mm[1] = t.y; mm[2] = t.z; mm[3] = t.w;
-        }
+    for (int o = 0; o < 6; ++o) so[o] = sc.s[o];
+    const bool has_res = (EPI == HOMO_NN_RELU || EPI == HOMO_NN_MASK) && res != nullptr;
+    int k = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++k) {
+      const int ac = k & 1;
+      const int tx = tile % tiles_x, rest = tile / tiles_x;
+      const int gx = tx * TXo + lane - 1, gy = (rest % tiles_y) * TYo + warp, z0 = (rest / tiles_y) * TZo;
+      size_t v[TZo];
+      bool live[TZo];
+      uint4 rr[TZo][4], mm[TZo][4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int o = 8 * q + 2 * j;
-          float v0 = acc[o] + bo[o], v1 = acc[o + 1] + bo[o + 1];
-          if (rp) {
-            const float2 r = unbf2(rr[j]);
-            v0 += r.x;
-            v1 += r.y;
-          }
-          if (EPI == HOMO_NN_RELU) {
-            v0 = fmaxf(v0, 0.f);
-            v1 = fmaxf(v1, 0.f);
-          } else {
-            const float2 m = unbf2(mm[j]);
-            v0 = m.x > 0.f ? v0 : 0.f;
-            v1 = m.y > 0.f ? v1 : 0.f;
-          }
-          pk[4 * q + j] = bf2(v0, v1);
+      for (int zo = 0; zo < TZo; ++zo) {   // the residual and the mask do not wait for the MMAs
+        live[zo] = xout && gx < n && gy < n && z0 + zo < n;
+        v[zo] = live[zo] ? static_cast<size_t>(gx) + static_cast<size_t>(n) * (gy + static_cast<size_t>(n) * (z0 + zo)) : 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          rr[zo][q] = has_res && live[zo] ? reinterpret_cast<const uint4*>(res + v[zo] * kC)[q] : make_uint4(0u, 0u, 0u, 0u);
+          mm[zo][q] = EPI == HOMO_NN_MASK && live[zo] ? reinterpret_cast<const uint4*>(mask + v[zo] * kC)[q]
+                                                      : make_uint4(0u, 0u, 0u, 0u);
         }
       }
-      uint4* dst = reinterpret_cast<uint4*>(out + v * kC);
+      ok = mbar_wait(tfull(ac), (k >> 1) & 1);
+      if (!__all_sync(0xffffffffu, ok)) {   // a warp takes one decision (its TMEM loads are collective)
+        ok = false;
+        break;
+      }
+      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+      float acc[TZo][32];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) dst[q] = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+      for (int zo = 0; zo < TZo; ++zo) tmem_ld32(tlane + (ac * TZo + zo) * kC, acc[zo]);
+      asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+      mbar_arrive(tempty(ac));
+#pragma unroll
+      for (int zo = 0; zo < TZo; ++zo)
+        if (live[zo]) conv_epilogue<EPI>(acc[zo], bo, so, v[zo], N, rr[zo], mm[zo], has_res, out, outf);
     }
-  }
-  if (timed_out) {
-    // the tile's MMAs may still be running: give them one more bounded wait before TMEM is freed
-    mbar_wait(mbar_s, phase ^ 1u);
+    if (!ok && lane == 0) {
+      // give up on this tile and the rest; MMAs still running get one more bounded wait before
+      // the TMEM is freed (the other roles' waits then run out too)
+      if (warp == 0) atomicAdd(&g_conv_tc_timeouts, 1);
+      mbar_wait(tfull(k & 1), (k >> 1) & 1);
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
@@ -345,7 +428,7 @@ cudaError_t tc_launch(int n, const void* x, const void* w, const float* bias, co
   if (e != cudaSuccess) return e;
   const int tiles_x = (n + TXo - 1) / TXo, tiles_y = (n + TYo - 1) / TYo, tiles_z = (n + TZo - 1) / TZo;
   const long long ntiles = static_cast<long long>(tiles_x) * tiles_y * tiles_z;
-  const int grid = static_cast<int>(std::min<long long>(ntiles, 2LL * sm_count()));
+  const int grid = static_cast<int>(std::min<long long>(ntiles, sm_count()));
   kern<<<grid, kThreads, S::kBytes, s>>>(n, tiles_x, tiles_y, static_cast<int>(ntiles),
                                          static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(w),
                                          bias, static_cast<const __nv_bfloat16*>(res),
