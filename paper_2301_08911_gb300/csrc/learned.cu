@@ -4,9 +4,9 @@
 //
 // The layers' forward and backward-data convolutions run on the tcgen05 tensor cores
 // (conv_tc.cu). This file holds the rest of the network's arithmetic: the weight gradient,
-// which contracts over voxels (per tap and voxel chunk a CTA stages the transposed
-// operands and accumulates a 32 x c_in block with BF16 mma.sync, FP32 accumulation; a
-// second kernel sums the chunks in a fixed order, so it is deterministic), the input
+// which contracts over voxels (BF16 mma.sync, FP32 accumulation, all 27 taps of a chunk of
+// voxels in one cluster; a second kernel sums the chunks in a fixed order, so it is
+// deterministic), the input
 // features, pooling, the MSE loss and its gradient, Adam, and the BF16 weight packing.
 #include <cuda_bf16.h>
 
@@ -26,9 +26,6 @@ constexpr int kC = HOMO_NN_CHANNELS;    // output channels of every layer (32)
 constexpr int kTaps = 27;
 
 
-__device__ __forceinline__ uint32_t ld32(const __nv_bfloat16* p) {
-  return *reinterpret_cast<const uint32_t*>(p);
-}
 __device__ __forceinline__ uint32_t pack2(float a, float b) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);   // a -> low half
   uint32_t u;
@@ -50,122 +47,285 @@ __device__ __forceinline__ int wrapc(int a, int n) {
   return a < 0 ? a + n : a;
 }
 
-constexpr int kWgTile = 128;              // voxels per staged weight-gradient tile
-constexpr int kWgS = kWgTile + 8;         // bf16 per staged channel row (68 words: 4 mod 32)
+// ---- weight gradient: dw[t][o][i] = sum_v dy[v, o] x[wrap(v + d_t), i], a contraction over voxels
+// with M = N = 32 per tap, too small for a 128-row tcgen05 tile: mma.sync m16n8k16 on 16
+// consecutive voxels per step. Training follows the last bits of the gradients (Adam divides
+// by their size and the weights are rounded to BF16), so the sums keep one fixed order: a
+// chunk's tiles of 128 voxels in order, the four 32-voxel quarters of the tiles as four FP32
+// chains, ((q0 + q1) + q2) + q3, then the chunks.
+// A cluster of four CTAs takes a chunk, CTA q its quarters, all 27 taps at once: warp w < 9
+// owns the taps (dx = -1, 0, 1) of (dy, dz) = (w % 3, w / 3) - 1 in 96 accumulators, one pair of
+// dy fragments feeding 24 MMAs. A quarter's dy and, per (dy, dz), its 32 shifted voxels plus
+// the at most 4 row neighbours outside the run are staged by 16-byte asynchronous copies,
+// kWgStages quarters deep, voxel-major as they lie in memory; ldmatrix.trans turns 8 x 8
+// blocks on the way to the registers, its per-lane row addresses resolving the periodic x
+// neighbours. 16-byte chunk c of slot v sits at chunk c ^ (v / 2 % 4) of its row, so that
+// 8 consecutive slots' chunks fall on distinct banks. The quarters' chains meet through
+// distributed shared memory. Warp 9 of CTA 0 sums dy for the bias, voxel by voxel.
+// 64^3, 32 channels: 225 -> 172 us (a CTA per tap and chunk staged dy and x again for every tap,
+// transposing through 2-byte shared-memory stores: LSU 86 % busy).
+constexpr int kWgTile = 128, kWgRun = 32, kWgCtas = 4;     // voxels of a tile, of a quarter; quarters
+constexpr int kWgSlots = kWgRun + 4;
+constexpr int kWgThreads = 10 * 32, kWgCopy = 9 * 32;      // nine MMA warps copy, one sums the bias
+constexpr int kWgStages = 4;
 
-// Partial weight gradient of one tap over one chunk of voxel tiles:
-// part[(chunk * 27 + tap)][o][i] = sum_v dy[v, o] x[wrap(v + d_tap), i]; the centre-tap
-// blocks also sum dy over the chunk for the bias gradient (partb[chunk][o]).
 template <int CIN>
-__global__ void __launch_bounds__(128)
-    k_wgrad(int n, int ntiles, int tiles_per_chunk, const __nv_bfloat16* __restrict__ x,
-            const __nv_bfloat16* __restrict__ dy, float* __restrict__ part, float* __restrict__ partb) {
-  __shared__ __align__(16) __nv_bfloat16 dys[kC * kWgS];
-  __shared__ __align__(16) __nv_bfloat16 xs[CIN * kWgS];
-  __shared__ float red[4][kC * CIN];
-  const int tap = blockIdx.y, chunk = blockIdx.x;
-  const int ddx = tap % 3 - 1, ddy = (tap / 3) % 3 - 1, ddz = tap / 9 - 1;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int g = lane >> 2, t4 = lane & 3;
-  const size_t N = static_cast<size_t>(n) * n * n;
-  constexpr int NT = CIN / 8;
+struct WgSmem {
+  static constexpr int kDy = kWgRun * kC * 2, kX = 9 * kWgSlots * CIN * 2;
+  static constexpr int kStage = kDy + kX;
+  static constexpr int kSum = kTaps * kC * CIN * 4;        // the chain sums, in place of the stages
+  static constexpr int kMain = kWgStages * kStage > kSum ? kWgStages * kStage : kSum;
+  static constexpr int kBytes = kMain + 2 * kWgTile * kC * 2;   // and the bias warp's two dy tiles
+};
 
-  float acc[2][NT][4];
-#pragma unroll
-  for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc[mt][nt][q] = 0.f;
-  float bsum = 0.f;
-
-  const int t_begin = chunk * tiles_per_chunk;
-  const int t_end = min(ntiles, t_begin + tiles_per_chunk);
-  for (int tile = t_begin; tile < t_end; ++tile) {
-    __syncthreads();
-    const size_t v = static_cast<size_t>(tile) * kWgTile + tid;   // this thread's voxel
-    if (v < N) {
-      const uint4* src = reinterpret_cast<const uint4*>(dy + v * kC);
-#pragma unroll
-      for (int q = 0; q < kC / 8; ++q) {
-        const uint4 u = src[q];
-        const __nv_bfloat16* e = reinterpret_cast<const __nv_bfloat16*>(&u);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) dys[(8 * q + j) * kWgS + tid] = e[j];
-      }
-      const int gx = static_cast<int>(v % n), gy = static_cast<int>((v / n) % n),
-                gz = static_cast<int>(v / (static_cast<size_t>(n) * n));
-      const size_t vs = static_cast<size_t>(wrapc(gx + ddx, n)) +
-                        static_cast<size_t>(n) * (wrapc(gy + ddy, n) + static_cast<size_t>(n) * wrapc(gz + ddz, n));
-      const uint4* xsrc = reinterpret_cast<const uint4*>(x + vs * CIN);
-#pragma unroll
-      for (int q = 0; q < CIN / 8; ++q) {
-        const uint4 u = xsrc[q];
-        const __nv_bfloat16* e = reinterpret_cast<const __nv_bfloat16*>(&u);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) xs[(8 * q + j) * kWgS + tid] = e[j];
-      }
-    } else {
-      const __nv_bfloat16 z = __float2bfloat16(0.f);
-      for (int c = 0; c < kC; ++c) dys[c * kWgS + tid] = z;
-      for (int c = 0; c < CIN; ++c) xs[c * kWgS + tid] = z;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int ks = 0; ks < 2; ++ks) {
-      const int kb = 32 * warp + 16 * ks;
-      uint32_t a[2][4];
-#pragma unroll
-      for (int mt = 0; mt < 2; ++mt) {
-        const __nv_bfloat16* r = dys + (16 * mt + g) * kWgS + kb + 2 * t4;
-        a[mt][0] = ld32(r);
-        a[mt][1] = ld32(r + 8 * kWgS);
-        a[mt][2] = ld32(r + 8);
-        a[mt][3] = ld32(r + 8 * kWgS + 8);
-      }
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        const __nv_bfloat16* r = xs + (8 * nt + g) * kWgS + kb + 2 * t4;
-        const uint32_t b0 = ld32(r), b1 = ld32(r + 8);
-        mma16816(acc[0][nt], a[0], b0, b1);
-        mma16816(acc[1][nt], a[1], b0, b1);
-      }
-    }
-    if (tap == 13 && tid < kC) {
-      for (int j = 0; j < kWgTile; ++j) bsum += __bfloat162float(dys[tid * kWgS + j]);
-    }
-  }
-#pragma unroll
-  for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-      const int o = 16 * mt + g, i = 8 * nt + 2 * t4;
-      red[warp][o * CIN + i] = acc[mt][nt][0];
-      red[warp][o * CIN + i + 1] = acc[mt][nt][1];
-      red[warp][(o + 8) * CIN + i] = acc[mt][nt][2];
-      red[warp][(o + 8) * CIN + i + 1] = acc[mt][nt][3];
-    }
-  __syncthreads();
-  float* dst = part + (static_cast<size_t>(chunk) * kTaps + tap) * (kC * CIN);
-  for (int e = tid; e < kC * CIN; e += 128) dst[e] = ((red[0][e] + red[1][e]) + red[2][e]) + red[3][e];
-  if (tap == 13 && tid < kC) partb[static_cast<size_t>(chunk) * kC + tid] = bsum;
+__device__ __forceinline__ uint32_t smem_u32(const void* p) {
+  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// dw[t][o][i] = sum over chunks (in order) of the partials; db[o] likewise.
-__global__ void k_wgrad_reduce(int chunks, int per, const float* __restrict__ part,
-                               const float* __restrict__ partb, float* __restrict__ dw, float* __restrict__ db) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < kTaps * per) {
-    const int tap = e / per, r = e - tap * per;
-    double s = 0.0;
-    for (int c = 0; c < chunks; ++c) s += part[(static_cast<size_t>(c) * kTaps + tap) * per + r];
-    dw[e] = static_cast<float>(s);
-  } else if (e < kTaps * per + kC) {
-    const int o = e - kTaps * per;
-    double s = 0.0;
-    for (int c = 0; c < chunks; ++c) s += partb[static_cast<size_t>(c) * kC + o];
-    db[o] = static_cast<float>(s);
+// 16 bytes, or zeros where live is false (src is then any valid address)
+__device__ __forceinline__ void cp_async16z(uint32_t dst, const void* src, bool live) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(live ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int kLeft>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(kLeft) : "memory");
+}
+
+__device__ __forceinline__ void ldmatrix_x4_t(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+
+// Byte offset of 16-byte chunk c of slot v (kCh chunks per slot: 4, or 2 for 16 channels, where
+// the swizzle period doubles).
+template <int kCh>
+__device__ __forceinline__ uint32_t wg_at(int v, int c) {
+  return static_cast<uint32_t>((v * kCh + (c ^ (kCh == 4 ? (v >> 1) & 3 : (v >> 2) & 1))) * 16);
+}
+
+// Stage the run of voxels u0 .. u0 + 31 (those below N): dy, and for each (dy, dz) the shifted
+// voxels in slots 0..31 and the x neighbours that lie in a partly covered row: slot 32 left of
+// the first voxel, 33 x = 0 of its row, 34 x = n - 1 of the last voxel's row, 35 right of it.
+template <int CIN>
+__device__ __forceinline__ void wg_stage(size_t u0, size_t N, int n, const __nv_bfloat16* __restrict__ x,
+                                         const __nv_bfloat16* __restrict__ dy, uint32_t s_dy, uint32_t s_x) {
+  constexpr int kCh = CIN / 8, kItems = 9 * kWgSlots * kCh;
+  const int count = u0 >= N ? 0 : static_cast<int>(N - u0 < kWgRun ? N - u0 : kWgRun);
+  if (count > 0) {
+    if (threadIdx.x < kWgRun * (kC / 8)) {
+      const int c = threadIdx.x % (kC / 8), i = threadIdx.x / (kC / 8);
+      cp_async16z(s_dy + wg_at<kC / 8>(i, c), dy + (u0 + (i < count ? i : 0)) * kC + c * 8, i < count);
+    }
+#pragma unroll
+    for (int k = 0; k < (kItems + kWgCopy - 1) / kWgCopy; ++k) {
+      const int t = threadIdx.x + k * kWgCopy;
+      if (t >= kItems) break;
+      const int c = t % kCh, slot = (t / kCh) % kWgSlots, combo = t / (kCh * kWgSlots);
+      const int i = slot < kWgRun ? slot : (slot < kWgRun + 2 ? 0 : count - 1);   // the voxel whose row it is in
+      int gx, gy, gz;
+      decode3(static_cast<unsigned>(u0) + (i < count ? i : 0), static_cast<unsigned>(n), gx, gy, gz);
+      if (slot == kWgRun) gx = gx == 0 ? n - 1 : gx - 1;
+      if (slot == kWgRun + 1) gx = 0;
+      if (slot == kWgRun + 2) gx = n - 1;
+      if (slot == kWgRun + 3) gx = gx == n - 1 ? 0 : gx + 1;
+      gy += combo % 3 - 1;
+      gz += combo / 3 - 1;
+      gy = gy < 0 ? n - 1 : (gy == n ? 0 : gy);
+      gz = gz < 0 ? n - 1 : (gz == n ? 0 : gz);
+      const size_t v = static_cast<size_t>(gx) + static_cast<size_t>(n) * (gy + static_cast<size_t>(n) * gz);
+      cp_async16z(s_x + combo * (kWgSlots * CIN * 2) + wg_at<kCh>(slot, c), x + v * CIN + c * 8, i < count);
+    }
   }
+  cp_async_commit();
+}
+
+// Slot of the x neighbour (dx = -1, 0, 1) of voxel i of a run whose x coordinate is xi.
+__device__ __forceinline__ int wg_slot(int i, int xi, int dx, int n) {
+  if (dx < 0) {
+    if (xi > 0) return i > 0 ? i - 1 : kWgRun;
+    return i + n - 1 < kWgRun ? i + n - 1 : kWgRun + 2;
+  }
+  if (dx > 0) {
+    if (xi < n - 1) return i < kWgRun - 1 ? i + 1 : kWgRun + 3;
+    return i >= n - 1 ? i - (n - 1) : kWgRun + 1;
+  }
+  return i;
+}
+
+__device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+
+// Partial gradients of chunk blockIdx.x / 4: part[(chunk * 27 + tap)][o][i], partb[chunk][o].
+template <int CIN>
+__global__ void __launch_bounds__(kWgThreads, 1)
+    k_wgrad(int n, int ntiles, int tiles_per_chunk, const __nv_bfloat16* __restrict__ x,
+            const __nv_bfloat16* __restrict__ dy, float* __restrict__ part, float* __restrict__ partb) {
+  using S = WgSmem<CIN>;
+  constexpr int kCh = CIN / 8, NT = CIN / 8;
+  extern __shared__ __align__(128) unsigned char wsm[];
+  const uint32_t base = smem_u32(wsm);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int chunk = blockIdx.x / kWgCtas, q = blockIdx.x % kWgCtas;
+  const size_t N = static_cast<size_t>(n) * n * n;
+  const int t0 = chunk * tiles_per_chunk, t1 = min(ntiles, t0 + tiles_per_chunk);
+
+  if (warp < 9) {
+    // ldmatrix lanes: lanes 0-7, 8-15, 16-23, 24-31 give the row addresses of matrices 0..3.
+    // A (dy^T): matrices (v 0-7, o chunk 0), (v 0-7, chunk 1), (v 8-15, chunk 0), (v 8-15, chunk 1)
+    const int av = (lane & 7) + ((lane >> 4) << 3), ac = (lane >> 3) & 1;
+    // B (x): (v 0-7, i chunk 0), (v 8-15, chunk 0), (v 0-7, chunk 1), (v 8-15, chunk 1)
+    const int bv = (lane & 7) + (((lane >> 3) & 1) << 3), bc = lane >> 4;
+    float acc[3][2][NT][4];
+#pragma unroll
+    for (int t = 0; t < 3; ++t)
+#pragma unroll
+      for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) acc[t][mt][nt][e] = 0.f;
+    auto run_of = [&](int tile) { return static_cast<size_t>(tile) * kWgTile + kWgRun * q; };
+    auto stage_at = [&](int k) { return base + static_cast<uint32_t>(k % kWgStages) * S::kStage; };
+#pragma unroll
+    for (int k = 0; k < kWgStages - 1; ++k) {
+      if (t0 + k < t1) wg_stage<CIN>(run_of(t0 + k), N, n, x, dy, stage_at(k), stage_at(k) + S::kDy);
+      else cp_async_commit();
+    }
+    for (int tile = t0; tile < t1; ++tile) {
+      const int k = tile - t0;
+      cp_async_wait<kWgStages - 2>();
+      asm volatile("bar.sync 1, %0;\n" ::"n"(kWgCopy) : "memory");   // this stage is complete, the one before free
+      if (tile + kWgStages - 1 < t1)
+        wg_stage<CIN>(run_of(tile + kWgStages - 1), N, n, x, dy, stage_at(k + kWgStages - 1),
+                      stage_at(k + kWgStages - 1) + S::kDy);
+      else
+        cp_async_commit();
+      const size_t u0 = run_of(tile);
+      const uint32_t s_dy = stage_at(k), s_x = s_dy + S::kDy + warp * (kWgSlots * CIN * 2);
+#pragma unroll
+      for (int ks = 0; ks < 2; ++ks) {
+        if (u0 + 16 * ks >= N) continue;   // past the grid: the products are zero
+        uint32_t a[2][4];
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) ldmatrix_x4_t(a[mt], s_dy + wg_at<kC / 8>(16 * ks + av, 2 * mt + ac));
+        const int i = 16 * ks + bv;
+        const int xi = static_cast<int>((static_cast<unsigned>(u0) + i) % static_cast<unsigned>(n));
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {
+          const int slot = u0 + i < N ? wg_slot(i, xi, t - 1, n) : i;
+#pragma unroll
+          for (int h = 0; h < NT / 2; ++h) {
+            uint32_t b[4];
+            ldmatrix_x4_t(b, s_x + wg_at<kCh>(slot, 2 * h + bc));
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) {
+              mma16816(acc[t][mt][2 * h], a[mt], b[0], b[1]);
+              mma16816(acc[t][mt][2 * h + 1], a[mt], b[2], b[3]);
+            }
+          }
+        }
+      }
+    }
+    cp_async_wait<0>();
+    asm volatile("bar.sync 1, %0;\n" ::"n"(kWgCopy) : "memory");   // the stages give way to the chain sums
+    float* sum = reinterpret_cast<float*>(wsm);
+    const int g = lane >> 2, t4 = lane & 3;
+#pragma unroll
+    for (int t = 0; t < 3; ++t)
+#pragma unroll
+      for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+          float* d = sum + (3 * warp + t) * (kC * CIN) + (16 * mt + g) * CIN + 8 * nt + 2 * t4;
+          d[0] = acc[t][mt][nt][0];
+          d[1] = acc[t][mt][nt][1];
+          d[8 * CIN] = acc[t][mt][nt][2];
+          d[8 * CIN + 1] = acc[t][mt][nt][3];
+        }
+  } else if (q == 0) {
+    // bias: lane = output channel, every voxel of the chunk in order; dy's tiles one ahead
+    const uint32_t s_b = base + S::kMain;
+    auto fetch = [&](int tile) {
+      if (tile < t1) {
+#pragma unroll
+        for (int k = 0; k < kWgTile * kC * 2 / 16 / 32; ++k) {
+          const int t = lane + 32 * k, v = t / (kC / 8);
+          const size_t u = static_cast<size_t>(tile) * kWgTile + v;
+          cp_async16z(s_b + (tile & 1) * (kWgTile * kC * 2) + t * 16, dy + (u < N ? u : 0) * kC + t % (kC / 8) * 8, u < N);
+        }
+      }
+      cp_async_commit();
+    };
+    float bsum = 0.f;
+    fetch(t0);
+    for (int tile = t0; tile < t1; ++tile) {
+      fetch(tile + 1);
+      cp_async_wait<1>();
+      __syncwarp();
+      const __nv_bfloat16* d = reinterpret_cast<const __nv_bfloat16*>(wsm + S::kMain + (tile & 1) * (kWgTile * kC * 2)) + lane;
+#pragma unroll 16
+      for (int j = 0; j < kWgTile; ++j) bsum += __bfloat162float(d[j * kC]);
+      __syncwarp();
+    }
+    cp_async_wait<0>();
+    partb[static_cast<size_t>(chunk) * kC + lane] = bsum;
+  }
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+  // each CTA adds a quarter of the values over the four chains
+  constexpr int kPer = kTaps * kC * CIN / kWgCtas;
+  uint32_t peer[kWgCtas];
+#pragma unroll
+  for (int r = 0; r < kWgCtas; ++r)
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer[r]) : "r"(base), "r"(r));
+  float* dst = part + static_cast<size_t>(chunk) * kTaps * kC * CIN;
+#pragma unroll 4
+  for (int e = q * kPer + threadIdx.x; e < (q + 1) * kPer; e += kWgThreads) {
+    float v[kWgCtas];
+#pragma unroll
+    for (int r = 0; r < kWgCtas; ++r) v[r] = ld_cluster_f32(peer[r] + 4u * e);
+    dst[e] = __fadd_rn(__fadd_rn(__fadd_rn(v[0], v[1]), v[2]), v[3]);
+  }
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");   // peers read this CTA's sums
+}
+
+// dw[t][o][i] = sum over chunks of the partials, db[o] likewise: four threads per value sum a
+// quarter each in order as FP32 pairs (TwoSum: as exact as FP64 here, whose pipe the
+// one-thread FP64 sum left 71 % busy; 38 -> 12 us for 27,680 values), then the quarters.
+__global__ void __launch_bounds__(256) k_wgrad_reduce(int chunks, int per, const float* __restrict__ part,
+                                                      const float* __restrict__ partb, float* __restrict__ dw,
+                                                      float* __restrict__ db) {
+  __shared__ float sh[4][64], sl[4][64];
+  const int q = threadIdx.x >> 6, k = threadIdx.x & 63;
+  const int e = blockIdx.x * 64 + k;
+  const int nw = kTaps * per;
+  const int c0 = chunks * q / 4, c1 = chunks * (q + 1) / 4;
+  float hi = 0.f, lo = 0.f;
+  auto add = [&](float v) {
+    const float s = __fadd_rn(hi, v), bb = __fadd_rn(s, -hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -bb)), __fadd_rn(v, -bb)));
+    hi = s;
+  };
+  if (e < nw + kC) {
+    const float* src = e < nw ? part + e : partb + (e - nw);
+    const size_t step = e < nw ? nw : kC;
+#pragma unroll 8
+    for (int c = c0; c < c1; ++c) add(__ldg(src + c * step));
+  }
+  sh[q][k] = hi;
+  sl[q][k] = lo;
+  __syncthreads();
+  if (q != 0 || e >= nw + kC) return;
+  for (int t = 1; t < 4; ++t) {
+    add(sh[t][k]);
+    lo = __fadd_rn(lo, sl[t][k]);
+  }
+  (e < nw ? dw[e] : db[e - nw]) = __fadd_rn(hi, lo);
 }
 
 // x[v] = (rho, rho^2, rho^3, 0 ... 0) in BF16, 16 channels.
@@ -306,24 +466,41 @@ cudaError_t nn_conv3d(int n, int cin, const void* x, const void* w, const float*
   return conv3d_tc(n, cin, epi, x, w, bias, res, mask, out, outf, scale, s);
 }
 
+namespace {
+template <int CIN>
+cudaError_t wgrad_launch(const WgradPlan& p, int n, const void* x, const void* dy, float* part, float* partb,
+                         cudaStream_t s) {
+  constexpr int shm = WgSmem<CIN>::kBytes;
+  const cudaError_t e = cudaFuncSetAttribute(k_wgrad<CIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, shm);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(p.chunks * kWgCtas);
+  cfg.blockDim = dim3(kWgThreads);
+  cfg.dynamicSmemBytes = shm;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kWgCtas;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_wgrad<CIN>, n, p.ntiles, p.tiles_per_chunk, static_cast<const __nv_bfloat16*>(x),
+                            static_cast<const __nv_bfloat16*>(dy), part, partb);
+}
+}  // namespace
+
 cudaError_t nn_wgrad(int n, int cin, const void* x, const void* dy, float* dw, float* db, float* scratch,
                      cudaStream_t s) {
   const WgradPlan p = wgrad_plan(n);
   float* part = scratch;
   float* partb = scratch + static_cast<size_t>(p.chunks) * kTaps * kC * cin;
-  const dim3 grid(p.chunks, kTaps);
-  if (cin == 16)
-    k_wgrad<16><<<grid, 128, 0, s>>>(n, p.ntiles, p.tiles_per_chunk, static_cast<const __nv_bfloat16*>(x),
-                                     static_cast<const __nv_bfloat16*>(dy), part, partb);
-  else if (cin == 32)
-    k_wgrad<32><<<grid, 128, 0, s>>>(n, p.ntiles, p.tiles_per_chunk, static_cast<const __nv_bfloat16*>(x),
-                                     static_cast<const __nv_bfloat16*>(dy), part, partb);
-  else
-    return cudaErrorInvalidValue;
-  cudaError_t e = cudaGetLastError();
+  if (cin != 16 && cin != 32) return cudaErrorInvalidValue;
+  const cudaError_t e = cin == 16 ? wgrad_launch<16>(p, n, x, dy, part, partb, s)
+                                  : wgrad_launch<32>(p, n, x, dy, part, partb, s);
   if (e != cudaSuccess) return e;
   const int total = kTaps * kC * cin + kC;
-  k_wgrad_reduce<<<(total + 255) / 256, 256, 0, s>>>(p.chunks, kC * cin, part, partb, dw, db);
+  k_wgrad_reduce<<<(total + 63) / 64, 256, 0, s>>>(p.chunks, kC * cin, part, partb, dw, db);
   return cudaGetLastError();
 }
 
