@@ -400,7 +400,7 @@ __device__ __forceinline__ void pair_add(float& hi, float& lo, float v) {
 // Block sums of NV FP32 pairs into part[blockIdx.x * NV + k] (FP64 across the warps).
 template <int NV>
 __device__ __forceinline__ void pair_block_sum(float (&hi)[NV], float (&lo)[NV], double* part) {
-  __shared__ double sh[kOcBlock / 32][NV];
+  __shared__ float sh[kOcBlock / 32][NV], sl[kOcBlock / 32][NV];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
@@ -410,13 +410,17 @@ __device__ __forceinline__ void pair_block_sum(float (&hi)[NV], float (&lo)[NV],
       pair_add(hi[k], lo[k], h);
       lo[k] = __fadd_rn(lo[k], l);
     }
-    if (lane == 0) sh[wid][k] = static_cast<double>(hi[k]) + static_cast<double>(lo[k]);
+    if (lane == 0) {
+      sh[wid][k] = hi[k];
+      sl[wid][k] = lo[k];
+    }
   }
   __syncthreads();
   if (threadIdx.x < NV) {
     double s = 0.0;
 #pragma unroll
-    for (int w = 0; w < kOcBlock / 32; ++w) s += sh[w][threadIdx.x];
+    for (int w = 0; w < kOcBlock / 32; ++w)
+      s += static_cast<double>(sh[w][threadIdx.x]) + static_cast<double>(sl[w][threadIdx.x]);
     part[static_cast<size_t>(blockIdx.x) * NV + threadIdx.x] = s;
   }
 }
@@ -553,10 +557,13 @@ __global__ void __launch_bounds__(kOcBlock) k_oc_pass(const float* __restrict__ 
                                                       size_t stride, float move, float rmin, double V,
                                                       double* oc, double* __restrict__ part) {
   if (oc[OC_MODE] != 0) return;
+  __shared__ float cand_s[kOcCand];   // rounded to FP32 by one warp (a conversion is FP64-pipe work)
+  if (threadIdx.x < kOcCand) cand_s[threadIdx.x] = static_cast<float>(oc[OC_CAND + threadIdx.x]);
+  __syncthreads();
   float cand[kOcCand], hi[kOcCand], lo[kOcCand];
 #pragma unroll
   for (int k = 0; k < kOcCand; ++k) {
-    cand[k] = static_cast<float>(oc[OC_CAND + k]);
+    cand[k] = cand_s[k];
     hi[k] = lo[k] = 0.f;
   }
   const size_t runs = (N + 8 * stride - 1) / (8 * stride);
