@@ -2,28 +2,29 @@
 // (tcgen05.mma, accumulators in tensor memory). Implicit GEMM: M = 128 voxels, N = 32
 // output channels, K = 27 taps x c_in, BF16 operands, FP32 accumulation.
 //
-// A persistent CTA keeps the layer's weights in shared memory and walks tiles of 30 x 4 x 2
-// output voxels. Each tile's periodic halo box (32 x 6 x 4 voxels, all input channels) is
-// staged with 16-byte asynchronous copies into a K-major, non-swizzled operand layout whose
-// rows are 16 bytes apart along the box's (z, y, x) order: channel chunk c (8 channels) of
-// box row r sits at plane c, row r. For a tap with offset d, the 128 rows of the A operand
-// are then the output rows shifted by the constant row offset of d, so every tap's operand
-// is the same staged box seen through a shifted descriptor, with no per-tap copy. Output
-// rows 0 and 31 of each 32-row run are halo positions: computed and discarded (30 of every
-// 32 rows are outputs).
-//
-// Nine warps in three roles, handing tiles on through mbarriers, so that the copies of the
+// A persistent CTA keeps the layer's weights in shared memory and walks tiles of TX x TY x TZ
+// output voxels. Each tile's periodic halo box ((TX + 2) x (TY + 2) x (TZ + 2) voxels, all input
+// channels) is staged with 16-byte asynchronous copies into a K-major, non-swizzled operand
+// layout whose rows are 16 bytes apart along the box's (z, y, x) order: channel chunk c (8
+// channels) of box row r sits at plane c, row r. The outputs of a z-plane are then consecutive
+// box rows but for the two halo rows between lines, so blocks of 128 rows from the first
+// output on are the M of an MMA, and for a tap the A operand is the same staged box seen
+// through a descriptor shifted by the tap's constant row offset: no per-tap copy. Rows on
+// halo positions are computed and discarded.
+// Thirteen warps in three roles, handing tiles on through mbarriers, so that the copies of the
 // next tiles, the MMAs of one and the epilogue of the one before run at the same time:
-//   warps 4..7  copy boxes into a ring of kStages buffers;
-//   warp 8      issues (one elected lane) the tile's 27 x c_in/16 MMAs per output plane into one of
-//               two pairs of 32-column TMEM accumulators and commits them to the barriers
-//               that free the box and publish the accumulators;
-//   warps 0..3  read their 32 TMEM lanes (one voxel per thread, 32 channels), free the
-//               accumulators and apply the epilogue: bias, residual, ReLU or a backward ReLU
+//   warps 8..11 copy boxes into a ring of buffers;
+//   warp 12     issues (one elected lane) the 27 x c_in/16 MMAs of each of the tile's row blocks
+//               into one of two sets of 32-column TMEM accumulators and commits them to the
+//               barriers that free the box and publish the accumulators;
+//   warps 0..7  (four per row block) read their 32 TMEM lanes (one voxel per thread, 32
+//               channels), free the accumulators and apply the epilogue: bias, residual, ReLU or a backward ReLU
 //               mask, BF16 voxel-major output or scaled FP32 displacement planes.
 // Every wait is bounded. Bound: an MMA of 128 x 32 x 16 reads 5 KB of operands for 16 cycles
-// of math, so about 40 cycles of shared-memory bandwidth each. 64^3, 32 -> 32 channels: 70 -> 39 us
-// (four warps did all three in turn, two CTAs per SM: tensor pipe 14 % busy).
+// of math; measured 68 cycles each, back to back (two thirds of the time on operands at 64 B a
+// clock), so what counts is the share of rows that are outputs. 64^3, 32 -> 32 channels:
+// 70 -> 39 us with 30 x 4 x 2 tiles (four warps did all three in turn before, two CTAs per
+// SM: tensor pipe 14 % busy), 37 us with 32 x 11 x 1 (most of the rest a fixed 8 us of prologue and tail).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -37,28 +38,37 @@ namespace {
 
 constexpr int kC = HOMO_NN_CHANNELS;     // 32 output channels
 constexpr int kTaps = 27;
-constexpr int TXo = 30, TYo = 4, TZo = 2;                 // output voxels per tile
-constexpr int BXr = TXo + 2, BYr = TYo + 2, BZr = TZo + 2; // box (32 x 6 x 4)
-constexpr int kBoxRows = BXr * BYr * BZr;                  // 768
-constexpr int kRowPad = 1;                                 // row 0: guard below the box
-constexpr int kRows = 776;                                 // >= kRowPad + kBoxRows + 1, multiple of 8
-constexpr int kPlaneBytes = kRows * 16;                    // one 8-channel chunk of every row
-constexpr int kThreads = 9 * 32;                           // epilogue, copy and MMA warps
-constexpr int kRole = 128;                                 // threads of the epilogue and of the copy role
-constexpr int kStages = 3;                                 // boxes in flight
-constexpr int kTmemCols = 128;                             // two pairs of 128 x 32 FP32 accumulators
+constexpr int kThreads = 13 * 32;                          // 8 epilogue, 4 copy and one MMA warp
+constexpr int kEpi = 256, kRole = 128;                     // threads of the epilogue and of the copy role
 constexpr long long kWaitLimit = 1LL << 18;                // bounded mbarrier polls (~1 s on a GB300)
 
-static_assert(kRowPad + kBoxRows + 1 <= kRows, "guard rows");
-static_assert(kRole == 4 * 32 && TYo == 4, "epilogue warp w owns output row y = w of each plane");
+// A tile shape and its box, row blocks and shared memory for CIN input channels.
+template <int X, int Y, int Z, int kStagesOf>
+struct TcTile {
+  static constexpr int TX = X, TY = Y, TZ = Z, kStages = kStagesOf;   // kStages: boxes in flight
+  static constexpr int BX = TX + 2, BY = TY + 2, BZ = TZ + 2;
+  static constexpr int kBoxRows = BX * BY * BZ;
+  static constexpr int kBlocks = (TY * BX - 2 + 127) / 128;   // row blocks per z-plane (y rows are BX apart)
+  static constexpr int kUnits = TZ * kBlocks;                 // accumulators of a tile
+  // rows the last block of the last plane reads for tap (1, 1, 1), a multiple of 8
+  static constexpr int kLast = ((TZ + 1) * BY + 2) * BX + 2 + 128 * kBlocks;
+  static constexpr int kRows = ((kLast > kBoxRows ? kLast : kBoxRows) + 7) / 8 * 8;
+  static constexpr int kPlaneBytes = kRows * 16;              // one 8-channel chunk of every row
+  static constexpr int kTmemUse = 2 * kUnits * kC;
+  static constexpr int kTmemCols = kTmemUse <= 128 ? 128 : 256;
+  static constexpr int kBarriers = 2 * kStages + 4;
+  static_assert(kTmemUse <= kTmemCols, "two sets of accumulators");
+};
+typedef TcTile<30, 4, 2, 3> TileA;     // a line of 32 rows, 126 of 128 rows per block, 3 of 4 lines' halo
+typedef TcTile<32, 11, 1, 2> TileB;    // 352 outputs of 3 x 128 rows
 
-template <int CIN>
+template <int CIN, typename TL>
 struct TcShape {
   static constexpr int kChunks = CIN / 8;
-  static constexpr int kBoxBytes = kChunks * kPlaneBytes;
+  static constexpr int kBoxBytes = kChunks * TL::kPlaneBytes;
   static constexpr int kWBytes = kTaps * kChunks * kC * 16;
-  static constexpr int kBarriers = 2 * kStages + 4;
-  static constexpr int kBytes = kStages * kBoxBytes + kWBytes + 8 * kBarriers + 16;   // + mbarriers, TMEM address
+  static constexpr int kBytes = TL::kStages * kBoxBytes + kWBytes + 8 * TL::kBarriers + 16;   // + mbarriers, TMEM address
+  static_assert(kBytes <= 227 * 1024, "shared memory of a CTA");
 };
 
 struct TcScale {
@@ -214,18 +224,19 @@ __device__ __forceinline__ void conv_epilogue(const float (&acc)[32], const floa
   }
 }
 
-template <int CIN, int EPI>
+template <int CIN, int EPI, typename TL>
 __global__ void __launch_bounds__(kThreads, 1)
     k_conv3d_tc(int n, int tiles_x, int tiles_y, int ntiles, const __nv_bfloat16* __restrict__ x,
                 const __nv_bfloat16* __restrict__ w, const float* __restrict__ bias,
                 const __nv_bfloat16* __restrict__ res, const __nv_bfloat16* __restrict__ mask,
                 __nv_bfloat16* __restrict__ out, float* __restrict__ outf, TcScale sc) {
-  using S = TcShape<CIN>;
-  constexpr int kCh = S::kChunks;
+  using S = TcShape<CIN, TL>;
+  constexpr int kCh = S::kChunks, kStages = TL::kStages, kRows = TL::kRows, kBoxRows = TL::kBoxRows;
+  constexpr int kPlaneBytes = TL::kPlaneBytes, BX = TL::BX, BY = TL::BY;
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned char* wsm = smem + kStages * S::kBoxBytes;     // [tap][chunk][o][16 B]
   uint64_t* mbar = reinterpret_cast<uint64_t*>(wsm + S::kWBytes);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mbar + S::kBarriers);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mbar + TL::kBarriers);
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const size_t N = static_cast<size_t>(n) * n * n;
   const uint32_t box_s = smem_u32(smem), w_s = smem_u32(wsm), bar_s = smem_u32(mbar);
@@ -242,9 +253,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   asm volatile("cp.async.commit_group;\n" ::: "memory");
   for (int c = tid; c < kStages * kCh * (kRows - kBoxRows); c += kThreads) {
-    const int p = c / (kRows - kBoxRows), r = c % (kRows - kBoxRows);   // plane p of all stages
-    const int row = r < kRowPad ? r : kRowPad + kBoxRows + (r - kRowPad);
-    *reinterpret_cast<uint4*>(smem + p * kPlaneBytes + row * 16) = make_uint4(0u, 0u, 0u, 0u);
+    const int p = c / (kRows - kBoxRows), r = kBoxRows + c % (kRows - kBoxRows);   // plane p of all stages
+    *reinterpret_cast<uint4*>(smem + p * kPlaneBytes + r * 16) = make_uint4(0u, 0u, 0u, 0u);
   }
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -253,13 +263,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int t = 0; t < 2; ++t) {
       mbar_init(tfull(t), 1);
-      mbar_init(tempty(t), kRole);
+      mbar_init(tempty(t), kEpi);
     }
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)),
-                 "r"(kTmemCols)
+                 "r"(TL::kTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
   }
@@ -270,41 +280,35 @@ __global__ void __launch_bounds__(kThreads, 1)
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   const uint32_t tmem = *tmem_slot;
 
-  if (warp >= 4 && warp < 8) {
-    // ---- copies: box row br = t + 128 k (k < 6) and all its chunks per thread
-    const int t = tid - kRole;
+  if (warp >= 8 && warp < 12) {
+    // ---- copies: box rows t, t + 128, ... and all their chunks per thread
+    const int t = tid - kEpi;
     int k = 0;
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++k) {
       const int st = k % kStages;
       if (!mbar_wait(empty(st), ((k / kStages) & 1) ^ 1)) break;   // a fresh barrier passes parity 1
       const int tx = tile % tiles_x, rest = tile / tiles_x;
-      const int x0 = tx * TXo, y0 = (rest % tiles_y) * TYo, z0 = (rest / tiles_y) * TZo;
-      const uint32_t dst = box_s + st * S::kBoxBytes + kRowPad * 16;
-#pragma unroll
-      for (int q = 0; q < kBoxRows / kRole; ++q) {
-        const int br = t + kRole * q;
-        const int bx = br % BXr, by = (br / BXr) % BYr, bz = br / (BXr * BYr);
-        // a box spans at most x0 - 1 .. x0 + 30: past one period only on grids below 32
+      const int x0 = tx * TL::TX, y0 = (rest % tiles_y) * TL::TY, z0 = (rest / tiles_y) * TL::TZ;
+      const uint32_t dst = box_s + st * S::kBoxBytes;
+#pragma unroll 4
+      for (int br = t; br < kBoxRows; br += kRole) {
+        const int bx = br % BX, by = (br / BX) % BY, bz = br / (BX * BY);
+        // a box starts at most one period in and spans at most BX: past it only on small grids
         const int gx = x0 - 1 + bx, gy = y0 - 1 + by, gz = z0 - 1 + bz;
-        const size_t gv = n >= BXr ? static_cast<size_t>(wrap1(gx, n)) +
-                                         static_cast<size_t>(n) * (wrap1(gy, n) + static_cast<size_t>(n) * wrap1(gz, n))
-                                   : static_cast<size_t>(wrapc(gx, n)) +
-                                         static_cast<size_t>(n) * (wrapc(gy, n) + static_cast<size_t>(n) * wrapc(gz, n));
+        const size_t gv = n >= BX ? static_cast<size_t>(wrap1(gx, n)) +
+                                        static_cast<size_t>(n) * (wrap1(gy, n) + static_cast<size_t>(n) * wrap1(gz, n))
+                                  : static_cast<size_t>(wrapc(gx, n)) +
+                                        static_cast<size_t>(n) * (wrapc(gy, n) + static_cast<size_t>(n) * wrapc(gz, n));
         const __nv_bfloat16* src = x + gv * CIN;
 #pragma unroll
         for (int ch = 0; ch < kCh; ++ch) cp_async16(dst + ch * kPlaneBytes + br * 16, src + ch * 8);
       }
       asm volatile("cp.async.commit_group;\n" ::: "memory");
-      if (k > 0) {   // the previous tile's copies have landed: hand it on
-        asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        mbar_arrive(full((k - 1) % kStages));
-      }
+      asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+      mbar_arrive(full(st));
     }
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-    if (k > 0) mbar_arrive(full((k - 1) % kStages));
-  } else if (warp == 8) {
+  } else if (warp == 12) {
     // ---- MMAs: the warp runs the loop, one elected lane issues
     uint32_t leader;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(leader));
@@ -316,13 +320,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!__all_sync(0xffffffffu, ok)) break;
       asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 #pragma unroll 1
-      for (int zo = 0; zo < TZo; ++zo) {
-        // box row of output (x = -1, y = 0, z = zo); descriptor addresses count 16-byte rows
-        const uint64_t az = a0 + static_cast<uint32_t>(st * (S::kBoxBytes / 16) + kRowPad + ((zo + 1) * BYr + 1) * BXr);
-        const uint32_t d = tmem + (ac * TZo + zo) * kC;
+      for (int unit = 0; unit < TL::kUnits; ++unit) {
+        const int zo = unit / TL::kBlocks, blk = unit - zo * TL::kBlocks;
+        // box row of output (0, 0, zo), then the unit's block; descriptor addresses count 16-byte rows
+        const uint64_t az = a0 + static_cast<uint32_t>(st * (S::kBoxBytes / 16) + ((zo + 1) * BY + 1) * BX + 1 + 128 * blk);
+        const uint32_t d = tmem + (ac * TL::kUnits + unit) * kC;
 #pragma unroll
         for (int tap = 0; tap < kTaps; ++tap) {
-          const int row = ((tap / 9 - 1) * BYr + (tap / 3) % 3 - 1) * BXr + tap % 3 - 1;
+          const int row = ((tap / 9 - 1) * BY + (tap / 3) % 3 - 1) * BX + tap % 3 - 1;
 #pragma unroll
           for (int ks = 0; ks < CIN / 16; ++ks)
             mma_bf16(d, az + static_cast<int64_t>(row + 2 * ks * kRows), b0 + (tap * kCh + 2 * ks) * kC,
@@ -334,9 +339,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else {
-    // ---- epilogue: this thread's TMEM lane (warp w reads lanes 32 w .. 32 w + 31) and output position
-    const uint32_t tlane = tmem + (static_cast<uint32_t>(32 * warp) << 16);
-    const bool xout = lane >= 1 && lane <= TXo;             // rows 0 and 31 of a run are halo
+    // ---- epilogue: warps 0..3 take the even units, 4..7 the odd ones; warp w can read TMEM lanes
+    // 32 (w % 4) .. + 31, the same rows of a unit's block
+    const int set = warp >> 2, row0 = 32 * (warp & 3) + lane;
+    const uint32_t tlane = tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16);
     float bo[kC], so[6];
 #pragma unroll
     for (int o = 0; o < kC; ++o) bo[o] = (EPI != HOMO_NN_MASK && bias) ? bias[o] : 0.f;
@@ -348,35 +354,36 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++k) {
       const int ac = k & 1;
       const int tx = tile % tiles_x, rest = tile / tiles_x;
-      const int gx = tx * TXo + lane - 1, gy = (rest % tiles_y) * TYo + warp, z0 = (rest / tiles_y) * TZo;
-      size_t v[TZo];
-      bool live[TZo];
-      uint4 rr[TZo][4], mm[TZo][4];
+      const int x0 = tx * TL::TX, y0 = (rest % tiles_y) * TL::TY, z0 = (rest / tiles_y) * TL::TZ;
+#pragma unroll 1
+      for (int unit = set; unit < TL::kUnits; unit += 2) {
+        const int zo = unit / TL::kBlocks, row = (unit - zo * TL::kBlocks) * 128 + row0;
+        const int ly = row / BX, lx = row - ly * BX;
+        const int gx = x0 + lx, gy = y0 + ly, gz = z0 + zo;
+        const bool live = lx < TL::TX && ly < TL::TY && gx < n && gy < n && gz < n;
+        const size_t v = live ? static_cast<size_t>(gx) + static_cast<size_t>(n) * (gy + static_cast<size_t>(n) * gz) : 0;
+        uint4 rr[4], mm[4];
 #pragma unroll
-      for (int zo = 0; zo < TZo; ++zo) {   // the residual and the mask do not wait for the MMAs
-        live[zo] = xout && gx < n && gy < n && z0 + zo < n;
-        v[zo] = live[zo] ? static_cast<size_t>(gx) + static_cast<size_t>(n) * (gy + static_cast<size_t>(n) * (z0 + zo)) : 0;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          rr[zo][q] = has_res && live[zo] ? reinterpret_cast<const uint4*>(res + v[zo] * kC)[q] : make_uint4(0u, 0u, 0u, 0u);
-          mm[zo][q] = EPI == HOMO_NN_MASK && live[zo] ? reinterpret_cast<const uint4*>(mask + v[zo] * kC)[q]
-                                                      : make_uint4(0u, 0u, 0u, 0u);
+        for (int q = 0; q < 4; ++q) {   // the residual and the mask do not wait for the MMAs
+          rr[q] = has_res && live ? reinterpret_cast<const uint4*>(res + v * kC)[q] : make_uint4(0u, 0u, 0u, 0u);
+          mm[q] = EPI == HOMO_NN_MASK && live ? reinterpret_cast<const uint4*>(mask + v * kC)[q] : make_uint4(0u, 0u, 0u, 0u);
         }
+        if (unit == set) {
+          ok = mbar_wait(tfull(ac), (k >> 1) & 1);
+          ok = __all_sync(0xffffffffu, ok);   // a warp takes one decision (its TMEM loads are collective)
+          if (!ok) break;
+          asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        }
+        float acc[32];
+        tmem_ld32(tlane + (ac * TL::kUnits + unit) * kC, acc);
+        if (unit + 2 >= TL::kUnits) {
+          asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+          mbar_arrive(tempty(ac));
+        }
+        if (live) conv_epilogue<EPI>(acc, bo, so, v, N, rr, mm, has_res, out, outf);
+        __syncwarp();
       }
-      ok = mbar_wait(tfull(ac), (k >> 1) & 1);
-      if (!__all_sync(0xffffffffu, ok)) {   // a warp takes one decision (its TMEM loads are collective)
-        ok = false;
-        break;
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-      float acc[TZo][32];
-#pragma unroll
-      for (int zo = 0; zo < TZo; ++zo) tmem_ld32(tlane + (ac * TZo + zo) * kC, acc[zo]);
-      asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-      mbar_arrive(tempty(ac));
-#pragma unroll
-      for (int zo = 0; zo < TZo; ++zo)
-        if (live[zo]) conv_epilogue<EPI>(acc[zo], bo, so, v[zo], N, rr[zo], mm[zo], has_res, out, outf);
+      if (!ok) break;
     }
     if (!ok && lane == 0) {
       // give up on this tile and the rest; MMAs still running get one more bounded wait before
@@ -389,7 +396,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(TL::kTmemCols) : "memory");
   }
 }
 
@@ -417,16 +424,14 @@ int sm_count() {
   return g_sms;
 }
 
-template <int CIN, int EPI>
-cudaError_t tc_launch(int n, const void* x, const void* w, const float* bias, const void* res, const void* mask,
-                      void* out, float* outf, const double* scale, cudaStream_t s) {
-  TcScale sc;
-  for (int k = 0; k < 6; ++k) sc.s[k] = scale ? static_cast<float>(scale[k]) : 1.f;
-  using S = TcShape<CIN>;
-  auto kern = k_conv3d_tc<CIN, EPI>;
+template <int CIN, int EPI, typename TL>
+cudaError_t tc_launch_tile(int n, const void* x, const void* w, const float* bias, const void* res, const void* mask,
+                           void* out, float* outf, const TcScale& sc, cudaStream_t s) {
+  using S = TcShape<CIN, TL>;
+  auto kern = k_conv3d_tc<CIN, EPI, TL>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kBytes);
   if (e != cudaSuccess) return e;
-  const int tiles_x = (n + TXo - 1) / TXo, tiles_y = (n + TYo - 1) / TYo, tiles_z = (n + TZo - 1) / TZo;
+  const int tiles_x = (n + TL::TX - 1) / TL::TX, tiles_y = (n + TL::TY - 1) / TL::TY, tiles_z = (n + TL::TZ - 1) / TL::TZ;
   const long long ntiles = static_cast<long long>(tiles_x) * tiles_y * tiles_z;
   const int grid = static_cast<int>(std::min<long long>(ntiles, sm_count()));
   kern<<<grid, kThreads, S::kBytes, s>>>(n, tiles_x, tiles_y, static_cast<int>(ntiles),
@@ -435,6 +440,24 @@ cudaError_t tc_launch(int n, const void* x, const void* w, const float* bias, co
                                          static_cast<const __nv_bfloat16*>(mask), static_cast<__nv_bfloat16*>(out),
                                          outf, sc);
   return cudaGetLastError();
+}
+
+// Row blocks the busiest SM computes with a shape: what the kernel's time is proportional to.
+template <typename TL>
+long long tile_rounds(int n) {
+  const long long tiles = static_cast<long long>((n + TL::TX - 1) / TL::TX) * ((n + TL::TY - 1) / TL::TY) *
+                          ((n + TL::TZ - 1) / TL::TZ);
+  return (tiles + sm_count() - 1) / sm_count() * TL::kUnits;
+}
+
+template <int CIN, int EPI>
+cudaError_t tc_launch(int n, const void* x, const void* w, const float* bias, const void* res, const void* mask,
+                      void* out, float* outf, const double* scale, cudaStream_t s) {
+  TcScale sc;
+  for (int k = 0; k < 6; ++k) sc.s[k] = scale ? static_cast<float>(scale[k]) : 1.f;
+  return tile_rounds<TileB>(n) < tile_rounds<TileA>(n)
+             ? tc_launch_tile<CIN, EPI, TileB>(n, x, w, bias, res, mask, out, outf, sc, s)
+             : tc_launch_tile<CIN, EPI, TileA>(n, x, w, bias, res, mask, out, outf, sc, s);
 }
 
 }  // namespace
