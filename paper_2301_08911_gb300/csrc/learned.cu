@@ -53,20 +53,23 @@ __device__ __forceinline__ int wrapc(int a, int n) {
 // by their size and the weights are rounded to BF16), so the sums keep one fixed order: a
 // chunk's tiles of 128 voxels in order, the four 32-voxel quarters of the tiles as four FP32
 // chains, ((q0 + q1) + q2) + q3, then the chunks.
-// A cluster of four CTAs takes a chunk, CTA q its quarters, all 27 taps at once: warp w < 9
-// owns the taps (dx = -1, 0, 1) of (dy, dz) = (w % 3, w / 3) - 1 in 96 accumulators, one pair of
-// dy fragments feeding 24 MMAs. A quarter's dy and, per (dy, dz), its 32 shifted voxels plus
-// the at most 4 row neighbours outside the run are staged by 16-byte asynchronous copies,
-// kWgStages quarters deep, voxel-major as they lie in memory; ldmatrix.trans turns 8 x 8
+// A cluster of four CTAs takes a chunk, CTA q its quarters, all 27 taps at once: MMA warp w < 14
+// owns taps 2 w and 2 w + 1 in 64 accumulators (so that 16 warps of 128 registers fill an SM),
+// one pair of dy fragments feeding 16 MMAs. Two warps stage a quarter's dy and, per (dy, dz), its
+// 32 shifted voxels plus the at most 4 row neighbours outside the run by 16-byte asynchronous
+// copies, kWgStages quarters deep, voxel-major as they lie in memory; ldmatrix.trans turns 8 x 8
 // blocks on the way to the registers, its per-lane row addresses resolving the periodic x
 // neighbours. 16-byte chunk c of slot v sits at chunk c ^ (v / 2 % 4) of its row, so that
 // 8 consecutive slots' chunks fall on distinct banks. The quarters' chains meet through
-// distributed shared memory. Warp 9 of CTA 0 sums dy for the bias, voxel by voxel.
-// 64^3, 32 channels: 225 -> 172 us (a CTA per tap and chunk staged dy and x again for every tap,
-// transposing through 2-byte shared-memory stores: LSU 86 % busy).
+// distributed shared memory. Extra clusters in front sum dy for the bias, a chunk per warp,
+// voxel by voxel.
+// 64^3, 32 channels: 124 us (a CTA per tap and chunk staged dy and x again for every tap,
+// transposing through 2-byte shared-memory stores: 225 us, LSU 86 % busy; nine MMA warps
+// of three taps that also copied: 171 us, most of it copy instructions and their latency).
 constexpr int kWgTile = 128, kWgRun = 32, kWgCtas = 4;     // voxels of a tile, of a quarter; quarters
 constexpr int kWgSlots = kWgRun + 4;
-constexpr int kWgThreads = 10 * 32, kWgCopy = 9 * 32;      // nine MMA warps copy, one sums the bias
+constexpr int kWgMma = 14, kWgWarps = 16, kWgThreads = 32 * kWgWarps, kWgCopy = kWgThreads - 32 * kWgMma;
+constexpr int kWgBias = kWgCtas * kWgWarps;                // chunks of a bias cluster
 constexpr int kWgStages = 4;
 
 template <int CIN>
@@ -74,8 +77,7 @@ struct WgSmem {
   static constexpr int kDy = kWgRun * kC * 2, kX = 9 * kWgSlots * CIN * 2;
   static constexpr int kStage = kDy + kX;
   static constexpr int kSum = kTaps * kC * CIN * 4;        // the chain sums, in place of the stages
-  static constexpr int kMain = kWgStages * kStage > kSum ? kWgStages * kStage : kSum;
-  static constexpr int kBytes = kMain + 2 * kWgTile * kC * 2;   // and the bias warp's two dy tiles
+  static constexpr int kBytes = kWgStages * kStage > kSum ? kWgStages * kStage : kSum;
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -112,31 +114,33 @@ __device__ __forceinline__ uint32_t wg_at(int v, int c) {
 template <int CIN>
 __device__ __forceinline__ void wg_stage(size_t u0, size_t N, int n, const __nv_bfloat16* __restrict__ x,
                                          const __nv_bfloat16* __restrict__ dy, uint32_t s_dy, uint32_t s_x) {
-  constexpr int kCh = CIN / 8, kItems = 9 * kWgSlots * kCh;
+  constexpr int kCh = CIN / 8, kPerPass = kWgCopy / kCh;     // slots per pass of the copy warps
+  const int t = threadIdx.x - 32 * kWgMma;
   const int count = u0 >= N ? 0 : static_cast<int>(N - u0 < kWgRun ? N - u0 : kWgRun);
   if (count > 0) {
-    if (threadIdx.x < kWgRun * (kC / 8)) {
-      const int c = threadIdx.x % (kC / 8), i = threadIdx.x / (kC / 8);
+#pragma unroll
+    for (int k = 0; k < kWgRun * (kC / 8) / kWgCopy; ++k) {
+      const int c = t % (kC / 8), i = t / (kC / 8) + k * (kWgCopy / (kC / 8));
       cp_async16z(s_dy + wg_at<kC / 8>(i, c), dy + (u0 + (i < count ? i : 0)) * kC + c * 8, i < count);
     }
-#pragma unroll
-    for (int k = 0; k < (kItems + kWgCopy - 1) / kWgCopy; ++k) {
-      const int t = threadIdx.x + k * kWgCopy;
-      if (t >= kItems) break;
-      const int c = t % kCh, slot = (t / kCh) % kWgSlots, combo = t / (kCh * kWgSlots);
+#pragma unroll 1
+    for (int slot = t / kCh; slot < kWgSlots; slot += kPerPass) {
+      const int c = t % kCh;
       const int i = slot < kWgRun ? slot : (slot < kWgRun + 2 ? 0 : count - 1);   // the voxel whose row it is in
+      const bool live = i < count;
       int gx, gy, gz;
-      decode3(static_cast<unsigned>(u0) + (i < count ? i : 0), static_cast<unsigned>(n), gx, gy, gz);
+      decode3(static_cast<unsigned>(u0) + (live ? i : 0), static_cast<unsigned>(n), gx, gy, gz);
       if (slot == kWgRun) gx = gx == 0 ? n - 1 : gx - 1;
       if (slot == kWgRun + 1) gx = 0;
       if (slot == kWgRun + 2) gx = n - 1;
       if (slot == kWgRun + 3) gx = gx == n - 1 ? 0 : gx + 1;
-      gy += combo % 3 - 1;
-      gz += combo / 3 - 1;
-      gy = gy < 0 ? n - 1 : (gy == n ? 0 : gy);
-      gz = gz < 0 ? n - 1 : (gz == n ? 0 : gz);
-      const size_t v = static_cast<size_t>(gx) + static_cast<size_t>(n) * (gy + static_cast<size_t>(n) * gz);
-      cp_async16z(s_x + combo * (kWgSlots * CIN * 2) + wg_at<kCh>(slot, c), x + v * CIN + c * 8, i < count);
+      const Nb nb = make_nb(gx, gy, gz, n);   // the nine (dy, dz) rows share the slot's x
+      const uint32_t dst = s_x + wg_at<kCh>(slot, c);
+      const __nv_bfloat16* src = x + static_cast<size_t>(gx) * CIN + c * 8;
+#pragma unroll
+      for (int combo = 0; combo < 9; ++combo)
+        cp_async16z(dst + combo * (kWgSlots * CIN * 2),
+                    src + static_cast<size_t>(nb.Y[combo % 3] + nb.Z[combo / 3]) * CIN, live);
     }
   }
   cp_async_commit();
@@ -161,53 +165,82 @@ __device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
   return v;
 }
 
-// Partial gradients of chunk blockIdx.x / 4: part[(chunk * 27 + tap)][o][i], partb[chunk][o].
+// Partial gradients: part[(chunk * 27 + tap)][o][i], partb[chunk][o]. Clusters 0 .. bias - 1 take the
+// bias, the others one chunk each.
 template <int CIN>
 __global__ void __launch_bounds__(kWgThreads, 1)
-    k_wgrad(int n, int ntiles, int tiles_per_chunk, const __nv_bfloat16* __restrict__ x,
+    k_wgrad(int n, int ntiles, int tiles_per_chunk, int chunks, int bias, const __nv_bfloat16* __restrict__ x,
             const __nv_bfloat16* __restrict__ dy, float* __restrict__ part, float* __restrict__ partb) {
   using S = WgSmem<CIN>;
   constexpr int kCh = CIN / 8, NT = CIN / 8;
   extern __shared__ __align__(128) unsigned char wsm[];
   const uint32_t base = smem_u32(wsm);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int chunk = blockIdx.x / kWgCtas, q = blockIdx.x % kWgCtas;
+  const int q = blockIdx.x % kWgCtas, cluster = blockIdx.x / kWgCtas;
   const size_t N = static_cast<size_t>(n) * n * n;
-  const int t0 = chunk * tiles_per_chunk, t1 = min(ntiles, t0 + tiles_per_chunk);
 
-  if (warp < 9) {
+  if (cluster < bias) {
+    // lane = output channel, every voxel of the chunk in order, 32 loads ahead of the sum
+    const int chunk = cluster * kWgBias + q * kWgWarps + warp;
+    if (chunk >= chunks) return;
+    const size_t v0 = static_cast<size_t>(chunk) * tiles_per_chunk * kWgTile;
+    const size_t v1 = min(N, v0 + static_cast<size_t>(tiles_per_chunk) * kWgTile);
+    const __nv_bfloat16* d = dy + lane;
+    float cur[32], nxt[32], bsum = 0.f;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) cur[j] = v0 + j < v1 ? __bfloat162float(d[(v0 + j) * kC]) : 0.f;
+    for (size_t v = v0; v < v1; v += 32) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j) nxt[j] = v + 32 + j < v1 ? __bfloat162float(d[(v + 32 + j) * kC]) : 0.f;
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        bsum += cur[j];
+        cur[j] = nxt[j];
+      }
+    }
+    partb[static_cast<size_t>(chunk) * kC + lane] = bsum;
+    return;
+  }
+  const int chunk = cluster - bias;
+  const int t0 = chunk * tiles_per_chunk, t1 = min(ntiles, t0 + tiles_per_chunk);
+  auto run_of = [&](int tile) { return static_cast<size_t>(tile) * kWgTile + kWgRun * q; };
+  auto stage_at = [&](int k) { return base + static_cast<uint32_t>(k % kWgStages) * S::kStage; };
+
+  if (warp >= kWgMma) {
+    // ---- copies: stage k is in flight while stages before it are consumed
+#pragma unroll 1
+    for (int k = 0; k < kWgStages - 1; ++k) {
+      if (t0 + k < t1) wg_stage<CIN>(run_of(t0 + k), N, n, x, dy, stage_at(k), stage_at(k) + S::kDy);
+      else cp_async_commit();
+    }
+    for (int tile = t0; tile < t1; ++tile) {
+      const int k = tile - t0 + kWgStages - 1;
+      cp_async_wait<kWgStages - 2>();
+      __syncthreads();   // this stage is complete, the one before it consumed
+      if (t0 + k < t1) wg_stage<CIN>(run_of(t0 + k), N, n, x, dy, stage_at(k), stage_at(k) + S::kDy);
+      else cp_async_commit();
+    }
+    cp_async_wait<0>();
+    __syncthreads();
+  } else {
     // ldmatrix lanes: lanes 0-7, 8-15, 16-23, 24-31 give the row addresses of matrices 0..3.
     // A (dy^T): matrices (v 0-7, o chunk 0), (v 0-7, chunk 1), (v 8-15, chunk 0), (v 8-15, chunk 1)
     const int av = (lane & 7) + ((lane >> 4) << 3), ac = (lane >> 3) & 1;
     // B (x): (v 0-7, i chunk 0), (v 8-15, chunk 0), (v 0-7, chunk 1), (v 8-15, chunk 1)
     const int bv = (lane & 7) + (((lane >> 3) & 1) << 3), bc = lane >> 4;
-    float acc[3][2][NT][4];
+    float acc[2][2][NT][4];
 #pragma unroll
-    for (int t = 0; t < 3; ++t)
+    for (int t = 0; t < 2; ++t)
 #pragma unroll
       for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
           for (int e = 0; e < 4; ++e) acc[t][mt][nt][e] = 0.f;
-    auto run_of = [&](int tile) { return static_cast<size_t>(tile) * kWgTile + kWgRun * q; };
-    auto stage_at = [&](int k) { return base + static_cast<uint32_t>(k % kWgStages) * S::kStage; };
-#pragma unroll
-    for (int k = 0; k < kWgStages - 1; ++k) {
-      if (t0 + k < t1) wg_stage<CIN>(run_of(t0 + k), N, n, x, dy, stage_at(k), stage_at(k) + S::kDy);
-      else cp_async_commit();
-    }
     for (int tile = t0; tile < t1; ++tile) {
-      const int k = tile - t0;
-      cp_async_wait<kWgStages - 2>();
-      asm volatile("bar.sync 1, %0;\n" ::"n"(kWgCopy) : "memory");   // this stage is complete, the one before free
-      if (tile + kWgStages - 1 < t1)
-        wg_stage<CIN>(run_of(tile + kWgStages - 1), N, n, x, dy, stage_at(k + kWgStages - 1),
-                      stage_at(k + kWgStages - 1) + S::kDy);
-      else
-        cp_async_commit();
+      __syncthreads();
       const size_t u0 = run_of(tile);
-      const uint32_t s_dy = stage_at(k), s_x = s_dy + S::kDy + warp * (kWgSlots * CIN * 2);
+      const uint32_t s_dy = stage_at(tile - t0), s_x = s_dy + S::kDy;
 #pragma unroll
       for (int ks = 0; ks < 2; ++ks) {
         if (u0 + 16 * ks >= N) continue;   // past the grid: the products are zero
@@ -217,12 +250,15 @@ __global__ void __launch_bounds__(kWgThreads, 1)
         const int i = 16 * ks + bv;
         const int xi = static_cast<int>((static_cast<unsigned>(u0) + i) % static_cast<unsigned>(n));
 #pragma unroll
-        for (int t = 0; t < 3; ++t) {
-          const int slot = u0 + i < N ? wg_slot(i, xi, t - 1, n) : i;
+        for (int t = 0; t < 2; ++t) {
+          const int tap = 2 * warp + t;
+          if (tap >= kTaps) break;
+          const int slot = u0 + i < N ? wg_slot(i, xi, tap % 3 - 1, n) : i;
+          const uint32_t s_row = s_x + (tap / 3) * (kWgSlots * CIN * 2);
 #pragma unroll
           for (int h = 0; h < NT / 2; ++h) {
             uint32_t b[4];
-            ldmatrix_x4_t(b, s_x + wg_at<kCh>(slot, 2 * h + bc));
+            ldmatrix_x4_t(b, s_row + wg_at<kCh>(slot, 2 * h + bc));
 #pragma unroll
             for (int mt = 0; mt < 2; ++mt) {
               mma16816(acc[t][mt][2 * h], a[mt], b[0], b[1]);
@@ -232,49 +268,23 @@ __global__ void __launch_bounds__(kWgThreads, 1)
         }
       }
     }
-    cp_async_wait<0>();
-    asm volatile("bar.sync 1, %0;\n" ::"n"(kWgCopy) : "memory");   // the stages give way to the chain sums
+    __syncthreads();   // the stages give way to the chain sums
     float* sum = reinterpret_cast<float*>(wsm);
     const int g = lane >> 2, t4 = lane & 3;
 #pragma unroll
-    for (int t = 0; t < 3; ++t)
+    for (int t = 0; t < 2; ++t) {
+      if (2 * warp + t >= kTaps) break;
 #pragma unroll
       for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
-          float* d = sum + (3 * warp + t) * (kC * CIN) + (16 * mt + g) * CIN + 8 * nt + 2 * t4;
+          float* d = sum + (2 * warp + t) * (kC * CIN) + (16 * mt + g) * CIN + 8 * nt + 2 * t4;
           d[0] = acc[t][mt][nt][0];
           d[1] = acc[t][mt][nt][1];
           d[8 * CIN] = acc[t][mt][nt][2];
           d[8 * CIN + 1] = acc[t][mt][nt][3];
         }
-  } else if (q == 0) {
-    // bias: lane = output channel, every voxel of the chunk in order; dy's tiles one ahead
-    const uint32_t s_b = base + S::kMain;
-    auto fetch = [&](int tile) {
-      if (tile < t1) {
-#pragma unroll
-        for (int k = 0; k < kWgTile * kC * 2 / 16 / 32; ++k) {
-          const int t = lane + 32 * k, v = t / (kC / 8);
-          const size_t u = static_cast<size_t>(tile) * kWgTile + v;
-          cp_async16z(s_b + (tile & 1) * (kWgTile * kC * 2) + t * 16, dy + (u < N ? u : 0) * kC + t % (kC / 8) * 8, u < N);
-        }
-      }
-      cp_async_commit();
-    };
-    float bsum = 0.f;
-    fetch(t0);
-    for (int tile = t0; tile < t1; ++tile) {
-      fetch(tile + 1);
-      cp_async_wait<1>();
-      __syncwarp();
-      const __nv_bfloat16* d = reinterpret_cast<const __nv_bfloat16*>(wsm + S::kMain + (tile & 1) * (kWgTile * kC * 2)) + lane;
-#pragma unroll 16
-      for (int j = 0; j < kWgTile; ++j) bsum += __bfloat162float(d[j * kC]);
-      __syncwarp();
     }
-    cp_async_wait<0>();
-    partb[static_cast<size_t>(chunk) * kC + lane] = bsum;
   }
   asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
   // each CTA adds a quarter of the values over the four chains
@@ -474,7 +484,8 @@ cudaError_t wgrad_launch(const WgradPlan& p, int n, const void* x, const void* d
   const cudaError_t e = cudaFuncSetAttribute(k_wgrad<CIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, shm);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(p.chunks * kWgCtas);
+  const int bias = (p.chunks + kWgBias - 1) / kWgBias;
+  cfg.gridDim = dim3((bias + p.chunks) * kWgCtas);
   cfg.blockDim = dim3(kWgThreads);
   cfg.dynamicSmemBytes = shm;
   cfg.stream = s;
@@ -485,7 +496,8 @@ cudaError_t wgrad_launch(const WgradPlan& p, int n, const void* x, const void* d
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_wgrad<CIN>, n, p.ntiles, p.tiles_per_chunk, static_cast<const __nv_bfloat16*>(x),
+  return cudaLaunchKernelEx(&cfg, k_wgrad<CIN>, n, p.ntiles, p.tiles_per_chunk, p.chunks, bias,
+                            static_cast<const __nv_bfloat16*>(x),
                             static_cast<const __nv_bfloat16*>(dy), part, partb);
 }
 }  // namespace
