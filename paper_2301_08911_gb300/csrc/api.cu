@@ -215,11 +215,17 @@ int ensure_hierarchy(homo_ctx* c) {
   return HOMO_OK;
 }
 
+// A coarse level above the on-chip form's sizes smooths in the staged form (a launch per
+// colour, the stencil through shared memory) wherever its rows allow the 16-byte copies; the
+// sizes of homo_set_coarse_smoother choose among the other forms.
+bool coarse_staged(const homo::Level& lv) { return lv.n > kStagedMinN && coarse_tile_ok(lv); }
+
 // One 8-colour sweep. first: the sweep starts from x = 0 (x need not be cleared; only
 // valid with colours in increasing order).
-// fmean (finest level only): plane means subtracted from f, or null.
+// fmean (finest level only): plane means subtracted from f, or null. chained: the launch before
+// on the stream was a colour pass of the same smoothing.
 int smooth_level(homo_ctx* c, int l, bool reverse, const float* f, float* x, bool first = false,
-                 const double* fmean = nullptr) {
+                 const float* fmean = nullptr, bool chained = false) {
   const int fz = first && !reverse ? 1 : 0;
   if (l == 0) {
     if (c->n <= c->gs_res_n && c->gs_resident > 0 && coarse_resident_ok(c->lev[0], c->gs_resident)) {
@@ -230,9 +236,13 @@ int smooth_level(homo_ctx* c, int l, bool reverse, const float* f, float* x, boo
       KL(c, HOMO_KC_FINE_GS, 1, launch_fine_gs(c, reverse ? 3 - k : k, reverse, f, x, fz, fmean));
     return HOMO_OK;
   }
+  const bool staged = coarse_staged(c->lev[l]);
   for (int k = 0; k < 8; ++k) {
     const int col = reverse ? 7 - k : k;
-    if (c->lev[l].n <= c->gs_split_n)
+    if (staged)
+      KL(c, HOMO_KC_COARSE_GS, 1,
+         launch_coarse_gs_tile(c->lev[l], col, f, x, fz, chained || k > 0 ? 1 : 0, c->stream));
+    else if (c->lev[l].n <= c->gs_split_n)
       KL(c, HOMO_KC_COARSE_GS, 1, launch_coarse_gs_item(c->lev[l], col, f, x, fz, c->stream));
     else KL(c, HOMO_KC_COARSE_GS, 1, launch_coarse_gs(c->lev[l], col, f, x, fz, c->stream));
   }
@@ -253,13 +263,13 @@ int smooth_level_sweeps(homo_ctx* c, int l, bool reverse, const float* f, float*
                                  c->gs_resident, c->stream));
     return HOMO_OK;
   }
-  if (l >= 1 && c->gs_cluster > 0 && c->lev[l].n <= c->gs_fuse_n) {
+  if (l >= 1 && c->gs_cluster > 0 && c->lev[l].n <= c->gs_fuse_n && !coarse_staged(c->lev[l])) {
     KL(c, HOMO_KC_COARSE_GS, 1,
        launch_coarse_gs_sweeps(c->lev[l], sweeps, reverse ? 1 : 0, first && !reverse ? 1 : 0, f, x,
                                c->gs_cluster, c->stream));
     return HOMO_OK;
   }
-  for (int k = 0; k < sweeps; ++k) RET(smooth_level(c, l, reverse, f, x, first && k == 0));
+  for (int k = 0; k < sweeps; ++k) RET(smooth_level(c, l, reverse, f, x, first && k == 0, nullptr, k > 0));
   return HOMO_OK;
 }
 
@@ -295,7 +305,7 @@ ChebCoef cheb_coef(double lam, int deg) {
 // One Chebyshev sweep of degree cheb_degree on level l. cur holds x (ignored when
 // from_zero), oth is free; on return cur holds the new x and oth is free. bmean (finest
 // level only): plane means subtracted from b, or null.
-int cheb_sweep(homo_ctx* c, int l, const float* b, const double* bmean, float*& cur, float*& oth,
+int cheb_sweep(homo_ctx* c, int l, const float* b, const float* bmean, float*& cur, float*& oth,
                bool from_zero) {
   const int deg = c->opts.cheb_degree;
   const ChebCoef k = cheb_coef(c->lam[l], deg);
@@ -323,7 +333,7 @@ int cheb_sweep(homo_ctx* c, int l, const float* b, const double* bmean, float*& 
 
 // V-cycle with Chebyshev smoothing (same polynomial before and after the coarse
 // correction, so M is symmetric); two buffers per level alternate as iterates.
-int vcycle_cheb(homo_ctx* c, const float* r, float* z, const double* rmean) {
+int vcycle_cheb(homo_ctx* c, const float* r, float* z, const float* rmean) {
   cudaStream_t s = c->stream;
   const int pre = c->opts.pre_sweeps, post = c->opts.post_sweeps;
   const int L = c->nlev - 1;
@@ -360,7 +370,7 @@ int vcycle_cheb(homo_ctx* c, const float* r, float* z, const double* rmean) {
 // Gauss-Seidel the post-smoother visits the colours in reverse order so M is symmetric.
 // rmean: the 18 plane means of r (the rigid-translation part, outside the range of K),
 // or null.
-int vcycle(homo_ctx* c, const float* r, float* z, const double* rmean = nullptr) {
+int vcycle(homo_ctx* c, const float* r, float* z, const float* rmean = nullptr) {
   cudaStream_t s = c->stream;
   if (c->nlev == 1) {   // the centred pseudo-inverse ignores the plane means
     KL(c, HOMO_KC_COARSEST, 1, launch_coarsest_apply(c, r, z));
@@ -406,7 +416,7 @@ int enq_read(homo_ctx* c, int slot, int count) {
 }
 
 // r = f - K (u + ulo); ||r_c - mean||^2 into S_RR, the plane means (the rigid
-// translations, outside the range of K) into S_RMEAN, active flags; enqueues the copy of
+// translations, outside the range of K) into F_RMEAN, active flags; enqueues the copy of
 // S_RR to the host (no synchronisation).
 // exact: double-float arithmetic throughout (residuals to ~1e-12 of the terms); otherwise
 // FP32 difference form from both parts of u (accurate to ~1e-7 of sum_d |A_d| |du_d|,
@@ -442,10 +452,12 @@ void record_history(homo_ctx* c) {
   }
 }
 
+const float* f32_slots(const homo_ctx* c) { return reinterpret_cast<const float*>(c->scal + S_F32); }
+
 int precondition_and_direction(homo_ctx* c, int first) {
   int g = 0;
-  RET(vcycle(c, c->r, c->z, c->scal + S_RMEAN));
-  KL(c, HOMO_KC_CG_VECTOR, 1, launch_dot6_zsum(c->r, c->z, c->N, c->scal + S_RMEAN, c->part, &g, c->stream));
+  RET(vcycle(c, c->r, c->z, f32_slots(c) + F_RMEAN));
+  KL(c, HOMO_KC_CG_VECTOR, 1, launch_dot6_zsum(c->r, c->z, c->N, f32_slots(c) + F_RMEAN, c->part, &g, c->stream));
   KL(c, HOMO_KC_CG_VECTOR, 1, launch_sum_step(kSumBeta, c->part, g, c->scal, first, 0.0, c->N, c->stream));
   KL(c, HOMO_KC_CG_VECTOR, 1, launch_cg_update_p(c->pv, c->z, c->scal, c->N, c->stream));
   return HOMO_OK;
@@ -900,7 +912,7 @@ int homo_create(homo_ctx** out, int n, double E0, double nu, double p, double Em
   }
   if (rc == HOMO_OK) {
     cudaError_t e = tiled_init();
-    if (e == cudaSuccess) e = coarsest_init();
+    if (e == cudaSuccess) e = coarse_init();
     if (e != cudaSuccess) rc = cuda_err(c, e, "tiled kernel attributes");
   }
   if (rc == HOMO_OK) {

@@ -135,6 +135,9 @@ __global__ void __launch_bounds__(256) k_galerkin_axis(const float* __restrict__
 __device__ __forceinline__ float ld_st(const float* p) { return __ldg(p); }
 __device__ __forceinline__ float ld_st(const __nv_bfloat16* p) { return __bfloat162float(__ldg(p)); }
 
+__device__ __forceinline__ float st_f32(float v) { return v; }
+__device__ __forceinline__ float st_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
+
 // Mixed precision: st16 = BF16 of (A_d(v) + A_-d(v+d)^T) / 2 for every vertex v and
 // neighbour d. Both partners of a pair are formed from the same two FP32 blocks (FP32
 // addition commutes and the halving is exact), so the rounded operator is exactly
@@ -365,6 +368,123 @@ __global__ void __launch_bounds__(kItemBlock) k_coarse_gs_item(const T* __restri
   }
 }
 
+// ---- colour pass with the stencil staged in shared memory
+// A CTA takes VERTS consecutive vertices of a colour and all six cases, CASES per thread. The
+// 243 stencil values of its vertices arrive by 16-byte asynchronous copies, three z-layers
+// as three groups, so that a layer computes while the next ones are in flight: the forms
+// above it keep at most a neighbour's or a layer's values in flight per thread, and the
+// thread-per-(vertex, case) form loads every stencil value six times. What is left are the
+// neighbour values (stride 2 along x) and, per case group, the stencil's shared-memory reads.
+// chained: the launch before in the stream is the colour pass before (programmatic dependent
+// launch): the copies start while that pass still runs, and only then does the kernel wait
+// for its results. The stencil was complete before the first, unchained pass of a chain.
+// Arithmetic and order are gs_item's: bitwise the iterates of the other forms.
+// Needs 16-byte aligned stencil rows: n a multiple of 4. One sweep with BF16 stencils, against
+// the L2 cluster form at 32^3 and the thread-per-vertex form above: 32^3 75 -> 36 us, 64^3
+// 216 -> 102 us, 128^3 885 -> 584 us; a 64^3 FP32 V-cycle 613 -> 508 us.
+// Start the copies of VERTS vertices' rows (positions m0 .. of the colour) into A[243][VERTS], a
+// commit group per z-layer.
+template <typename T, int CASES, int VERTS>
+__device__ __forceinline__ void stage_stencil(const T* __restrict__ st, size_t N, unsigned Nh, int colour, unsigned m0,
+                                              T* A) {
+  constexpr int kPer = 16 / static_cast<int>(sizeof(T)), kRowChunks = VERTS / kPer, kLayer = 81;
+  constexpr int kTileThreads = VERTS * kCases / CASES;
+  const T* src = st + static_cast<size_t>(colour) * Nh + m0;
+#pragma unroll 1
+  for (int layer = 0; layer < 3; ++layer) {
+    for (int t = threadIdx.x; t < kLayer * kRowChunks; t += kTileThreads) {
+      const int row = layer * kLayer + t / kRowChunks, c = t % kRowChunks * kPer;
+      if (m0 + c < Nh)   // Nh is a multiple of kPer: a chunk is inside or outside
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(
+                         static_cast<unsigned>(__cvta_generic_to_shared(A + row * VERTS + c))),
+                     "l"(src + static_cast<size_t>(row) * N + c)
+                     : "memory");
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  }
+}
+
+// The layer's rows are in shared memory for the whole block.
+__device__ __forceinline__ void stage_wait(int layer) {
+  if (layer == 0) asm volatile("cp.async.wait_group 2;\n" ::: "memory");
+  else if (layer == 1) asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+  else asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  __syncthreads();
+}
+
+template <typename T, int CASES, int VERTS>
+__global__ void __launch_bounds__(VERTS * kCases / CASES)
+    k_coarse_gs_tile(const T* __restrict__ st, const float* __restrict__ f, float* x, int n, int colour, int fz,
+                     int chained) {
+  extern __shared__ __align__(16) unsigned char tile_smem[];
+  T* A = reinterpret_cast<T*>(tile_smem);                   // [243][VERTS]
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const size_t N = static_cast<size_t>(n) * n * n;
+  const int h = n >> 1;
+  const unsigned Nh = static_cast<unsigned>(h) * h * h;
+  const unsigned m0 = blockIdx.x * VERTS;
+  stage_stencil<T, CASES, VERTS>(st, N, Nh, colour, m0, A);
+  if (chained) asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int j = static_cast<int>(threadIdx.x) % VERTS;
+  const int c0 = static_cast<int>(threadIdx.x) / VERTS * CASES;
+  const unsigned m = m0 + j;
+  const bool live = m < Nh;
+  int i, jj, kk;
+  decode3(live ? m : 0u, static_cast<unsigned>(h), i, jj, kk);
+  const int X = 2 * i + (colour & 1), Y = 2 * jj + ((colour >> 1) & 1), Z = 2 * kk + (colour >> 2);
+  const Nb nb = make_nb(X, Y, Z, n);
+  const size_t v = static_cast<size_t>(X) + static_cast<size_t>(n) * (Y + static_cast<size_t>(n) * Z);
+  const float* fc = f + static_cast<size_t>(3 * c0) * N + v;
+  const float* xc = x + static_cast<size_t>(3 * c0) * N;   // plain loads: the pass before wrote it
+  float b[3 * CASES];
+#pragma unroll
+  for (int q = 0; q < 3 * CASES; ++q) b[q] = __ldg(fc + q * N);
+  float S[9];
+#pragma unroll
+  for (int layer = 0; layer < 3; ++layer) {
+    float U[9][3 * CASES];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      const int d = 9 * layer + e;
+      const int odd = (d % 3 != 1) | (((d / 3) % 3 != 1) << 1) | ((d / 9 != 1) << 2);
+      if (d == 13 || (fz && (colour ^ odd) > colour)) continue;
+      const float* xw = xc + (nb.X[d % 3] + nb.Y[(d / 3) % 3] + nb.Z[d / 9]);
+#pragma unroll
+      for (int q = 0; q < 3 * CASES; ++q) U[e][q] = xw[q * N];
+    }
+    stage_wait(layer);
+    const T* Al = A + layer * 81 * VERTS + j;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      const int d = 9 * layer + e;
+      const int odd = (d % 3 != 1) | (((d / 3) % 3 != 1) << 1) | ((d / 9 != 1) << 2);
+      if (d == 13) {
+#pragma unroll
+        for (int q = 0; q < 9; ++q) S[q] = st_f32(Al[(9 * e + q) * VERTS]);
+        continue;
+      }
+      if (fz && (colour ^ odd) > colour) continue;
+      float a[9];
+#pragma unroll
+      for (int q = 0; q < 9; ++q) a[q] = st_f32(Al[(9 * e + q) * VERTS]);
+#pragma unroll
+      for (int c = 0; c < CASES; ++c)
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+          b[3 * c + r] = fmaf(-a[3 * r + 2], U[e][3 * c + 2],
+                              fmaf(-a[3 * r + 1], U[e][3 * c + 1], fmaf(-a[3 * r], U[e][3 * c], b[3 * c + r])));
+    }
+  }
+  if (!live) return;
+  const Factor3 F = factor3(S);
+#pragma unroll
+  for (int c = 0; c < CASES; ++c) {
+    solve3(F, b[3 * c], b[3 * c + 1], b[3 * c + 2]);
+#pragma unroll
+    for (int r = 0; r < 3; ++r) x[static_cast<size_t>(3 * (c0 + c) + r) * N + v] = b[3 * c + r];
+  }
+}
+
 // Every sweep of one smoothing phase on a small level in one launch. Gauss-Seidel does
 // not couple the load cases, so the grid is six thread-block clusters of csize CTAs, one
 // per case, that never wait on one another: a cluster's colour passes are separated by
@@ -510,8 +630,8 @@ struct StoredRows {   // a coarse level's stencil
 struct FineRows {   // the finest level: built from the moduli, as its other kernels do
   const KeParam& K;
   const float* E;
-  const double* fmean;
-  __device__ __forceinline__ float mean(int q) const { return fmean ? static_cast<float>(fmean[q]) : 0.f; }
+  const float* fmean;
+  __device__ __forceinline__ float mean(int q) const { return fmean ? __ldg(fmean + q) : 0.f; }
   template <typename Put>
   __device__ __forceinline__ void load(int colour, unsigned m, int n, int r, Put put, float (&S)[9]) const {
     int i, j, k;
@@ -596,6 +716,7 @@ __device__ __forceinline__ void gs_resident(const Rows& src, const float* __rest
   }
   __syncthreads();
   // the CTAs that read this one's vertices: owners of positions at most one half-grid step away
+  unsigned mine = 0u;
   for (int t = threadIdx.x; t < 27 * mcount; t += kResThreads) {
     const int d = t / mcount;
     int a, b, k;
@@ -603,8 +724,10 @@ __device__ __forceinline__ void gs_resident(const Rows& src, const float* __rest
     a = (a + d % 3 - 1 + h) % h;
     b = (b + (d / 3) % 3 - 1 + h) % h;
     k = (k + d / 9 - 1 + h) % h;
-    atomicOr(&need_s, 1u << ((a + h * (b + h * k)) / Mper));
+    mine |= 1u << ((a + h * (b + h * k)) / Mper);
   }
+  mine = __reduce_or_sync(0xffffffffu, mine);   // one atomic per warp, not one per neighbour
+  if (lane == 0 && mine) atomicOr(&need_s, mine);
   __syncthreads();
   unsigned target[kResTargets];   // displacement copies this lane writes (rows split them), 0: none
 #pragma unroll
@@ -689,7 +812,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_fine_gs_resident(const __gri
                                                                     const float* __restrict__ E,
                                                                     const float* __restrict__ f, float* x, int n,
                                                                     int reverse, int first,
-                                                                    const double* __restrict__ fmean, int csize,
+                                                                    const float* __restrict__ fmean, int csize,
                                                                     int Mper) {
   gs_resident<kGroups>(FineRows{K, E, fmean}, f, x, n, 1, reverse, first, csize, Mper);
 }
@@ -731,6 +854,67 @@ __global__ void __launch_bounds__(256) k_coarse_residual(const T* __restrict__ s
 #pragma unroll
     for (int q = 0; q < kPlanes; ++q) out[q * N + v] = __ldg(b + q * N + v) - acc[q];
   }
+}
+
+// The same in the staged form of k_coarse_gs_tile (the stencil of VERTS vertices of one colour
+// through shared memory, CASES load cases per thread, n a multiple of 4), with the FMA order of
+// k_coarse_residual: a thread of that kernel waits for 27 neighbours one after another
+// (8^3: 25 -> 6 us).
+template <typename T, int CASES, int VERTS>
+__global__ void __launch_bounds__(VERTS * kCases / CASES)
+    k_coarse_residual_tile(const T* __restrict__ st, const float* __restrict__ bv, const float* x,
+                           float* out, int n, unsigned blocks_per_colour) {
+  extern __shared__ __align__(16) unsigned char tile_smem[];
+  T* A = reinterpret_cast<T*>(tile_smem);                   // [243][VERTS]
+  const size_t N = static_cast<size_t>(n) * n * n;
+  const int h = n >> 1;
+  const unsigned Nh = static_cast<unsigned>(h) * h * h;
+  const int colour = static_cast<int>(blockIdx.x / blocks_per_colour);
+  const unsigned m0 = (blockIdx.x - colour * blocks_per_colour) * VERTS;
+  stage_stencil<T, CASES, VERTS>(st, N, Nh, colour, m0, A);
+  const int j = static_cast<int>(threadIdx.x) % VERTS;
+  const int c0 = static_cast<int>(threadIdx.x) / VERTS * CASES;
+  const unsigned m = m0 + j;
+  const bool live = m < Nh;
+  int i, jj, kk;
+  decode3(live ? m : 0u, static_cast<unsigned>(h), i, jj, kk);
+  const int X = 2 * i + (colour & 1), Y = 2 * jj + ((colour >> 1) & 1), Z = 2 * kk + (colour >> 2);
+  const Nb nb = make_nb(X, Y, Z, n);
+  const size_t v = static_cast<size_t>(X) + static_cast<size_t>(n) * (Y + static_cast<size_t>(n) * Z);
+  const float* xc = x + static_cast<size_t>(3 * c0) * N;
+  float acc[3 * CASES], b[3 * CASES];
+#pragma unroll
+  for (int q = 0; q < 3 * CASES; ++q) {
+    acc[q] = 0.f;
+    b[q] = __ldg(bv + (3 * c0 + q) * N + v);
+  }
+#pragma unroll
+  for (int layer = 0; layer < 3; ++layer) {
+    float U[9][3 * CASES];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      const float* xw = xc + (nb.X[e % 3] + nb.Y[e / 3] + nb.Z[layer]);
+#pragma unroll
+      for (int q = 0; q < 3 * CASES; ++q) U[e][q] = xw[q * N];   // plain loads: kept before the barrier
+    }
+    stage_wait(layer);
+    const T* Al = A + layer * 81 * VERTS + j;
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+      float a[9];
+#pragma unroll
+      for (int q = 0; q < 9; ++q) a[q] = st_f32(Al[(9 * e + q) * VERTS]);
+#pragma unroll
+      for (int c = 0; c < CASES; ++c)
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+          acc[3 * c + r] = fmaf(a[3 * r], U[e][3 * c], fmaf(a[3 * r + 1], U[e][3 * c + 1],
+                                fmaf(a[3 * r + 2], U[e][3 * c + 2], acc[3 * c + r])));
+    }
+  }
+  if (!live) return;
+#pragma unroll
+  for (int q = 0; q < 3 * CASES; ++q) out[static_cast<size_t>(3 * c0 + q) * N + v] = b[q] - acc[q];
 }
 
 // Chebyshev step with the stored stencil (threads walk vertices in lexicographic order):
@@ -978,11 +1162,10 @@ __device__ __forceinline__ void sweep_diagonal(double (&D)[kSw][kSw + 1], double
     const double ip = ip_s, cv = D[r][t], rv = D[t][c], av = D[r][c];
     if (c == t) b.dcol[r * kSw + t] = cv;
     if (r == t) b.drow[t * kSw + c] = rv;
-    double val;
-    if (r == t && c == t) val = ip;
-    else if (r == t) val = rv * ip;
-    else if (c == t) val = -cv * ip;
-    else val = sweep_update(av, cv, rv, ip);
+    // one product and one FMA in every lane: r[j] ip = fma(r[j], ip, 0), and so on
+    double p = __dmul_rn(cv, rv);
+    p = r == t ? (c == t ? -1.0 : -rv) : (c == t ? cv : p);
+    const double val = fma(-p, ip, r == t || c == t ? 0.0 : av);
     __syncthreads();
     D[r][c] = val;
   }
@@ -1000,46 +1183,52 @@ __global__ void __launch_bounds__(kSw * kSw) k_coarsest_first(double* __restrict
   A[static_cast<size_t>(r) * mp + c] = D[r][c];
 }
 
-// Panel k: block b < nb the column tile (b, k), block nb + b the row tile (k, b); b = k skipped
-// (its own steps ran before). Half a warp holds a tile row (column) of kSw values, lane s its
-// value s; step t broadcasts value t within the half warp.
-__global__ void __launch_bounds__(kSw * kSw) k_coarsest_panel(double* __restrict__ A, int mp, int k, SweepBuf b) {
+// Panel k: tile b < nb is the column tile (b, k), nb + b the row tile (k, b); b = k skipped (its own
+// steps ran before). Two CTAs of eight rows (columns) per tile: half a warp holds a tile row
+// (column) of kSw values, lane s its value s; step t broadcasts value t within the half
+// warp. The steps are a chain of two FP64 instructions, whose issue (a warp's takes 16
+// clocks) is what the small CTAs spread over the SMs.
+__global__ void __launch_bounds__(kSw * kSw / 2) k_coarsest_panel(double* __restrict__ A, int mp, int k, SweepBuf b) {
   const int nb = mp / kSw;
-  const bool is_row = static_cast<int>(blockIdx.x) >= nb;
-  const int tile = is_row ? static_cast<int>(blockIdx.x) - nb : static_cast<int>(blockIdx.x);
+  const int id = static_cast<int>(blockIdx.x) >> 1;
+  const bool is_row = id >= nb;
+  const int tile = is_row ? id - nb : id;
   if (tile == k) return;
-  __shared__ double dv[kSw][kSw + 1], ips[kSw], T[kSw][kSw + 1];
-  const int i = threadIdx.x / kSw, s = threadIdx.x % kSw;
+  __shared__ double dv[kSw][kSw + 1], ips[kSw], T[kSw / 2][kSw + 1];
+  const int il = threadIdx.x / kSw, s = threadIdx.x % kSw;
+  const int i = il + (blockIdx.x & 1) * (kSw / 2);
   // dv[t][s]: what step t multiplies value t with to update value s
-  dv[is_row ? s : i][is_row ? i : s] = is_row ? b.dcol[i * kSw + s] : b.drow[i * kSw + s];
+  for (int e = threadIdx.x; e < kSw * kSw; e += kSw * kSw / 2) {
+    const int x = e / kSw, y = e % kSw;
+    dv[is_row ? y : x][is_row ? x : y] = is_row ? b.dcol[e] : b.drow[e];
+  }
   if (threadIdx.x < kSw) ips[threadIdx.x] = b.ip[threadIdx.x];
-  const size_t at = is_row ? static_cast<size_t>(kSw * k + i) * mp + kSw * tile + s
+  // a row tile is transposed on the way: lane s of half warp il takes row s of column i
+  const int half = kSw / 2;
+  const size_t at = is_row ? static_cast<size_t>(kSw * k + threadIdx.x / half) * mp + kSw * tile +
+                                 (blockIdx.x & 1) * half + threadIdx.x % half
                            : static_cast<size_t>(kSw * tile + i) * mp + kSw * k + s;
   double v = A[at];
-  if (is_row) {   // lane s of half warp i takes row s of column i
-    T[i][s] = v;
-    __syncthreads();
-    v = T[s][i];
-  } else {
-    __syncthreads();
-  }
+  if (is_row) T[threadIdx.x % half][threadIdx.x / half] = v;
+  __syncthreads();
+  if (is_row) v = T[il][s];
   double save = 0.0;
 #pragma unroll
   for (int t = 0; t < kSw; ++t) {
     const double x = __shfl_sync(0xffffffffu, v, t, kSw);
+    double p = __dmul_rn(x, dv[t][s]);
     if (s == t) {
       save = x;
-      v = is_row ? x * ips[t] : -x * ips[t];
-    } else {
-      v = sweep_update(v, x, dv[t][s], ips[t]);
+      p = is_row ? -x : x;
     }
+    v = fma(-p, ips[t], s == t ? 0.0 : v);
   }
   (is_row ? b.row : b.col)[static_cast<size_t>(kSw * tile + i) * kSw + s] = save;
   if (is_row) {
     __syncthreads();
-    T[s][i] = v;
+    T[il][s] = v;
     __syncthreads();
-    v = T[i][s];
+    v = T[threadIdx.x % half][threadIdx.x / half];
   }
   A[at] = v;
 }
@@ -1111,36 +1300,39 @@ __global__ void __launch_bounds__(256) k_coarsest_centre(const double* __restric
   }
 }
 
-// x = G b for the 6 cases (FP64 dot products), one warp per output row for all cases: G is
-// read once and the right-hand sides are converted to FP64 once per CTA (a conversion
-// costs as much of the narrow FP64 pipe as a multiply-add). Two rows per CTA spread the
-// FP64 work (2 operations per clock and SM) over more SMs.
-constexpr int kApplyBlock = 64;
-
-__global__ void __launch_bounds__(kApplyBlock) k_coarsest_apply(const double* __restrict__ G, int m,
-                                                        const float* __restrict__ b,
-                                                        float* __restrict__ x) {
-  extern __shared__ double bs[];   // [case][j]
-  const int nv = m / 3;
-  for (int t = threadIdx.x; t < kCases * m; t += blockDim.x) {
-    const int c = t / m, j = t - c * m;
-    bs[t] = static_cast<double>(b[static_cast<size_t>(3 * c + j % 3) * nv + j / 3]);
-  }
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (i >= m) return;
-  double s[kCases] = {};
+// x = G b for the 6 cases (FP64 dot products), a warp per ROWS output rows for all cases, each in
+// a CTA of its own: the FP64 pipe (2 operations per clock and SM, a conversion from FP32
+// costing one) bounds it, so the rows spread over every SM, and where there are more rows
+// than that a warp shares the converted right-hand sides between two.
+template <int ROWS>
+__global__ void __launch_bounds__(32) k_coarsest_apply(const double* __restrict__ G, int m,
+                                                       const float* __restrict__ b,
+                                                       float* __restrict__ x) {
+  const int nv = m / 3, lane = threadIdx.x;
+  const int i0 = blockIdx.x * ROWS;
+  double s[ROWS][kCases] = {};
+#pragma unroll 2
   for (int j = lane; j < m; j += 32) {
-    const double g = G[static_cast<size_t>(i) * m + j];
+    const int w = j / 3, k = j - 3 * w;
+    double g[ROWS];
 #pragma unroll
-    for (int c = 0; c < kCases; ++c) s[c] = fma(g, bs[c * m + j], s[c]);
+    for (int r = 0; r < ROWS; ++r) g[r] = i0 + r < m ? __ldg(G + static_cast<size_t>(i0 + r) * m + j) : 0.0;
+#pragma unroll
+    for (int c = 0; c < kCases; ++c) {
+      const double v = static_cast<double>(__ldg(b + static_cast<size_t>(3 * c + k) * nv + w));
+#pragma unroll
+      for (int r = 0; r < ROWS; ++r) s[r][c] = fma(g[r], v, s[r][c]);
+    }
   }
 #pragma unroll
-  for (int c = 0; c < kCases; ++c) {
+  for (int r = 0; r < ROWS; ++r) {
+    const int i = i0 + r;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s[c] += __shfl_down_sync(0xffffffffu, s[c], o);
-    if (lane == 0) x[static_cast<size_t>(3 * c + i % 3) * nv + i / 3] = static_cast<float>(s[c]);
+    for (int c = 0; c < kCases; ++c) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s[r][c] += __shfl_down_sync(0xffffffffu, s[r][c], o);
+      if (lane == 0 && i < m) x[static_cast<size_t>(3 * c + i % 3) * nv + i / 3] = static_cast<float>(s[r][c]);
+    }
   }
 }
 
@@ -1179,11 +1371,80 @@ cudaError_t launch_galerkin(const Level& Lf, const Level& Lc, float* tmp1, float
   return cudaGetLastError();
 }
 
+namespace {
+
+template <typename T, int CASES, int VERTS>
+cudaError_t tile_launch(const Level& L, const T* st, int colour, int first, int chained, const float* f, float* x,
+                        cudaStream_t s) {
+  const size_t h = static_cast<size_t>(L.n / 2), Nh = h * h * h;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>((Nh + VERTS - 1) / VERTS));
+  cfg.blockDim = dim3(VERTS * kCases / CASES);
+  cfg.dynamicSmemBytes = static_cast<size_t>(kStencil) * VERTS * sizeof(T);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k_coarse_gs_tile<T, CASES, VERTS>, st, f, x, L.n, colour, first, chained);
+}
+
+// A colour pass in the staged form: a case per thread up to kTileSplitN cells per axis (the
+// threads to fill the chip), three above (the stencil's shared-memory reads per case).
+constexpr int kTileSplitN = 96;
+
+template <typename T>
+cudaError_t tile_pass(const Level& L, const T* st, int colour, int first, int chained, const float* f, float* x,
+                      cudaStream_t s) {
+  return L.n <= kTileSplitN ? tile_launch<T, 1, 32>(L, st, colour, first, chained, f, x, s)
+                            : tile_launch<T, 3, 64>(L, st, colour, first, chained, f, x, s);
+}
+
+template <typename T, int CASES, int VERTS>
+cudaError_t tile_attr() {
+  constexpr int shm = static_cast<int>(kStencil * VERTS * sizeof(T));
+  const cudaError_t e = cudaFuncSetAttribute(k_coarse_gs_tile<T, CASES, VERTS>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, shm);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_coarse_residual_tile<T, CASES, VERTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, shm);
+}
+
+}  // namespace
+
+bool coarse_tile_ok(const Level& L) { return L.n % 4 == 0; }
+
+namespace {
+template <typename T, int CASES, int VERTS>
+void residual_tile(const Level& L, const T* st, const float* b, const float* x, float* out, cudaStream_t s) {
+  const size_t h = static_cast<size_t>(L.n / 2);
+  const unsigned blocks = static_cast<unsigned>((h * h * h + VERTS - 1) / VERTS);
+  k_coarse_residual_tile<T, CASES, VERTS><<<8 * blocks, VERTS * kCases / CASES, kStencil * VERTS * sizeof(T), s>>>(
+      st, b, x, out, L.n, blocks);
+}
+
+template <typename T>
+cudaError_t residual_launch(const Level& L, const T* st, const float* b, const float* x, float* out, cudaStream_t s) {
+  if (!coarse_tile_ok(L))
+    k_coarse_residual<<<grid_for(L.N, 256), 256, 0, s>>>(st, b, x, out, L.n, L.colour_blocked);
+  else if (L.n <= kTileSplitN)
+    residual_tile<T, 1, 32>(L, st, b, x, out, s);
+  else
+    residual_tile<T, 3, 64>(L, st, b, x, out, s);
+  return cudaGetLastError();
+}
+}  // namespace
+
 cudaError_t launch_coarse_residual(const Level& L, const float* b, const float* x, float* out,
                                    cudaStream_t s) {
-  if (L.sth) k_coarse_residual<<<grid_for(L.N, 256), 256, 0, s>>>(L.sth, b, x, out, L.n, L.colour_blocked);
-  else k_coarse_residual<<<grid_for(L.N, 256), 256, 0, s>>>(L.st, b, x, out, L.n, L.colour_blocked);
-  return cudaGetLastError();
+  return L.sth ? residual_launch(L, static_cast<const __nv_bfloat16*>(L.sth), b, x, out, s)
+               : residual_launch(L, static_cast<const float*>(L.st), b, x, out, s);
+}
+
+cudaError_t launch_coarse_gs_tile(const Level& L, int colour, const float* f, float* x, int first, int chained,
+                                  cudaStream_t s) {
+  return L.sth ? tile_pass(L, static_cast<const __nv_bfloat16*>(L.sth), colour, first, chained, f, x, s)
+               : tile_pass(L, static_cast<const float*>(L.st), colour, first, chained, f, x, s);
 }
 
 cudaError_t launch_coarse_gs(const Level& L, int colour, const float* f, float* x, int first,
@@ -1346,7 +1607,7 @@ cudaError_t resident_launch(const Level& L, const T* st, int sweeps, int reverse
 }  // namespace
 
 cudaError_t launch_fine_gs_resident(const homo_ctx* c, int reverse, const float* f, float* u, int first,
-                                    const double* fmean) {
+                                    const float* fmean) {
   ResidentLaunch r;
   if (!r.set(c->lev[0], c->gs_resident, c->stream)) return cudaErrorInvalidValue;
   const float* E = c->E;
@@ -1454,7 +1715,7 @@ cudaError_t launch_coarsest_setup(homo_ctx* c) {
   k_coarsest_dense<<<grid_for(27 * L.N, 256), 256, 0, c->stream>>>(L.st, L.n, L.colour_blocked, mp, c->A);
   k_coarsest_first<<<1, kSw * kSw, 0, c->stream>>>(c->A, mp, buf[0], status);
   for (int k = 0; k < np; ++k) {
-    k_coarsest_panel<<<2 * np, kSw * kSw, 0, c->stream>>>(c->A, mp, k, buf[k & 1]);
+    k_coarsest_panel<<<4 * np, kSw * kSw / 2, 0, c->stream>>>(c->A, mp, k, buf[k & 1]);
     k_coarsest_rest<<<dim3(np, np), kSw * kSw, 0, c->stream>>>(c->A, mp, k, buf[k & 1], buf[(k + 1) & 1], status);
   }
   k_coarsest_means<<<(3 * m + 127) / 128, 128, 0, c->stream>>>(c->A, m, mp, rmean);
@@ -1463,14 +1724,18 @@ cudaError_t launch_coarsest_setup(homo_ctx* c) {
   return cudaGetLastError();
 }
 
-cudaError_t coarsest_init() {   // shared-memory limit, before any capture
-  return cudaFuncSetAttribute(k_coarsest_apply, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(sizeof(double) * kCases * 1536));
+cudaError_t coarse_init() {   // shared-memory limits, before any capture
+  cudaError_t e = tile_attr<float, 1, 32>();
+  if (e == cudaSuccess) e = tile_attr<float, 3, 64>();
+  if (e == cudaSuccess) e = tile_attr<__nv_bfloat16, 1, 32>();
+  if (e == cudaSuccess) e = tile_attr<__nv_bfloat16, 3, 64>();
+  return e;
 }
 
 cudaError_t launch_coarsest_apply(const homo_ctx* c, const float* b, float* x) {
   const int m = c->mc;
-  k_coarsest_apply<<<(m * 32 + kApplyBlock - 1) / kApplyBlock, kApplyBlock, sizeof(double) * kCases * m, c->stream>>>(c->G, m, b, x);
+  if (m <= 2 * 152) k_coarsest_apply<1><<<m, 32, 0, c->stream>>>(c->G, m, b, x);
+  else k_coarsest_apply<2><<<(m + 1) / 2, 32, 0, c->stream>>>(c->G, m, b, x);
   return cudaGetLastError();
 }
 

@@ -70,7 +70,7 @@ __device__ __forceinline__ void vertex_of_pos(size_t p, int n, bool cb, int& x, 
 // in FP64) and store them at out[blockIdx.x * NV + k]. Fixed order: deterministic.
 template <int NV>
 __device__ __forceinline__ void block_sum_store(const float (&v)[NV], double* out) {
-  __shared__ double sh[32][NV];
+  __shared__ float sh[32][NV];   // converted by the one warp that adds them: FP64 is narrow here
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nw = (blockDim.x + 31) >> 5;
 #pragma unroll
@@ -78,12 +78,12 @@ __device__ __forceinline__ void block_sum_store(const float (&v)[NV], double* ou
     float s = v[k];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) sh[wid][k] = static_cast<double>(s);
+    if (lane == 0) sh[wid][k] = s;
   }
   __syncthreads();
   for (int k = threadIdx.x; k < NV; k += blockDim.x) {
     double s = 0.0;
-    for (int w = 0; w < nw; ++w) s += sh[w][k];
+    for (int w = 0; w < nw; ++w) s += static_cast<double>(sh[w][k]);
     out[static_cast<size_t>(blockIdx.x) * NV + k] = s;
   }
 }

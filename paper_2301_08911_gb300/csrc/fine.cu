@@ -7,6 +7,7 @@
 // and its neighbour v + d is
 //     A_d = sum over (t, j) with bits(t) + bits(j) - 1 = d of E_t * K0[7 - t, j],
 // built once per vertex and applied to all 6 load cases (the 6 cases share E and K0).
+#include <cstring>
 #include <mutex>
 #include <string>
 
@@ -190,7 +191,7 @@ __global__ void __launch_bounds__(128) k_fine_true_residual(const __grid_constan
 __global__ void __launch_bounds__(256) k_fine_jacobi_start(const __grid_constant__ KeParam K,
                                                            const float* __restrict__ E,
                                                            const float* __restrict__ b,
-                                                           const double* __restrict__ bmean,
+                                                           const float* __restrict__ bmean,
                                                            float* __restrict__ out, int n, float c0) {
   const size_t N = static_cast<size_t>(n) * n * n;
   for (size_t v = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; v < N;
@@ -205,7 +206,7 @@ __global__ void __launch_bounds__(256) k_fine_jacobi_start(const __grid_constant
     float rhs[kPlanes];
 #pragma unroll
     for (int q = 0; q < kPlanes; ++q)
-      rhs[q] = __ldg(b + q * N + v) - (bmean ? static_cast<float>(bmean[q]) : 0.f);
+      rhs[q] = __ldg(b + q * N + v) - (bmean ? __ldg(bmean + q) : 0.f);
     solve3x6(S, rhs);
 #pragma unroll
     for (int q = 0; q < kPlanes; ++q) out[q * N + v] = c0 * rhs[q];
@@ -254,6 +255,10 @@ struct ElemParam {
   float invN;
 };
 
+struct KePairs {   // k[c][r] = (K0[r][c], K0[r][c]) for two-lane FMAs
+  f32x2 k[24][24];
+};
+
 constexpr int kElemCases = kCases;            // one warp per load case
 constexpr int kElemBlock = 32 * kElemCases;   // 32 lanes x 6 cases, two elements per lane
 constexpr int kElemPad = 25;                  // w row stride in shared memory (bank spread)
@@ -272,8 +277,8 @@ __host__ __device__ constexpr int pair_slot(int i, int j) {
 // pairs dealt to it (q_ij = q_ji: the diagonal, i+1, i+2 and, for i < 3, i+3 mod 6, so
 // 3 or 4 each), reading the other w_j from shared memory.
 // A thread takes its elements of two consecutive grid steps at once, on the two lanes of
-// f32x2 registers (each lane rounded as the scalar chain): every constant of K0, read from
-// shared memory as a broadcast pair, and every instruction then serves two elements, where
+// f32x2 registers (each lane rounded as the scalar chain): every constant of K0 (a pair in
+// the parameter bank) and every instruction then serves two elements, where
 // the scalar form spent an instruction per constant as well (1700 a thread and element, 850
 // of them FMA-pipe). The rows of y come in two halves of 12, which keeps the registers
 // at 2 blocks per SM. 192^3, C^H and sensitivities together: 5.27 -> 5.1 ms.
@@ -284,7 +289,7 @@ __host__ __device__ constexpr int pair_slot(int i, int j) {
 // quadratic form, so the sum does not cancel across the 21 products (for the bulk
 // objective G has rank one and the sensitivity is a single quadratic form).
 template <int MODE>
-__global__ void __launch_bounds__(kElemBlock, 2) k_fine_elem(const __grid_constant__ KeParam K,
+__global__ void __launch_bounds__(kElemBlock, 2) k_fine_elem(const __grid_constant__ KePairs K,
                                                              const __grid_constant__ ChiParam X,
                                                              const __grid_constant__ ElemParam P,
                                                              const float* __restrict__ E,
@@ -293,16 +298,11 @@ __global__ void __launch_bounds__(kElemBlock, 2) k_fine_elem(const __grid_consta
                                                              const float* __restrict__ ulo, int n,
                                                              float* __restrict__ sens,
                                                              double* __restrict__ part) {
-  __shared__ __align__(16) f32x2 Ks[24][24];   // Ks[k][r] = (K0[r][k], K0[r][k])
   __shared__ f32x2 ws[kElemCases][32][kElemPad];
   __shared__ f32x2 sp[kElemCases][32];
   __shared__ double sacc[21];
   const int lane = threadIdx.x & 31, i = threadIdx.x >> 5;   // element slot, load case
   const unsigned N = static_cast<unsigned>(n) * n * n;       // n <= 1024
-  for (int t = threadIdx.x; t < 576; t += kElemBlock) {
-    const float k = K.k[(t % 24) * 24 + t / 24];
-    Ks[t / 24][t % 24] = pack2(k, k);
-  }
   const int npair = i < 3 ? 4 : 3;
   int jp[4], slot[4];
 #pragma unroll
@@ -364,13 +364,8 @@ __global__ void __launch_bounds__(kElemBlock, 2) k_fine_elem(const __grid_consta
       for (int r = 0; r < 12; ++r) yv[r] = 0ull;
 #pragma unroll
       for (int k = 0; k < 24; ++k) {
-        const ulonglong2* kp = reinterpret_cast<const ulonglong2*>(&Ks[k][12 * half]);
 #pragma unroll
-        for (int r = 0; r < 6; ++r) {
-          const ulonglong2 kk = kp[r];
-          yv[2 * r] = ffma2(kk.x, w[k], yv[2 * r]);
-          yv[2 * r + 1] = ffma2(kk.y, w[k], yv[2 * r + 1]);
-        }
+        for (int r = 0; r < 12; ++r) yv[r] = ffma2(K.k[k][12 * half + r], w[k], yv[r]);
       }
       if (MODE == 1) {
 #pragma unroll
@@ -441,7 +436,7 @@ cudaError_t launch_simp(const float* rho_in, float* rho_out, float* E, size_t N,
   return cudaGetLastError();
 }
 
-cudaError_t launch_fine_jacobi_start(const homo_ctx* c, const float* b, const double* bmean, float* out,
+cudaError_t launch_fine_jacobi_start(const homo_ctx* c, const float* b, const float* bmean, float* out,
                                      float c0) {
   k_fine_jacobi_start<<<grid_for(c->N, 256), 256, 0, c->stream>>>(c->ke, c->E, b, bmean, out, c->n, c0);
   return cudaGetLastError();
@@ -464,7 +459,7 @@ cudaError_t launch_fine_apply(const homo_ctx* c, const float* u, float* out, dou
 
 cudaError_t launch_fine_residual(const homo_ctx* c, const float* b, const float* u,
                                  const float* ulo, float* out, double* part, int* grid_out,
-                                 const double* bmean) {
+                                 const float* bmean) {
   if (ulo) {
     const int g = grid_for(c->N, 128);
     if (grid_out) *grid_out = g;
@@ -493,11 +488,18 @@ cudaError_t launch_fine_elem(const homo_ctx* c, int mode, const double* g36, flo
   P.invN = static_cast<float>(1.0 / static_cast<double>(c->N));
   const int g = grid_for((c->N + 31) / 32, 1);   // one block per 32 elements, capped
   if (grid_out) *grid_out = g;
+  KePairs kp;
+  for (int col = 0; col < 24; ++col)
+    for (int row = 0; row < 24; ++row) {
+      uint32_t b;
+      std::memcpy(&b, &c->ke.k[row * 24 + col], 4);
+      kp.k[col][row] = (static_cast<f32x2>(b) << 32) | b;
+    }
   if (mode == 0)
-    k_fine_elem<0><<<g, kElemBlock, 0, c->stream>>>(c->ke, c->chi, P, c->E, c->rho, c->u, c->ulo,
+    k_fine_elem<0><<<g, kElemBlock, 0, c->stream>>>(kp, c->chi, P, c->E, c->rho, c->u, c->ulo,
                                                    c->n, sens, part);
   else
-    k_fine_elem<1><<<g, kElemBlock, 0, c->stream>>>(c->ke, c->chi, P, c->E, c->rho, c->u, c->ulo,
+    k_fine_elem<1><<<g, kElemBlock, 0, c->stream>>>(kp, c->chi, P, c->E, c->rho, c->u, c->ulo,
                                                    c->n, sens, part);
   return cudaGetLastError();
 }

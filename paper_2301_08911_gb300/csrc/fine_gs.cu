@@ -137,7 +137,7 @@ __device__ __forceinline__ void gs_vertex(const KeParam& K, const float* __restr
 template <int CASES, int MAXT, bool REVERSE, bool VEC>
 __global__ void __launch_bounds__(MAXT, MAXT == 256 ? (CASES == 3 ? 3 : 2) : 1)
     k_fine_gs(const __grid_constant__ KeParam K, const float* __restrict__ E, const float* __restrict__ f,
-              float* __restrict__ u, int n, int pair, int first, const double* __restrict__ fmean, int rows) {
+              float* __restrict__ u, int n, int pair, int first, const float* __restrict__ fmean, int rows) {
   extern __shared__ float sh[];                            // [3 CASES][blockDim.x], then the means
   const int T = static_cast<int>(blockDim.x), me = static_cast<int>(threadIdx.x);
   float* fm = sh + 3 * CASES * T;
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? (CASES == 3 ? 3 : 2) : 1)
   const size_t q0 = 3 * CASES * blockIdx.y;                // first plane of the case group
   f += q0 * N;
   u += q0 * N;
-  if (me < 3 * CASES) fm[me] = fmean ? static_cast<float>(fmean[q0 + me]) : 0.f;
+  if (me < 3 * CASES) fm[me] = fmean ? __ldg(fmean + q0 + me) : 0.f;
   __syncthreads();
   const int lrow = me / h, i = me - lrow * h;
   const int row = static_cast<int>(blockIdx.x) * rows + lrow;
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(MAXT, MAXT == 256 ? (CASES == 3 ? 3 : 2) : 1)
 
 template <int CASES, int MAXT, bool VEC>
 cudaError_t gs_launch(const homo_ctx* c, int block, int pair, int reverse, const float* f, float* u, int first,
-                      const double* fmean) {
+                      const float* fmean) {
   const int h = c->n / 2;
   const int rows = h >= block ? 1 : block / h;
   const int threads = (rows * h + 31) / 32 * 32;
@@ -213,7 +213,7 @@ cudaError_t gs_launch(const homo_ctx* c, int block, int pair, int reverse, const
 bool gs_variant_ok(int cases, int block) { return (cases == 3 || cases == 6) && (block == 128 || block == 256); }
 
 cudaError_t launch_fine_gs(const homo_ctx* c, int pair, int reverse, const float* f, float* u, int first,
-                           const double* fmean) {
+                           const float* fmean) {
   const int b = c->gs_block;
   const bool wide = c->n > 512;   // a row of more than 256 pairs
   if ((reinterpret_cast<uintptr_t>(f) | reinterpret_cast<uintptr_t>(u)) % 8 != 0)

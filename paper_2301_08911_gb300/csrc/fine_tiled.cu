@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(kTiledThreads, MODE == 2 ? 1 : 2)
     k_fine_tiled(const __grid_constant__ KeParam K, const float* __restrict__ E,
                  const float* __restrict__ u, const float* __restrict__ ulo,
                  const float* __restrict__ b, float* out, int n, int zchunk,
-                 double* __restrict__ part, const double* __restrict__ bmean, float c0, float c1) {
+                 double* __restrict__ part, const float* __restrict__ bmean, float c0, float c1) {
   constexpr bool kLo = MODE == 2;
   extern __shared__ float sm[];
   float* su = sm;                                   // kUSlots x PLANE x kCh
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kTiledThreads, MODE == 2 ? 1 : 2)
         // residual, block-diagonal solve, Chebyshev update
 #pragma unroll
         for (int q = 0; q < kPlanes; ++q)
-          acc[q] = (__ldg(b + q * N + v) - (bmean ? static_cast<float>(bmean[q]) : 0.f)) - acc[q];
+          acc[q] = (__ldg(b + q * N + v) - (bmean ? __ldg(bmean + q) : 0.f)) - acc[q];
         solve3x6(S, acc);
 #pragma unroll
         for (int q = 0; q < kPlanes; ++q) {
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(kTiledThreads, MODE == 2 ? 1 : 2)
         for (int q = 0; q < kPlanes; ++q) {
           const size_t o = q * N + v;
           float val = acc[q];
-          if (MODE == 3) val = (__ldg(b + o) - (bmean ? static_cast<float>(bmean[q]) : 0.f)) - val;
+          if (MODE == 3) val = (__ldg(b + o) - (bmean ? __ldg(bmean + q) : 0.f)) - val;
           if (MODE == 2) val = __ldg(b + o) - val;
           out[o] = val;
           if (MODE == 1) red[q / 3] = fmaf(own1[kDiff ? q : 0], val, red[q / 3]);
@@ -291,7 +291,7 @@ int tiled_grid_blocks(int n) {
 namespace {
 template <int MODE>
 cudaError_t run_tiled(const homo_ctx* c, dim3 grid, int zc, const float* u, const float* ulo, const float* b,
-                      float* out, double* part, const double* bmean, float c0, float c1) {
+                      float* out, double* part, const float* bmean, float c0, float c1) {
   const size_t shm = tiled_smem_bytes(MODE);   // limit set by tiled_init at context creation
   k_fine_tiled<MODE><<<grid, kTiledThreads, shm, c->stream>>>(c->ke, c->E, u, ulo, b, out, c->n, zc, part,
                                                               bmean, c0, c1);
@@ -316,7 +316,7 @@ cudaError_t tiled_init() {
 }
 
 cudaError_t launch_fine_tiled(const homo_ctx* c, int mode, const float* u, const float* b, float* out,
-                              double* part, int* grid_out, const double* bmean, float c0, float c1,
+                              double* part, int* grid_out, const float* bmean, float c0, float c1,
                               const float* ulo) {
   const int n = c->n;
   const int zc = tiled_zchunk(n);

@@ -102,8 +102,20 @@ enum Slot : int {
   S_ACTIVE = 96,   // 1.0 while case c iterates  [6]
   S_CH = 102,      // C^H sums                   [21]
   S_OC = 128,      // OC scratch                 [64]
-  S_RMEAN = 192,   // plane means of r, subtracted by every consumer of r [18]
-  S_COUNT = 210
+  S_F32 = 192,     // FP32 copies for the vector kernels (homo::SlotF floats from here on)
+  S_COUNT = 225
+};
+
+// The scalars the vector kernels use, rounded to FP32 once by the step that forms them (FP64
+// divisions and conversions by every thread of a vector kernel cost more than its loads on
+// small cells, and half a millisecond a launch on 256^3: 2 FP64 operations per clock and SM).
+// Floats from scal + S_F32.
+enum SlotF : int {
+  F_RMEAN = 0,     // plane means of r, subtracted by every consumer of r [18]
+  F_ZMEAN = 18,    // plane means of z [18]
+  F_QMEAN = 36,    // plane means of q = K p [18]
+  F_ALPHA = 54,    // alpha_c [6]
+  F_BETA = 60      // beta_c [6]
 };
 
 struct homo_ctx_impl;
@@ -214,10 +226,10 @@ cudaError_t launch_fine_apply(const homo_ctx* c, const float* u, float* out, dou
 // 4 = u + c0 S^-1 (b - bmean - K u); 5 = u + c0 (u - out) + c1 S^-1 (b - bmean - K u), in
 // place on out; 6 = (1 + c0) u + c1 S^-1 (b - bmean - K u) (Chebyshev steps)
 cudaError_t launch_fine_tiled(const homo_ctx* c, int mode, const float* u, const float* b, float* out,
-                              double* part, int* grid_out, const double* bmean = nullptr,
+                              double* part, int* grid_out, const float* bmean = nullptr,
                               float c0 = 0.f, float c1 = 0.f, const float* ulo = nullptr);
 // out = c0 S^-1 (b - bmean) pointwise on level 0 (first Chebyshev step from zero)
-cudaError_t launch_fine_jacobi_start(const homo_ctx* c, const float* b, const double* bmean, float* out,
+cudaError_t launch_fine_jacobi_start(const homo_ctx* c, const float* b, const float* bmean, float* out,
                                      float c0);
 // coarse Chebyshev step with the stored stencil: x_in == null means x_in = 0;
 // mode 0: out = x_in + c0 S^-1 (b - K x_in); mode 1: out = x_in + c0 (x_in - out) + c1 S^-1 (b - K x_in);
@@ -242,16 +254,16 @@ int tiled_grid_blocks(int n);
 // plane means or null).
 cudaError_t launch_fine_residual(const homo_ctx* c, const float* b, const float* u,
                                  const float* ulo, float* out, double* part, int* grid_out,
-                                 const double* bmean);
+                                 const float* bmean);
 // Colours 2 pair and 2 pair + 1 (reverse: the odd one first) of one sweep on the finest level.
 // first != 0: first sweep from u = 0 (colours 0..7; u need not be cleared); fmean: plane
 // means subtracted from f, or null
 cudaError_t launch_fine_gs(const homo_ctx* c, int pair, int reverse, const float* f, float* u, int first,
-                           const double* fmean);
+                           const float* fmean);
 // The whole sweep in one launch (coarse.cu, the resident form with rows built from E and K0);
 // the finest level must satisfy coarse_resident_ok. Bitwise the sweep of launch_fine_gs.
 cudaError_t launch_fine_gs_resident(const homo_ctx* c, int reverse, const float* f, float* u, int first,
-                                    const double* fmean);
+                                    const float* fmean);
 // (cases, block) is a compiled variant of the fine Gauss-Seidel kernel
 bool gs_variant_ok(int cases, int block);
 cudaError_t launch_fine_elem(const homo_ctx* c, int mode, const double* g36, float* sens,
@@ -266,6 +278,13 @@ cudaError_t launch_coarse_residual(const Level& L, const float* b, const float* 
                                    cudaStream_t s);
 cudaError_t launch_coarse_gs(const Level& L, int colour, const float* f, float* x, int first,
                              cudaStream_t s);
+// One colour pass of level L with the stencil staged in shared memory (coarse_tile_ok: rows are
+// 16-byte aligned); bitwise launch_coarse_gs. chained: the launch before on s was the colour
+// pass before of the same smoothing, whose end this one overlaps.
+constexpr int kStagedMinN = 16;   // levels above this many cells per axis take it
+bool coarse_tile_ok(const Level& L);
+cudaError_t launch_coarse_gs_tile(const Level& L, int colour, const float* f, float* x, int first, int chained,
+                                  cudaStream_t s);
 // Every sweep of one smoothing phase of level L (sweeps 8-colour sweeps, colours 7..0 when
 // reverse, the first from x = 0 when first) as one launch of a thread-block cluster of at
 // most cluster_max CTAs; bitwise the iterates of the per-colour launches.
@@ -291,7 +310,7 @@ cudaError_t launch_prolong_add(int nf, const float* coarse, float* fine, int ove
 // doubles of homo_ctx::A and kernels launched for a coarsest matrix of m unknowns
 size_t coarsest_work_doubles(int m);
 int coarsest_setup_kernels(int m);
-cudaError_t coarsest_init();   // kernel attributes on the current device (before any capture)
+cudaError_t coarse_init();   // kernel attributes on the current device (before any capture)
 cudaError_t launch_coarsest_setup(homo_ctx* c);
 cudaError_t launch_coarsest_apply(const homo_ctx* c, const float* b, float* x);
 cudaError_t launch_stencil_export(const Level& L, float* out, cudaStream_t s);
@@ -326,8 +345,8 @@ cudaError_t launch_sum_step(int step, const double* part, int nblk, double* scal
                             cudaStream_t s);
 cudaError_t launch_dot6(const float* a, const float* b, size_t N, double* part, int* grid_out,
                         cudaStream_t s);
-// (r - rmean, z) per case and plane sums of z; rmean: 18 doubles or null
-cudaError_t launch_dot6_zsum(const float* r, const float* z, size_t N, const double* rmean,
+// (r - rmean, z) per case and plane sums of z; rmean: 18 floats or null
+cudaError_t launch_dot6_zsum(const float* r, const float* z, size_t N, const float* rmean,
                              double* part, int* grid_out, cudaStream_t s);
 // e += alpha p, r -= alpha (q - mean q), partials of ||r||^2 and plane sums of r
 cudaError_t launch_cg_update_er(float* e, float* elo, float* r, const float* p, const float* q,

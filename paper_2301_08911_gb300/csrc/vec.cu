@@ -59,12 +59,20 @@ __device__ __forceinline__ void df_add(float& hi, float& lo, float d, float dlo)
   hi = s2;
 }
 
-// CG scalar steps (thread c < 6 of a block that has just written the sums they read).
+// CG scalar steps (thread c < 6 of a block that has just written the sums they read; the FP32
+// plane means by thread q < 18 of its second warp).
+__device__ __forceinline__ float* f32_of(double* s) { return reinterpret_cast<float*>(s + S_F32); }
+
+__device__ __forceinline__ void plane_mean(double* s, int sum_slot, int mean_slot, int q, double N) {
+  f32_of(s)[mean_slot + q] = static_cast<float>(s[sum_slot + q] / N);
+}
+
 __device__ __forceinline__ void cg_alpha(double* s, int c) {
   const double pq = s[S_PQ + c];
   double a = 0.0;
   if (s[S_ACTIVE + c] != 0.0 && pq > 0.0 && isfinite(pq)) a = s[S_RZ + c] / pq;
   s[S_ALPHA + c] = a;
+  f32_of(s)[F_ALPHA + c] = static_cast<float>(a);
 }
 
 // beta = rz_new / rz_old (0 on the first step or for finished cases); rz_old <- rz_new.
@@ -73,6 +81,7 @@ __device__ __forceinline__ void cg_beta(double* s, int c, int first) {
   double b = 0.0;
   if (!first && s[S_ACTIVE + c] != 0.0 && old != 0.0 && isfinite(rz)) b = rz / old;
   s[S_BETA + c] = b;
+  f32_of(s)[F_BETA + c] = static_cast<float>(b);
   s[S_RZ_OLD + c] = rz;
 }
 
@@ -85,7 +94,6 @@ __device__ __forceinline__ void cg_active(double* s, int c, double tol2, double 
   for (int k = 0; k < 3; ++k) {
     const double sum = s[S_RSUM + 3 * c + k];
     rr -= sum * sum / N;
-    s[S_RMEAN + 3 * c + k] = sum / N;
   }
   rr = fmax(rr, 0.0);
   s[S_RR + c] = rr;
@@ -130,10 +138,40 @@ __global__ void __launch_bounds__(256) k_sum_partials(const double* __restrict__
   }
   if (STEP == kSumOnly) return;
   __syncthreads();
+  if (t >= 32 && t < 32 + kPlanes)
+    plane_mean(scal, STEP == kSumAlpha ? S_QSUM : STEP == kSumBeta ? S_ZSUM : S_RSUM,
+               STEP == kSumAlpha ? F_QMEAN : STEP == kSumBeta ? F_ZMEAN : F_RMEAN, t - 32, N);
   if (t >= kCases) return;
   if (STEP == kSumAlpha) cg_alpha(scal, t);
   if (STEP == kSumBeta) cg_beta(scal, t, first);
   if (STEP == kSumActive) cg_active(scal, t, tol2, N);
+}
+
+// The CG vector kernels take one load case per blockIdx.y (3 planes a thread): six times the
+// blocks of a thread for all 18 planes, whose loads a small cell waits for one plane after
+// another (16^3: 12 to 17 us a kernel). A case's sums keep their order and their block: row
+// blockIdx.x of the partials holds the 6 dots, then the 18 plane sums.
+constexpr int kCgSums = kCases + kPlanes;
+
+// Block sums of (dot, 3 plane sums) of case c into their slots of partial row blockIdx.x.
+__device__ __forceinline__ void case_sums_store(const float (&v)[4], int c, double* part) {
+  __shared__ float sh[32][4];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int nw = (blockDim.x + 31) >> 5;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    float s = v[k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) sh[wid][k] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x < 4) {
+    const int k = threadIdx.x;
+    double s = 0.0;
+    for (int w = 0; w < nw; ++w) s += static_cast<double>(sh[w][k]);
+    part[static_cast<size_t>(blockIdx.x) * kCgSums + (k == 0 ? c : kCases + 3 * c + k - 1)] = s;
+  }
 }
 
 // Per case c: sum over the 3 planes of case c of a*b. Each thread takes W consecutive
@@ -159,31 +197,36 @@ __global__ void __launch_bounds__(256) k_dot6(const float* __restrict__ a,
 }
 
 // (r_c - mean r, z_c) for the 6 cases and the 18 plane sums of z (for removing its mean).
-// rmean: 18 plane means of r (doubles), or null.
+// rmean: 18 plane means of r, or null.
 template <int W>
 __global__ void __launch_bounds__(256) k_dot6_zsum(const float* __restrict__ r,
                                                    const float* __restrict__ z, size_t N,
-                                                   const double* __restrict__ rmean,
+                                                   const float* __restrict__ rmean,
                                                    double* __restrict__ part) {
-  float red[kCases + kPlanes], rm[kPlanes];
+  const int c = blockIdx.y;
+  float red[4] = {0.f, 0.f, 0.f, 0.f}, rm[3];
 #pragma unroll
-  for (int c = 0; c < kCases + kPlanes; ++c) red[c] = 0.f;
-#pragma unroll
-  for (int q = 0; q < kPlanes; ++q) rm[q] = rmean ? static_cast<float>(rmean[q]) : 0.f;
+  for (int k = 0; k < 3; ++k) rm[k] = rmean ? __ldg(rmean + 3 * c + k) : 0.f;
+  r += 3 * c * N;
+  z += 3 * c * N;
   for (size_t i = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < N / W;
        i += static_cast<size_t>(gridDim.x) * blockDim.x) {
     const size_t v = i * W;
+    Pk<W> zz[3], rr[3];
 #pragma unroll
-    for (int q = 0; q < kPlanes; ++q) {
-      const Pk<W> zz = ldg_pk<W>(z + q * N + v), rr = ldg_pk<W>(r + q * N + v);
+    for (int k = 0; k < 3; ++k) {
+      zz[k] = ldg_pk<W>(z + k * N + v);
+      rr[k] = ldg_pk<W>(r + k * N + v);
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
 #pragma unroll
       for (int w = 0; w < W; ++w) {
-        red[q / 3] = fmaf(rr.v[w] - rm[q], zz.v[w], red[q / 3]);
-        red[kCases + q] += zz.v[w];
+        red[0] = fmaf(rr[k].v[w] - rm[k], zz[k].v[w], red[0]);
+        red[1 + k] += zz[k].v[w];
       }
-    }
   }
-  block_sum_store<kCases + kPlanes>(red, part);
+  case_sums_store(red, c, part);
 }
 
 // e += alpha p, e kept in double-float (e + elo): the product is split exactly (its
@@ -191,52 +234,62 @@ __global__ void __launch_bounds__(256) k_dot6_zsum(const float* __restrict__ r,
 // transformations, so the correction carries no FP32 rounding noise; K applied to such
 // noise would be amplified by the operator's spread of eigenvalues and leave the true
 // residual far above the recursive one. r -= alpha (q - mean q) in FP32. Partial sums of
-// ||r_c||^2 and of the 18 plane sums of r.
+// ||r_c||^2 and of the 18 plane sums of r. s: the FP32 scalars (SlotF).
 template <int W>
 __global__ void __launch_bounds__(256) k_cg_update_er(float* __restrict__ e, float* __restrict__ elo,
                                                       float* __restrict__ r,
                                                       const float* __restrict__ p,
                                                       const float* __restrict__ q,
-                                                      const double* __restrict__ s, size_t N,
+                                                      const float* __restrict__ s, size_t N,
                                                       double* __restrict__ part) {
-  float a[kCases];
+  const int c = blockIdx.y;
+  const float a = __ldg(s + F_ALPHA + c);
+  float red[4] = {0.f, 0.f, 0.f, 0.f}, qm[3];
 #pragma unroll
-  for (int c = 0; c < kCases; ++c) a[c] = static_cast<float>(s[S_ALPHA + c]);
-  float red[kCases + kPlanes], qm[kPlanes];
-#pragma unroll
-  for (int c = 0; c < kCases + kPlanes; ++c) red[c] = 0.f;
-#pragma unroll
-  for (int k = 0; k < kPlanes; ++k) qm[k] = static_cast<float>(s[S_QSUM + k] / static_cast<double>(N));
+  for (int k = 0; k < 3; ++k) qm[k] = __ldg(s + F_QMEAN + 3 * c + k);
+  e += 3 * c * N;
+  elo += 3 * c * N;
+  r += 3 * c * N;
+  p += 3 * c * N;
+  q += 3 * c * N;
   for (size_t i = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < N / W;
        i += static_cast<size_t>(gridDim.x) * blockDim.x) {
     const size_t v = i * W;
+    Pk<W> rv[3];
 #pragma unroll
-    for (int k = 0; k < kPlanes; ++k) {
-      const int c = k / 3;
-      const size_t o = static_cast<size_t>(k) * N + v;
-      Pk<W> rv = ld_pk<W>(r + o);
-      if (a[c] != 0.f) {
-        const Pk<W> pv = ldg_pk<W>(p + o), qv = ldg_pk<W>(q + o);
-        Pk<W> hi = ld_pk<W>(e + o), lo = ld_pk<W>(elo + o);
+    for (int k = 0; k < 3; ++k) rv[k] = ld_pk<W>(r + k * N + v);
+    if (a != 0.f) {
+      Pk<W> pv[3], qv[3], hi[3], lo[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        pv[k] = ldg_pk<W>(p + k * N + v);
+        qv[k] = ldg_pk<W>(q + k * N + v);
+        hi[k] = ld_pk<W>(e + k * N + v);
+        lo[k] = ld_pk<W>(elo + k * N + v);
+      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
 #pragma unroll
         for (int w = 0; w < W; ++w) {
-          const float pr = __fmul_rn(a[c], pv.v[w]);        // TwoProd: pr + pe = a p exactly
-          const float pe = fmaf(a[c], pv.v[w], -pr);
-          df_add(hi.v[w], lo.v[w], pr, pe);
-          rv.v[w] = fmaf(-a[c], qv.v[w] - qm[k], rv.v[w]);
+          const float pr = __fmul_rn(a, pv[k].v[w]);        // TwoProd: pr + pe = a p exactly
+          const float pe = fmaf(a, pv[k].v[w], -pr);
+          df_add(hi[k].v[w], lo[k].v[w], pr, pe);
+          rv[k].v[w] = fmaf(-a, qv[k].v[w] - qm[k], rv[k].v[w]);
         }
-        st_pk<W>(e + o, hi);
-        st_pk<W>(elo + o, lo);
-        st_pk<W>(r + o, rv);
-      }
-#pragma unroll
-      for (int w = 0; w < W; ++w) {
-        red[c] = fmaf(rv.v[w], rv.v[w], red[c]);
-        red[kCases + k] += rv.v[w];
+        st_pk<W>(e + k * N + v, hi[k]);
+        st_pk<W>(elo + k * N + v, lo[k]);
+        st_pk<W>(r + k * N + v, rv[k]);
       }
     }
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        red[0] = fmaf(rv[k].v[w], rv[k].v[w], red[0]);
+        red[1 + k] += rv[k].v[w];
+      }
   }
-  block_sum_store<kCases + kPlanes>(red, part);
+  case_sums_store(red, c, part);
 }
 
 // (u + ulo) += (e + elo) in double-float arithmetic (error-free transformations with
@@ -262,33 +315,33 @@ __global__ void __launch_bounds__(256) k_fold(float* __restrict__ u, float* __re
   }
 }
 
-// p = (z - mean(z)) + beta p per plane.
+// p = (z - mean(z)) + beta p per plane. s: the FP32 scalars (SlotF).
 template <int W>
 __global__ void __launch_bounds__(256) k_cg_update_p(float* __restrict__ p,
                                                      const float* __restrict__ z,
-                                                     const double* __restrict__ s, size_t N) {
-  float b[kCases], mz[kPlanes];
+                                                     const float* __restrict__ s, size_t N) {
+  const int c = blockIdx.y;
+  const float b = __ldg(s + F_BETA + c);
+  float mz[3];
 #pragma unroll
-  for (int c = 0; c < kCases; ++c) b[c] = static_cast<float>(s[S_BETA + c]);
-#pragma unroll
-  for (int k = 0; k < kPlanes; ++k) mz[k] = static_cast<float>(s[S_ZSUM + k] / static_cast<double>(N));
+  for (int k = 0; k < 3; ++k) mz[k] = __ldg(s + F_ZMEAN + 3 * c + k);
+  p += 3 * c * N;
+  z += 3 * c * N;
   for (size_t i = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < N / W;
        i += static_cast<size_t>(gridDim.x) * blockDim.x) {
     const size_t v = i * W;
+    Pk<W> zz[3], pp[3];
 #pragma unroll
-    for (int k = 0; k < kPlanes; ++k) {
-      const size_t o = static_cast<size_t>(k) * N + v;
-      const Pk<W> zz = ldg_pk<W>(z + o);
-      Pk<W> pp;
-      if (b[k / 3] != 0.f) {
-        pp = ld_pk<W>(p + o);
+    for (int k = 0; k < 3; ++k) {
+      zz[k] = ldg_pk<W>(z + k * N + v);
+      if (b != 0.f) pp[k] = ld_pk<W>(p + k * N + v);
+    }
 #pragma unroll
-        for (int w = 0; w < W; ++w) pp.v[w] = fmaf(b[k / 3], pp.v[w], zz.v[w] - mz[k]);
-      } else {
+    for (int k = 0; k < 3; ++k) {
 #pragma unroll
-        for (int w = 0; w < W; ++w) pp.v[w] = zz.v[w] - mz[k];
-      }
-      st_pk<W>(p + o, pp);
+      for (int w = 0; w < W; ++w)
+        pp[k].v[w] = b != 0.f ? fmaf(b, pp[k].v[w], zz[k].v[w] - mz[k]) : zz[k].v[w] - mz[k];
+      st_pk<W>(p + k * N + v, pp[k]);
     }
   }
 }
@@ -759,9 +812,9 @@ cudaError_t launch_sum_step(int step, const double* part, int nblk, double* scal
                             cudaStream_t s) {
   const int nv = kCases + kPlanes;
   if (step == kSumAlpha)
-    k_sum_partials<kSumAlpha><<<1, 256, 0, s>>>(part, nblk, nv, scal + S_PQ, scal, 0, 0.0, 0.0);
+    k_sum_partials<kSumAlpha><<<1, 256, 0, s>>>(part, nblk, nv, scal + S_PQ, scal, 0, 0.0, static_cast<double>(N));
   else if (step == kSumBeta)
-    k_sum_partials<kSumBeta><<<1, 256, 0, s>>>(part, nblk, nv, scal + S_RZ, scal, first, 0.0, 0.0);
+    k_sum_partials<kSumBeta><<<1, 256, 0, s>>>(part, nblk, nv, scal + S_RZ, scal, first, 0.0, static_cast<double>(N));
   else if (step == kSumActive)
     k_sum_partials<kSumActive><<<1, 256, 0, s>>>(part, nblk, nv, scal + S_RR, scal, 0, tol * tol, static_cast<double>(N));
   else
@@ -778,12 +831,12 @@ cudaError_t launch_dot6(const float* a, const float* b, size_t N, double* part, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_dot6_zsum(const float* r, const float* z, size_t N, const double* rmean,
+cudaError_t launch_dot6_zsum(const float* r, const float* z, size_t N, const float* rmean,
                              double* part, int* grid_out, cudaStream_t s) {
   const int g = grid_for(N % 4 == 0 ? N / 4 : N, 256);
   *grid_out = g;
-  if (N % 4 == 0) k_dot6_zsum<4><<<g, 256, 0, s>>>(r, z, N, rmean, part);
-  else k_dot6_zsum<1><<<g, 256, 0, s>>>(r, z, N, rmean, part);
+  if (N % 4 == 0) k_dot6_zsum<4><<<dim3(g, kCases), 256, 0, s>>>(r, z, N, rmean, part);
+  else k_dot6_zsum<1><<<dim3(g, kCases), 256, 0, s>>>(r, z, N, rmean, part);
   return cudaGetLastError();
 }
 
@@ -792,8 +845,9 @@ cudaError_t launch_cg_update_er(float* e, float* elo, float* r, const float* p, 
                                 cudaStream_t s) {
   const int g = grid_for(N % 4 == 0 ? N / 4 : N, 256);
   *grid_out = g;
-  if (N % 4 == 0) k_cg_update_er<4><<<g, 256, 0, s>>>(e, elo, r, p, q, scal, N, part);
-  else k_cg_update_er<1><<<g, 256, 0, s>>>(e, elo, r, p, q, scal, N, part);
+  const float* fs = reinterpret_cast<const float*>(scal + S_F32);
+  if (N % 4 == 0) k_cg_update_er<4><<<dim3(g, kCases), 256, 0, s>>>(e, elo, r, p, q, fs, N, part);
+  else k_cg_update_er<1><<<dim3(g, kCases), 256, 0, s>>>(e, elo, r, p, q, fs, N, part);
   return cudaGetLastError();
 }
 
@@ -805,8 +859,8 @@ cudaError_t launch_fold(float* u, float* ulo, float* e, float* elo, size_t n, cu
 
 cudaError_t launch_cg_update_p(float* p, const float* z, const double* scal, size_t N,
                                cudaStream_t s) {
-  if (N % 4 == 0) k_cg_update_p<4><<<grid_for(N / 4, 256), 256, 0, s>>>(p, z, scal, N);
-  else k_cg_update_p<1><<<grid_for(N, 256), 256, 0, s>>>(p, z, scal, N);
+  if (N % 4 == 0) k_cg_update_p<4><<<dim3(grid_for(N / 4, 256), kCases), 256, 0, s>>>(p, z, reinterpret_cast<const float*>(scal + S_F32), N);
+  else k_cg_update_p<1><<<dim3(grid_for(N, 256), kCases), 256, 0, s>>>(p, z, reinterpret_cast<const float*>(scal + S_F32), N);
   return cudaGetLastError();
 }
 
