@@ -14,6 +14,8 @@
 #include "dev_common.cuh"
 #include "stencil.cuh"
 
+#include <utility>
+
 namespace homo {
 
 namespace {
@@ -78,18 +80,96 @@ __global__ void __launch_bounds__(256) k_loads(const __grid_constant__ LoadParam
 }
 
 
+// The signed sums of moduli that the blocks A_d are products of: with F the axes where d is 0,
+// a block needs, for every subset g of F, the sum over the contributing elements (in the order
+// of t) of E_t times the signs of t along g. 8 corners need 1, 12 edges 2, 6 faces 4.
+constexpr int kDSums = 56;
+
+struct DBlocks {
+  float k[27][9];            // K0[0][|d|][r][c] with the signs d_a d_b of the axes where d is not 0
+  unsigned char o[27][4];    // which sum: diagonal, (0,1), (0,2), (1,2)
+};
+
+__host__ __device__ constexpr int dsum_slot(int d, int sub) {   // sub: bit k = sign along axis k
+  int base = 0;
+  for (int e = 0; e < d; ++e) {
+    const int f = (e % 3 == 1) + (e / 3 % 3 == 1) + (e / 9 == 1);
+    base += f == 3 ? 0 : 1 << f;
+  }
+  int pos = 0, bit = 0;
+  const int D[3] = {d % 3 - 1, d / 3 % 3 - 1, d / 9 - 1};
+  for (int k = 0; k < 3; ++k)
+    if (D[k] == 0) {
+      if (sub >> k & 1) pos |= 1 << bit;
+      ++bit;
+    }
+  return base + pos;
+}
+
+DBlocks make_dblocks(const KeParam& K) {
+  DBlocks B;
+  for (int d = 0; d < 27; ++d) {
+    const int D[3] = {d % 3 - 1, d / 3 % 3 - 1, d / 9 - 1};
+    const int m = (D[0] != 0 ? 1 : 0) + (D[1] != 0 ? 2 : 0) + (D[2] != 0 ? 4 : 0);
+    for (int r = 0; r < 3; ++r)
+      for (int c = 0; c < 3; ++c) {
+        float v = K.k[24 * r + 3 * m + c];
+        if (r != c) v *= static_cast<float>((D[r] != 0 ? D[r] : 1) * (D[c] != 0 ? D[c] : 1));
+        B.k[d][3 * r + c] = v;
+      }
+    const int ax[4][2] = {{0, 0}, {0, 1}, {0, 2}, {1, 2}};
+    for (int i = 0; i < 4; ++i) {
+      int sub = 0;
+      if (i > 0) sub = (D[ax[i][0]] == 0 ? 1 << ax[i][0] : 0) | (D[ax[i][1]] == 0 ? 1 << ax[i][1] : 0);
+      B.o[d][i] = static_cast<unsigned char>(d == 13 ? 0 : dsum_slot(d, sub));
+    }
+  }
+  return B;
+}
+
+constexpr int kTrueResThreads = 128;
+
+// Sum for block i / 8 and axes i % 8, if the block has it, stored with stride kTrueResThreads.
+template <int i>
+__device__ __forceinline__ void store_dsum(const float (&Et)[8], float* s) {
+  constexpr int d = i / 8, sub = i % 8, dx = d % 3 - 1, dy = d / 3 % 3 - 1, dz = d / 9 - 1;
+  if constexpr (d != 13 && !((sub & 1) && dx != 0) && !((sub & 2) && dy != 0) && !((sub & 4) && dz != 0)) {
+    constexpr int slot = dsum_slot(d, sub);
+    float acc = 0.f;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      const int a = t & 1, b = t >> 1 & 1, c = t >> 2;
+      if ((dx != 0 && a != (dx > 0)) || (dy != 0 && b != (dy > 0)) || (dz != 0 && c != (dz > 0))) continue;
+      const bool neg = ((sub & 1) && !a) != (((sub & 2) && !b) != ((sub & 4) && !c));
+      acc += neg ? -Et[t] : Et[t];
+    }
+    s[slot * kTrueResThreads] = acc;
+  }
+}
+
+template <int... i>
+__device__ __forceinline__ void store_dsums(const float (&Et)[8], float* s, std::integer_sequence<int, i...>) {
+  (store_dsum<i>(Et, s), ...);
+}
+
 // r = (b + blo) - K (u + ulo) evaluated in double-float arithmetic (difference form, products
 // and sums error-free up to the final rounding), then partials of ||r_c||^2 and of the
 // 18 plane sums. This is the accurate true residual the CG driver restarts from; it uses
 // exactly the FP32 blocks A_d of the CG product, so both see the same operator.
-__global__ void __launch_bounds__(128) k_fine_true_residual(const __grid_constant__ KeParam K,
-                                                            const float* __restrict__ E,
-                                                            const float* __restrict__ u,
-                                                            const float* __restrict__ ulo,
-                                                            const float* __restrict__ b,
-                                                            const float* __restrict__ blo,
-                                                            float* __restrict__ out, int n,
-                                                            double* __restrict__ part) {
+//
+// Bound by the FMA pipe (69 % busy with 12 warps an SM): 369 two-lane operations per neighbour,
+// two cycles each. Around them a block costs 4 shared loads (its signed sums, formed once per
+// vertex) and 9 products with uniform constants; rebuilt from the 8 moduli at a runtime d it
+// took as many instructions as a third of the arithmetic. 160^3: 3.52 -> 3.27 ms.
+__global__ void __launch_bounds__(kTrueResThreads) k_fine_true_residual(const __grid_constant__ DBlocks B,
+                                                                     const float* __restrict__ E,
+                                                                     const float* __restrict__ u,
+                                                                     const float* __restrict__ ulo,
+                                                                     const float* __restrict__ b,
+                                                                     const float* __restrict__ blo,
+                                                                     float* __restrict__ out, int n,
+                                                                     double* __restrict__ part) {
+  __shared__ float ssum[kDSums][kTrueResThreads];   // each thread its own column
   const size_t N = static_cast<size_t>(n) * n * n;
   float red[kCases + kPlanes];
 #pragma unroll
@@ -99,8 +179,11 @@ __global__ void __launch_bounds__(128) k_fine_true_residual(const __grid_constan
     int x, y, z;
     decode3(static_cast<unsigned>(v), static_cast<unsigned>(n), x, y, z);
     const Nb nb = make_nb(x, y, z, n);
-    float Et[8];
-    load_E8(E, nb, Et);
+    {
+      float Et[8];
+      load_E8(E, nb, Et);
+      store_dsums(Et, &ssum[0][threadIdx.x], std::make_integer_sequence<int, 27 * 8>{});
+    }
     // The 6 cases advance in pairs (2p, 2p + 1) on the two lanes of f32x2 registers. Every
     // lane performs exactly the scalar operations of the double-float recurrence below,
     // in the same order (the negated-operand forms are exact: round to nearest is
@@ -109,6 +192,7 @@ __global__ void __launch_bounds__(128) k_fine_true_residual(const __grid_constan
     //   p = a dh, pe = a dh - p (FMA), hi + e' = hi + p (two-sum),
     //   lo += e' + (a dl + pe).
     f32x2 hi[9], lo[9], nown[9], ownlo[9];
+    const unsigned v32 = static_cast<unsigned>(v);
 #pragma unroll
     for (int p = 0; p < 3; ++p)
 #pragma unroll
@@ -116,37 +200,40 @@ __global__ void __launch_bounds__(128) k_fine_true_residual(const __grid_constan
         const int q0 = 6 * p + k, q1 = q0 + 3;
         hi[3 * p + k] = 0ull;
         lo[3 * p + k] = 0ull;
-        nown[3 * p + k] = pack2(-__ldg(u + q0 * N + v), -__ldg(u + q1 * N + v));
-        ownlo[3 * p + k] = pack2(__ldg(ulo + q0 * N + v), __ldg(ulo + q1 * N + v));
+        nown[3 * p + k] = pack2(-__ldg(u + q0 * N + v32), -__ldg(u + q1 * N + v32));
+        ownlo[3 * p + k] = pack2(__ldg(ulo + q0 * N + v32), __ldg(ulo + q1 * N + v32));
       }
 #pragma unroll 1
     for (int d = 0; d < 27; ++d) {
       if (d == 13) continue;
-      const int dx = d % 3 - 1, dy = (d / 3) % 3 - 1, dz = d / 9 - 1;
-      float A[9];
-      // runtime d: the block is rebuilt with runtime offsets (same FP32 operations and
-      // order as the compile-time version in the CG product)
-      nb_block(K, Et, dx, dy, dz, A);
+      const int rx = d % 3, ry = (d / 3) % 3, rz = d / 9;
+      const int yz = (ry == 0 ? nb.Y[0] : (ry == 1 ? nb.Y[1] : nb.Y[2])) +
+                     (rz == 0 ? nb.Z[0] : (rz == 1 ? nb.Z[1] : nb.Z[2]));
+      const float s0 = ssum[B.o[d][0]][threadIdx.x], s01 = ssum[B.o[d][1]][threadIdx.x],
+                  s02 = ssum[B.o[d][2]][threadIdx.x], s12 = ssum[B.o[d][3]][threadIdx.x];
+      const float* C = B.k[d];
+      const float A[9] = {C[0] * s0,  C[1] * s01, C[2] * s02, C[3] * s01, C[4] * s0,
+                          C[5] * s12, C[6] * s02, C[7] * s12, C[8] * s0};
       f32x2 Ap[9], An[9];
 #pragma unroll
       for (int e = 0; e < 9; ++e) {
         Ap[e] = pack2(A[e], A[e]);
         An[e] = pack2(-A[e], -A[e]);
       }
-      const size_t w = static_cast<size_t>(nb.X[dx + 1] + nb.Y[dy + 1] + nb.Z[dz + 1]);
+      const unsigned w = static_cast<unsigned>((rx == 0 ? nb.X[0] : (rx == 1 ? nb.X[1] : nb.X[2])) + yz);
 #pragma unroll
       for (int p = 0; p < 3; ++p) {
         f32x2 dh[3], dl[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-          const size_t o0 = static_cast<size_t>(6 * p + k) * N + w, o1 = o0 + 3 * N;
-          const f32x2 a = pack2(__ldg(u + o0), __ldg(u + o1));
+          const size_t q0 = static_cast<size_t>(6 * p + k) * N, q1 = q0 + 3 * N;
+          const f32x2 a = pack2(__ldg(u + q0 + w), __ldg(u + q1 + w));
           const f32x2 b = nown[3 * p + k];
           const f32x2 s = fadd2(a, b);                      // two-sum of u_(v+d) and -u_v
           const f32x2 bb = fsub2(s, a);
           const f32x2 e = fadd2(fsub2(a, fsub2(s, bb)), fsub2(b, bb));
           dh[k] = s;
-          dl[k] = fadd2(e, fsub2(pack2(__ldg(ulo + o0), __ldg(ulo + o1)), ownlo[3 * p + k]));
+          dl[k] = fadd2(e, fsub2(pack2(__ldg(ulo + q0 + w), __ldg(ulo + q1 + w)), ownlo[3 * p + k]));
         }
 #pragma unroll
         for (int r = 0; r < 3; ++r)
@@ -281,7 +368,7 @@ __host__ __device__ constexpr int pair_slot(int i, int j) {
 // the parameter bank) and every instruction then serves two elements, where
 // the scalar form spent an instruction per constant as well (1700 a thread and element, 850
 // of them FMA-pipe). The rows of y come in two halves of 12, which keeps the registers
-// at 2 blocks per SM. 192^3, C^H and sensitivities together: 5.27 -> 5.1 ms.
+// at 2 blocks per SM. 192^3, C^H and sensitivities together: 5.27 -> 4.85 ms.
 // MODE 0: block partial sums of E_e q_ij (21 values, Kahan-compensated per thread).
 // MODE 1: sensitivity (Eq. 8-9) p rho^(p-1) dE sum_ij g_ij q_ij / N, evaluated as
 // sum_k mu_k z_k^T K0 z_k with G = sym(g) = sum_k mu_k v_k v_k^T and z_k = sum_i v_k[i] w_i
@@ -454,16 +541,17 @@ cudaError_t launch_loads(const homo_ctx* c, float* f) {
 
 cudaError_t launch_fine_apply(const homo_ctx* c, const float* u, float* out, double* part,
                               int* grid_out) {
-  return launch_fine_tiled(c, 1, u, nullptr, out, part, grid_out);
+  return launch_fine_tiled(c, part ? 1 : 7, u, nullptr, out, part, grid_out);
 }
 
 cudaError_t launch_fine_residual(const homo_ctx* c, const float* b, const float* u,
                                  const float* ulo, float* out, double* part, int* grid_out,
                                  const float* bmean) {
   if (ulo) {
-    const int g = grid_for(c->N, 128);
+    const int g = grid_for(c->N, kTrueResThreads);
     if (grid_out) *grid_out = g;
-    k_fine_true_residual<<<g, 128, 0, c->stream>>>(c->ke, c->E, u, ulo, b, c->flo, out, c->n, part);
+    k_fine_true_residual<<<g, kTrueResThreads, 0, c->stream>>>(make_dblocks(c->ke), c->E, u, ulo, b, c->flo, out, c->n,
+                                                               part);
     return cudaGetLastError();
   }
   return launch_fine_tiled(c, 3, u, b, out, nullptr, grid_out, bmean);

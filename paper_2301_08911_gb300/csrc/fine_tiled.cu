@@ -107,6 +107,7 @@ __device__ __forceinline__ void load_pairs(const float* site, f32x2 (&pr)[9]) {
 
 // MODE 1: out = K u in difference form (sum_d A_d (u_(v+d) - u_v)) with partials of the
 //         dots (u_c, out_c) and the 18 plane sums of out (the CG product);
+// MODE 7: the same product without the partials (homo_apply_K);
 // MODE 2: out = b - K (u + ulo) in difference form, each neighbour difference formed from
 //         the high and the low parts, (u_(v+d) - u_v) + (ulo_(v+d) - ulo_v), with partials of
 //         ||out_c||^2 and the 18 plane sums of out (the true residual of a double-float
@@ -157,12 +158,14 @@ __global__ void __launch_bounds__(kTiledThreads, MODE == 2 ? 1 : 2)
   cp_async_commit();
 
   for (int z = z0; z < z1; ++z) {
-    // prefetch u plane z+2 and modulus plane z+1 (their slots were released at the end
-    // of the previous step)
-    issue_u_plane(u, N, static_cast<size_t>(wrapi(z + 2, n)) * nn, s, su + ((z + 2) & 3) * kUPlaneFloats);
-    if (kLo)
-      issue_u_plane(ulo, N, static_cast<size_t>(wrapi(z + 2, n)) * nn, s, sl + ((z + 2) & 3) * kUPlaneFloats);
-    issue_e_plane(E, static_cast<size_t>(wrapi(z + 1, n)) * nn, s, se + ((z + 1) % kESlots) * EPLANE);
+    // prefetch u plane z+2 and modulus plane z+1 for the next step, if there is one (their
+    // slots were released at the end of the previous step)
+    if (z + 1 < z1) {
+      issue_u_plane(u, N, static_cast<size_t>(wrapi(z + 2, n)) * nn, s, su + ((z + 2) & 3) * kUPlaneFloats);
+      if (kLo)
+        issue_u_plane(ulo, N, static_cast<size_t>(wrapi(z + 2, n)) * nn, s, sl + ((z + 2) & 3) * kUPlaneFloats);
+      issue_e_plane(E, static_cast<size_t>(wrapi(z + 1, n)) * nn, s, se + ((z + 1) % kESlots) * EPLANE);
+    }
     cp_async_commit();
     cp_async_wait1();
     __syncthreads();
@@ -176,7 +179,7 @@ __global__ void __launch_bounds__(kTiledThreads, MODE == 2 ? 1 : 2)
       for (int t = 0; t < 8; ++t)
         Et[t] = ((t >> 2) ? e0 : em)[(ty + ((t >> 1) & 1)) * EX + tx + (t & 1)];
       const int cidx = (ty + 1) * HX + tx + 1;
-      constexpr bool kDiff = MODE == 1 || MODE == 2;
+      constexpr bool kDiff = MODE == 1 || MODE == 2 || MODE == 7;
       // the 6 cases advance in pairs (2p, 2p + 1) on the two lanes of f32x2 registers;
       // every lane is rounded as the scalar chain in the same order would be
       constexpr int kPairs = kCases / 2;
@@ -256,13 +259,13 @@ __global__ void __launch_bounds__(kTiledThreads, MODE == 2 ? 1 : 2)
           out[o] = val;
           if (MODE == 1) red[q / 3] = fmaf(own1[kDiff ? q : 0], val, red[q / 3]);
           if (MODE == 2) red[q / 3] = fmaf(val, val, red[q / 3]);
-          if (kDiff) red[kCases + q] += val;
+          if (MODE == 1 || MODE == 2) red[kCases + q] += val;
         }
       }
     }
     __syncthreads();
   }
-  if ((MODE == 1 || MODE == 2) && part != nullptr) {
+  if (MODE == 1 || MODE == 2) {
     // block_sum_store writes row blockIdx.x; shift the base to the flattened 3-D index
     const size_t flat = (static_cast<size_t>(blockIdx.z) * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
     block_sum_store<kCases + kPlanes>(red, part + (flat - blockIdx.x) * (kCases + kPlanes));
@@ -275,6 +278,19 @@ int tiled_zchunk(int n) {
   int chunk = n;
   while (chunk > 4 && xy * ((n + chunk - 1) / chunk) < 152L * 2 * 8) chunk = (chunk + 1) / 2;
   return chunk;
+}
+
+// Planes per block where nothing is summed (the chunks of the dots are part of their rounding).
+// A block's first planes cost little (its neighbour's last ones, from L2), so short chunks
+// that even the SMs out win until there are some ten rounds of long ones. Product with 1 / 2 /
+// 8 / 16 planes: 16^3 9 / 13 / 33 / 60 us, 128^3 250 / 228 / 238 / 267, 160^3 - / 446 / 479 / 478,
+// 256^3 1941 / 1738 / 1775 / 1733.
+// Product before, with the chunks of the dots and the dots: 16^3 19 us, 128^3 242 us, 320^3 3.83 ms;
+// now 9 us, 228 us, 3.54 ms.
+int tiled_zchunk_free(int n) {
+  const long xy = static_cast<long>((n + TX - 1) / TX) * ((n + TY - 1) / TY);
+  if (xy * ((n + 15) / 16) >= 4096) return 16;
+  return xy * ((n + 1) / 2) >= 1216 ? 2 : 1;
 }
 
 }  // namespace
@@ -312,6 +328,7 @@ cudaError_t tiled_init() {
   if (e == cudaSuccess) e = tiled_attr<4>();
   if (e == cudaSuccess) e = tiled_attr<5>();
   if (e == cudaSuccess) e = tiled_attr<6>();
+  if (e == cudaSuccess) e = tiled_attr<7>();
   return e;
 }
 
@@ -319,18 +336,21 @@ cudaError_t launch_fine_tiled(const homo_ctx* c, int mode, const float* u, const
                               double* part, int* grid_out, const float* bmean, float c0, float c1,
                               const float* ulo) {
   const int n = c->n;
-  const int zc = tiled_zchunk(n);
+  const int zc = mode == 1 || mode == 2 ? tiled_zchunk(n) : tiled_zchunk_free(n);
   dim3 grid((n + TX - 1) / TX, (n + TY - 1) / TY, (n + zc - 1) / zc);
   if (grid_out) *grid_out = static_cast<int>(grid.x * grid.y * grid.z);
   switch (mode) {
-    case 1: return run_tiled<1>(c, grid, zc, u, nullptr, nullptr, out, part, nullptr, 0.f, 0.f);
+    case 1:
+      if (!part) return cudaErrorInvalidValue;
+      return run_tiled<1>(c, grid, zc, u, nullptr, nullptr, out, part, nullptr, 0.f, 0.f);
     case 2:
-      if (!ulo) return cudaErrorInvalidValue;
+      if (!ulo || !part) return cudaErrorInvalidValue;
       return run_tiled<2>(c, grid, zc, u, ulo, b, out, part, nullptr, 0.f, 0.f);
     case 3: return run_tiled<3>(c, grid, zc, u, nullptr, b, out, nullptr, bmean, 0.f, 0.f);
     case 4: return run_tiled<4>(c, grid, zc, u, nullptr, b, out, nullptr, bmean, c0, c1);
     case 5: return run_tiled<5>(c, grid, zc, u, nullptr, b, out, nullptr, bmean, c0, c1);
     case 6: return run_tiled<6>(c, grid, zc, u, nullptr, b, out, nullptr, bmean, c0, c1);
+    case 7: return run_tiled<7>(c, grid, zc, u, nullptr, nullptr, out, nullptr, nullptr, 0.f, 0.f);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -221,7 +221,7 @@ cudaError_t launch_loads(const homo_ctx* c, float* f);
 // dots (u_c, out_c) and the 18 plane sums of out (24 doubles per block; *grid_out blocks).
 cudaError_t launch_fine_apply(const homo_ctx* c, const float* u, float* out, double* part,
                               int* grid_out);
-// tiled finest-level stencil (fine_tiled.cu): mode 1 = launch_fine_apply; 2 = b - K (u + ulo)
+// tiled finest-level stencil (fine_tiled.cu): modes 1, 7 = launch_fine_apply; 2 = b - K (u + ulo)
 // in difference form from both parts, with norms (FP32 true residual); 3 = (b - bmean) - K u;
 // 4 = u + c0 S^-1 (b - bmean - K u); 5 = u + c0 (u - out) + c1 S^-1 (b - bmean - K u), in
 // place on out; 6 = (1 + c0) u + c1 S^-1 (b - bmean - K u) (Chebyshev steps)
