@@ -109,3 +109,79 @@ def test_blocked_coarsest_inverse_inverts_K(B, n):
     torch.cuda.synchronize()
     assert ((back - r).norm() / r.norm()).item() < 6e-5
     assert z.reshape(18, -1).double().mean(dim=1).abs().max().item() < 1e-6 * z.abs().max().item()
+
+
+def apply_stencil(st, u):
+    """FP64 sum_d A_d u(v + d) of a level's stencil (z, y, x, 27, 9) on (6, 3, z, y, x) fields."""
+    n = st.shape[0]
+    out = torch.zeros_like(u)
+    for d in range(27):
+        s = (-(d // 9 - 1), -((d // 3) % 3 - 1), -(d % 3 - 1))
+        A = st[..., d, :].double().view(n, n, n, 3, 3)
+        out += torch.einsum("zyxrc,kczyx->krzyx", A, torch.roll(u, s, dims=(2, 3, 4)))
+    return out
+
+
+def bf16_stencil(st):
+    """The stored BF16 stencil: each block averaged with its transposed counterpart, then rounded."""
+    n, out = st.shape[0], torch.empty_like(st)
+    for d in range(27):
+        s = (-(d // 9 - 1), -((d // 3) % 3 - 1), -(d % 3 - 1))
+        other = torch.roll(st[..., 26 - d, :], s, dims=(0, 1, 2)).view(n, n, n, 3, 3).transpose(-1, -2)
+        out[..., d, :] = (0.5 * (st[..., d, :] + other.reshape(n, n, n, 9))).bfloat16().float()
+    return out
+
+
+@pytest.mark.parametrize("n,level", [(40, 1), (48, 1), (56, 1), (112, 2), (224, 1)])
+def test_staged_coarse_sweep_matches_its_stencil(B, n, level):
+    """Levels 20, 24, 28 and 112: stencil rows of one tile and a ragged one, shorter than a warp's
+    vertices and both tile splits (<= 96 and above), both stencil precisions and colour
+    orders, two sweeps in a row (the second chained to the first), against an FP64 sweep with the
+    same stencil. Bound 2e-6 a sweep, as for one sweep of any coarse form against the oracle."""
+    nl = n >> level
+    rho = cuda(uniform_density(n, 730 + n, 0.05, 1.0))
+    f, u0 = cuda(uniform_field(18 * nl ** 3, 731, -1, 1)), cuda(uniform_field(18 * nl ** 3, 732, -1, 1))
+    hom = B.Homogenization(n)
+    hom.set_density(rho)
+    st = torch.empty(nl ** 3 * 243, device="cuda")
+    hom.get_stencil(level, st)
+    st = st.view(nl, nl, nl, 27, 9)
+    ax = torch.arange(nl, device="cuda") & 1
+    colour = ax[None, None, :] + 2 * ax[None, :, None] + 4 * ax[:, None, None]
+    for precision in ("fp32", "mixed"):
+        if precision == "mixed":
+            hom = B.Homogenization(n, precision=precision)
+            hom.set_density(rho)
+            st = bf16_stencil(st)
+        S = st[..., 13, :].double().view(nl, nl, nl, 3, 3)
+        for reverse in (False, True):
+            u = u0.clone()
+            for _ in range(2):
+                hom.smooth(level, reverse, f, u)
+            ref = u0.double().view(6, 3, nl, nl, nl).clone()
+            fd = f.double().view_as(ref)
+            for _ in range(2):
+                for k in range(8):
+                    r = fd - apply_stencil(st, ref)
+                    du = torch.linalg.solve(S, r.permute(2, 3, 4, 1, 0)).permute(4, 3, 0, 1, 2)
+                    ref += du * (colour == (7 - k if reverse else k))
+            err = u.double().view_as(ref) - ref
+            assert (err.norm() / ref.norm()).item() < 4e-6, (precision, reverse)
+            assert (err.abs().max() / ref.abs().max()).item() < 4e-6, (precision, reverse)
+
+
+@pytest.mark.parametrize("n", [4, 16, 20, 40, 80, 112])
+def test_product_over_chunk_sizes(B, n):
+    """One and two planes a block, ragged tiles in x and y, against the level's own stencil in
+    FP64: 2e-6 of the terms each output sums, as against the oracle."""
+    hom = B.Homogenization(n)
+    hom.set_density(cuda(uniform_density(n, 740 + n, 0.05, 1.0)))
+    u = cuda(uniform_field(18 * n ** 3, 741, -1, 1))
+    out = torch.empty_like(u)
+    hom.apply_K(u, out)
+    st = torch.empty(n ** 3 * 243, device="cuda")
+    hom.get_stencil(0, st)
+    st = st.view(n, n, n, 27, 9)
+    ud = u.double().view(6, 3, n, n, n)
+    err = (out.double().view_as(ud) - apply_stencil(st, ud)).abs()
+    assert torch.all(err <= 2e-6 * apply_stencil(st.abs(), ud.abs()))
