@@ -421,7 +421,8 @@ def coarse_forms(hom, n, stream, dev):
     return {"sweep_us": sweep, "vcycle_ms": vc,
             "settings": "resident_max_n,cluster_max_n,split_max_n; library default " + ",".join(map(str, saved)),
             "note": "one homo_smooth sweep per level and form (the resident form times its shared-memory setup "
-                    "once per sweep; inside a V-cycle it runs many sweeps per launch), then homo_vcycle"}
+                    "once per sweep; inside a V-cycle it runs many sweeps per launch), then homo_vcycle; levels "
+                    "above 16 that are a multiple of 4 run the staged kernel under every setting"}
 
 
 # ------------------------------------------------------------------ reference arm

@@ -380,7 +380,7 @@ int homo_prolong_add(homo_ctx* ctx, int level, const float* coarse, float* fine)
 int homo_set_tuning(homo_ctx* ctx, int gs_cases, int gs_block);
 int homo_autotune(homo_ctx* ctx, int flags, int* gs_cases, int* gs_block, double* ms);
 
-/* Coarse-level Gauss-Seidel kernels (Eq. 15-16 on levels >= 1). All four forms compute
+/* Coarse-level Gauss-Seidel kernels (Eq. 15-16 on levels >= 1). All forms compute
  * bitwise the same iterates; they differ in how the work reaches the GPU:
  *  - levels with at most resident_max_n cells per axis (up to 16^3, where the device launches
  *    clusters large enough): every sweep of one smoothing phase (the pre- or post-smoothing
@@ -390,6 +390,9 @@ int homo_autotune(homo_ctx* ctx, int flags, int* gs_cases, int* gs_block, double
  *    (half of them in shared memory at 14^3 and 16^3), and writes each update into the copies
  *    of the CTAs that read it; the colour passes are separated by the cluster's hardware
  *    barrier (default 16);
+ *  - other levels of more than 16 cells per axis, a multiple of 4: one launch per colour pass that
+ *    stages the stencil through shared memory while the pass before it runs, whatever the two
+ *    sizes below say;
  *  - other levels with at most cluster_max_n cells per axis: the same per-case cluster
  *    launch, reading the displacement and stencils through L2 (default 32);
  *  - larger levels with at most split_max_n cells per axis: one launch per colour pass with
@@ -398,7 +401,7 @@ int homo_autotune(homo_ctx* ctx, int flags, int* gs_cases, int* gs_block, double
  *  - larger levels: one launch per colour pass with a thread per vertex and all 6 cases.
  * The small levels are bound by load latency and launch overhead, not by bytes: with the
  * default sweep counts a V-cycle of a 512^3 cell runs about 2,500 colour passes on levels
- * of 32^3 and below. Sizes in [0, 1024]; 0 disables a form. Changing them drops the
+ * of 32^3 and below, 2,050 of them inside the launches of the first form. Sizes in [0, 1024]; 0 disables a form. Changing them drops the
  * context's captured CUDA graphs. Where the device cannot launch the clusters, the next
  * form applies whatever the sizes say. homo_coarse_smoother reports the sizes and the
  * largest cluster of the L2 and of the resident form the device launches (-1: none);

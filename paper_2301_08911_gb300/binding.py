@@ -354,7 +354,8 @@ class Homogenization:
 
     def set_coarse_smoother(self, resident_max_n: int, cluster_max_n: int, split_max_n: int):
         """Coarse Gauss-Seidel kernels by level size: at most resident_max_n cells per axis
-        smooth as one cluster launch per phase with the displacement in shared memory, at
+        smooth as one cluster launch per phase with the displacement in shared memory; larger
+        ones that are a multiple of 4 above 16 stage the stencil, a launch per colour; of the rest at
         most cluster_max_n as one cluster launch through L2, at most split_max_n with a
         thread per (vertex, case) per colour, larger levels with a thread per vertex
         (0 disables a form)."""

@@ -24,7 +24,7 @@
 // of math; measured 68 cycles each, back to back (two thirds of the time on operands at 64 B a
 // clock), so what counts is the share of rows that are outputs. 64^3, 32 -> 32 channels:
 // 70 -> 39 us with 30 x 4 x 2 tiles (four warps did all three in turn before, two CTAs per
-// SM: tensor pipe 14 % busy), 37 us with 32 x 11 x 1 (most of the rest a fixed 8 us of prologue and tail).
+// SM: tensor pipe 14 % busy), 37 us with 32 x 11 x 1.
 #include <cuda_bf16.h>
 
 #include <algorithm>
