@@ -450,7 +450,9 @@ __device__ __forceinline__ void pair_add(float& hi, float& lo, float v) {
   hi = s;
 }
 
-// Block sums of NV FP32 pairs into part[blockIdx.x * NV + k] (FP64 across the warps).
+// Block sums of NV FP32 pairs into part[blockIdx.x * NV + k] (FP64 across the warps). A high part
+// that is infinite stays so (it is the plain FP32 sum), but TwoSum then leaves inf - inf in the low
+// part, which does not count: the sum of a density with an infinite value is infinite, not NaN.
 template <int NV>
 __device__ __forceinline__ void pair_block_sum(float (&hi)[NV], float (&lo)[NV], double* part) {
   __shared__ float sh[kOcBlock / 32][NV], sl[kOcBlock / 32][NV];
@@ -473,7 +475,8 @@ __device__ __forceinline__ void pair_block_sum(float (&hi)[NV], float (&lo)[NV],
     double s = 0.0;
 #pragma unroll
     for (int w = 0; w < kOcBlock / 32; ++w)
-      s += static_cast<double>(sh[w][threadIdx.x]) + static_cast<double>(sl[w][threadIdx.x]);
+      s += static_cast<double>(sh[w][threadIdx.x]) +
+           (isinf(sh[w][threadIdx.x]) ? 0.0 : static_cast<double>(sl[w][threadIdx.x]));
     part[static_cast<size_t>(blockIdx.x) * NV + threadIdx.x] = s;
   }
 }
