@@ -305,8 +305,11 @@ __global__ void __launch_bounds__(kWgThreads, 1)
 }
 
 // dw[t][o][i] = sum over chunks of the partials, db[o] likewise: four threads per value sum a
-// quarter each in order as FP32 pairs (TwoSum: as exact as FP64 here, whose pipe the
-// one-thread FP64 sum left 71 % busy; 38 -> 12 us for 27,680 values), then the quarters.
+// quarter each in order as FP32 pairs (TwoSum), then the quarters. What is left of the error is the
+// rounding of the low parts' own FP32 sum, far below half a unit of the FP32 result. (A one-thread
+// FP64 sum kept the FP64 pipe 71 % busy: 38 -> 12 us for 27,680 values.) A pair has the range of
+// FP32: where a sum is not finite, by an infinite partial or because its high part left that range
+// on the way, the value is summed again in FP64.
 __global__ void __launch_bounds__(256) k_wgrad_reduce(int chunks, int per, const float* __restrict__ part,
                                                       const float* __restrict__ partb, float* __restrict__ dw,
                                                       float* __restrict__ db) {
@@ -335,7 +338,15 @@ __global__ void __launch_bounds__(256) k_wgrad_reduce(int chunks, int per, const
     add(sh[t][k]);
     lo = __fadd_rn(lo, sl[t][k]);
   }
-  (e < nw ? dw[e] : db[e - nw]) = __fadd_rn(hi, lo);
+  float sum = __fadd_rn(hi, lo);
+  if (!isfinite(sum)) {
+    const float* src = e < nw ? part + e : partb + (e - nw);
+    const size_t step = e < nw ? nw : kC;
+    double d = 0.0;
+    for (int c = 0; c < chunks; ++c) d += __ldg(src + c * step);
+    sum = static_cast<float>(d);
+  }
+  (e < nw ? dw[e] : db[e - nw]) = sum;
 }
 
 // x[v] = (rho, rho^2, rho^3, 0 ... 0) in BF16, 16 channels.
