@@ -527,18 +527,18 @@ int homo_nn_conv3d(int n, int c_in, const void* x, const void* w, const float* b
                    const void* mask, int epilogue, void* out, float* out_planes, const double* scale,
                    void* stream);
 
-/* The layer runs on the tcgen05 tensor cores: one thread per CTA issues the MMAs and the
- * CTA waits for their completion on an mbarrier with a bounded number of polls. Returns
- * the number of tile waits that ran out since the last call (0 in normal operation; the
- * outputs of such a tile are not written) and resets it; -1 if it cannot be read.
- * Synchronous (reads a device counter). */
+/* The layer runs on the tcgen05 tensor cores: a CTA's copy, MMA and epilogue warps hand tiles
+ * on through mbarriers, every wait with a bounded number of polls. Returns the number of CTAs
+ * in which a wait of any warp ran out since the last call (0 in normal operation; outputs of
+ * such a CTA's tiles from that one on may not be written) and resets it; -1 if it cannot be
+ * read. Synchronous (reads a device counter). */
 int homo_nn_tc_timeouts(void);
 
-/* Exercises that bounded wait on its own: launches `blocks` CTAs (1..1024) that wait on an
- * mbarrier nothing arrives on, each giving up after the same poll limit and counting one
- * timeout (read with homo_nn_tc_timeouts). No tensor-core work is issued. For failure-
- * detection tests; takes about a second (each CTA polls 2^18 times). Synchronises the
- * device. */
+/* Exercises that bounded wait on its own: launches `blocks` CTAs (1..1024) of the layer's 13
+ * warps; in CTA b warp b mod 13 waits on an mbarrier nothing arrives on and gives up after
+ * the same poll limit, so the CTA counts one timeout (read with homo_nn_tc_timeouts). No
+ * tensor-core work is issued. For failure-detection tests; takes about a second (each such
+ * warp polls 2^18 times). Synchronises the device. */
 int homo_nn_tc_wait_probe(int blocks);
 
 /* Weight and bias gradients of one layer: dw[t][o][i] = sum_v dy[v,o] x[wrap(v + d_t), i],

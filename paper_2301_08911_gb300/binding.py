@@ -478,12 +478,12 @@ def nn_conv3d(n: int, c_in: int, x, w, bias=None, res=None, mask=None, epilogue:
 
 
 def nn_tc_timeouts() -> int:
-    """Tensor-core convolution tiles whose completion wait ran out since the last call."""
+    """CTAs of tensor-core layers in which a wait ran out since the last call (resets the count)."""
     return load_library().homo_nn_tc_timeouts()
 
 
 def nn_tc_wait_probe(blocks: int = 4):
-    """Run the bounded mbarrier wait against a barrier nothing arrives on (timeouts counted)."""
+    """Let one warp of each of `blocks` CTAs (b mod 13 in CTA b) run out of its bounded wait."""
     _nn_check(load_library().homo_nn_tc_wait_probe(blocks), "homo_nn_tc_wait_probe")
 
 

@@ -75,7 +75,7 @@ struct TcScale {
   float s[6];
 };
 
-__device__ int g_conv_tc_timeouts = 0;   // tiles whose MMA completion wait ran out
+__device__ int g_conv_tc_timeouts = 0;   // CTAs in which a wait ran out
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -143,6 +143,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity) {
     if (done) return true;
   }
   return false;
+}
+
+// The verdict of the whole CTA (every thread calls it once its role is done): true when a wait of
+// any role and warp ran out, since each decides for itself; counted once per CTA.
+__device__ __forceinline__ bool cta_gave_up(bool ok) {
+  const bool any = __syncthreads_or(ok ? 0 : 1) != 0;
+  if (any && threadIdx.x == 0) atomicAdd(&g_conv_tc_timeouts, 1);
+  return any;
 }
 
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
@@ -279,6 +287,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   const uint32_t tmem = *tmem_slot;
+  bool ok = true;    // no wait of this thread's role ran out
+  int issued = 0;    // MMA warp: tiles whose MMAs were issued
 
   if (warp >= 8 && warp < 12) {
     // ---- copies: box rows t, t + 128, ... and all their chunks per thread
@@ -286,7 +296,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     int k = 0;
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++k) {
       const int st = k % kStages;
-      if (!mbar_wait(empty(st), ((k / kStages) & 1) ^ 1)) break;   // a fresh barrier passes parity 1
+      ok = mbar_wait(empty(st), ((k / kStages) & 1) ^ 1);   // a fresh barrier passes parity 1
+      if (!ok) break;
       const int tx = tile % tiles_x, rest = tile / tiles_x;
       const int x0 = tx * TL::TX, y0 = (rest % tiles_y) * TL::TY, z0 = (rest / tiles_y) * TL::TZ;
       const uint32_t dst = box_s + st * S::kBoxBytes;
@@ -313,11 +324,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t leader;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(leader));
     const uint64_t a0 = smem_desc(box_s, kPlaneBytes, 128), b0 = smem_desc(w_s, kC * 16, 128);
-    int k = 0;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++k) {
-      const int st = k % kStages, ac = k & 1;
-      const bool ok = mbar_wait(tempty(ac), ((k >> 1) & 1) ^ 1) && mbar_wait(full(st), (k / kStages) & 1);
-      if (!__all_sync(0xffffffffu, ok)) break;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++issued) {
+      const int k = issued, st = k % kStages, ac = k & 1;
+      ok = mbar_wait(tempty(ac), ((k >> 1) & 1) ^ 1) && mbar_wait(full(st), (k / kStages) & 1);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 #pragma unroll 1
       for (int unit = 0; unit < TL::kUnits; ++unit) {
@@ -350,7 +361,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int o = 0; o < 6; ++o) so[o] = sc.s[o];
     const bool has_res = (EPI == HOMO_NN_RELU || EPI == HOMO_NN_MASK) && res != nullptr;
     int k = 0;
-    bool ok = true;
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++k) {
       const int ac = k & 1;
       const int tx = tile % tiles_x, rest = tile / tiles_x;
@@ -385,31 +395,33 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       if (!ok) break;
     }
-    if (!ok && lane == 0) {
-      // give up on this tile and the rest; MMAs still running get one more bounded wait before
-      // the TMEM is freed (the other roles' waits then run out too)
-      if (warp == 0) atomicAdd(&g_conv_tc_timeouts, 1);
-      mbar_wait(tfull(k & 1), (k >> 1) & 1);
-    }
+    // a warp that gives up leaves this tile and the rest unwritten; the other roles' waits then run
+    // out too
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-  __syncthreads();
+  if (cta_gave_up(ok)) {
+    // MMAs of up to two tiles may still be running: one more bounded wait, on the last commit,
+    // which covers those before it, before the TMEM and the shared memory they use are freed
+    if (warp == 12 && issued > 0) mbar_wait(tfull((issued - 1) & 1), ((issued - 1) >> 1) & 1);
+    __syncthreads();
+  }
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(TL::kTmemCols) : "memory");
   }
 }
 
-// The bounded completion wait on an mbarrier that no one arrives on: every CTA gives up
-// after kWaitLimit polls and counts the timeout, the path a tile takes when its MMAs never
-// complete (no MMA is issued here, so nothing is left in flight).
-__global__ void k_wait_probe() {
+// The bounded wait and the CTA's verdict on their own: in CTA b one warp, b mod 13, waits on an
+// mbarrier that no one arrives on and gives up after kWaitLimit polls, the others' waits complete
+// at once; the CTA counts one timeout whichever warp it was (no MMA is issued here, so nothing is
+// left in flight).
+__global__ void __launch_bounds__(kThreads) k_wait_probe() {
   __shared__ __align__(8) uint64_t bar;
   const uint32_t b = smem_u32(&bar);
-  if (threadIdx.x == 0) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(b) : "memory");
+  if (threadIdx.x == 0) mbar_init(b, 1);
   __syncthreads();
-  const bool ok = mbar_wait(b, 0);
-  if (__syncthreads_or(!ok) && threadIdx.x == 0) atomicAdd(&g_conv_tc_timeouts, 1);
+  const bool stuck = threadIdx.x / 32 == blockIdx.x % (kThreads / 32);
+  cta_gave_up(mbar_wait(b, stuck ? 0 : 1));   // a fresh barrier passes parity 1
 }
 
 int g_sms = 0;
@@ -478,12 +490,12 @@ cudaError_t conv3d_tc(int n, int cin, int epi, const void* x, const void* w, con
 }
 
 cudaError_t conv3d_tc_wait_probe(int blocks) {
-  k_wait_probe<<<blocks, 32>>>();
+  k_wait_probe<<<blocks, kThreads>>>();
   const cudaError_t e = cudaGetLastError();
   return e != cudaSuccess ? e : cudaDeviceSynchronize();
 }
 
-// Number of tiles whose completion wait ran out since the last call (and reset it).
+// Number of CTAs in which a wait ran out since the last call (and reset it).
 int conv3d_tc_take_timeouts() {
   int h = 0;
   if (cudaMemcpyFromSymbol(&h, g_conv_tc_timeouts, sizeof(int)) != cudaSuccess) return -1;
