@@ -145,12 +145,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity) {
   return false;
 }
 
-// The verdict of the whole CTA (every thread calls it once its role is done): true when a wait of
-// any role and warp ran out, since each decides for itself; counted once per CTA.
-__device__ __forceinline__ bool cta_gave_up(bool ok) {
-  const bool any = __syncthreads_or(ok ? 0 : 1) != 0;
+// The CTA's closing barrier, which every thread reaches once its role is done: a wait that ran out
+// in any role and warp (each decides for itself) counts, once per CTA.
+__device__ __forceinline__ void close_cta(bool ok) {
+  const int any = __syncthreads_or(ok ? 0 : 1);
   if (any && threadIdx.x == 0) atomicAdd(&g_conv_tc_timeouts, 1);
-  return any;
 }
 
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
@@ -288,7 +287,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   const uint32_t tmem = *tmem_slot;
   bool ok = true;    // no wait of this thread's role ran out
-  int issued = 0;    // MMA warp: tiles whose MMAs were issued
 
   if (warp >= 8 && warp < 12) {
     // ---- copies: box rows t, t + 128, ... and all their chunks per thread
@@ -324,8 +322,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t leader;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(leader));
     const uint64_t a0 = smem_desc(box_s, kPlaneBytes, 128), b0 = smem_desc(w_s, kC * 16, 128);
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++issued) {
-      const int k = issued, st = k % kStages, ac = k & 1;
+    int k = 0;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++k) {
+      const int st = k % kStages, ac = k & 1;
       ok = mbar_wait(tempty(ac), ((k >> 1) & 1) ^ 1) && mbar_wait(full(st), (k / kStages) & 1);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
@@ -348,6 +347,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       mma_commit(empty(st), leader);
       mma_commit(tfull(ac), leader);
     }
+    // the last commit covers every MMA issued: none runs when the CTA frees its TMEM and shared
+    // memory, whoever gave up (bounded like the others; the epilogue waits for the same)
+    if (k > 0) ok = mbar_wait(tfull((k - 1) & 1), ((k - 1) >> 1) & 1) && ok;
     __syncwarp();
   } else {
     // ---- epilogue: warps 0..3 take the even units, 4..7 the odd ones; warp w can read TMEM lanes
@@ -399,12 +401,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     // out too
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-  if (cta_gave_up(ok)) {
-    // MMAs of up to two tiles may still be running: one more bounded wait, on the last commit,
-    // which covers those before it, before the TMEM and the shared memory they use are freed
-    if (warp == 12 && issued > 0) mbar_wait(tfull((issued - 1) & 1), ((issued - 1) >> 1) & 1);
-    __syncthreads();
-  }
+  close_cta(ok);
   if (warp == 0) {
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(TL::kTmemCols) : "memory");
@@ -421,7 +418,7 @@ __global__ void __launch_bounds__(kThreads) k_wait_probe() {
   if (threadIdx.x == 0) mbar_init(b, 1);
   __syncthreads();
   const bool stuck = threadIdx.x / 32 == blockIdx.x % (kThreads / 32);
-  cta_gave_up(mbar_wait(b, stuck ? 0 : 1));   // a fresh barrier passes parity 1
+  close_cta(mbar_wait(b, stuck ? 0 : 1));   // a fresh barrier passes parity 1
 }
 
 int g_sms = 0;
