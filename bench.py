@@ -63,7 +63,8 @@ def parse_args(argv=None):
                     help="coarse Gauss-Seidel kernels: levels of at most RESIDENT_MAX_N cells per axis smooth as "
                          "one cluster launch per phase with the displacement in shared memory, at most "
                          "CLUSTER_MAX_N as one cluster launch through L2, at most SPLIT_MAX_N with a thread per "
-                         "(vertex, case) (default: the library's)")
+                         "(vertex, case), others in a launch per colour (default: the library's, which stages "
+                         "every level above 16)")
     ap.add_argument("--coarse-forms", action="store_true",
                     help="after the timed region, time one Gauss-Seidel sweep of every coarse level in each kernel "
                          "form and V-cycles under several form settings (the cell's own hierarchy)")
@@ -421,8 +422,8 @@ def coarse_forms(hom, n, stream, dev):
     return {"sweep_us": sweep, "vcycle_ms": vc,
             "settings": "resident_max_n,cluster_max_n,split_max_n; library default " + ",".join(map(str, saved)),
             "note": "one homo_smooth sweep per level and form (the resident form times its shared-memory setup "
-                    "once per sweep; inside a V-cycle it runs many sweeps per launch), then homo_vcycle; levels "
-                    "above 16 that are a multiple of 4 run the staged kernel under every setting"}
+                    "once per sweep; inside a V-cycle it runs many sweeps per launch), then homo_vcycle; "
+                    "vertex: the per-colour form for all cases, staged above 16"}
 
 
 # ------------------------------------------------------------------ reference arm

@@ -389,19 +389,22 @@ int homo_autotune(homo_ctx* ctx, int flags, int* gs_cases, int* gs_block, double
  *    displacement in shared memory and the stencil rows of its own vertices in registers
  *    (half of them in shared memory at 14^3 and 16^3), and writes each update into the copies
  *    of the CTAs that read it; the colour passes are separated by the cluster's hardware
- *    barrier (default 16);
- *  - other levels of more than 16 cells per axis, a multiple of 4: one launch per colour pass that
- *    stages the stencil through shared memory while the pass before it runs, whatever the two
- *    sizes below say;
+ *    barrier (default 16). The size also governs the finest level of a cell that small: its
+ *    sweeps are then one launch each instead of the variants of homo_set_tuning;
  *  - other levels with at most cluster_max_n cells per axis: the same per-case cluster
  *    launch, reading the displacement and stencils through L2 (default 32);
- *  - larger levels with at most split_max_n cells per axis: one launch per colour pass with
+ *  - other levels with at most split_max_n cells per axis: one launch per colour pass with
  *    a thread per (vertex, load case), each loading a z-layer of 9 neighbours before its
  *    FMAs (default 32);
- *  - larger levels: one launch per colour pass with a thread per vertex and all 6 cases.
+ *  - other levels: one launch per colour pass for all 6 cases, which above 16 cells per axis
+ *    stages the stencil through shared memory while the pass before it runs, and at or below
+ *    takes a thread per vertex.
+ * While cluster_max_n and split_max_n are both at their defaults, levels above 16 cells per
+ * axis run the staged form, which is the fastest there; any other pair of sizes rules as above.
  * The small levels are bound by load latency and launch overhead, not by bytes: with the
  * default sweep counts a V-cycle of a 512^3 cell runs about 2,500 colour passes on levels
- * of 32^3 and below, 2,050 of them inside the launches of the first form. Sizes in [0, 1024]; 0 disables a form. Changing them drops the
+ * of 32^3 and below, 2,050 of them inside the launches of the first form. Sizes in [0, 1024];
+ * 0 disables a form. Changing them drops the
  * context's captured CUDA graphs. Where the device cannot launch the clusters, the next
  * form applies whatever the sizes say. homo_coarse_smoother reports the sizes and the
  * largest cluster of the L2 and of the resident form the device launches (-1: none);
@@ -414,15 +417,16 @@ int homo_coarse_smoother(const homo_ctx* ctx, int* resident_max_n, int* cluster_
 /* Autotuner of the coarse Gauss-Seidel forms. Times, on every smoothed coarse level of the
  * context's own hierarchy, the two smoothing phases of a V-cycle (the level's sweep count
  * from zero in colour order 0..7, then in order 7..0) in each form the level can take (the
- * thread-per-vertex form everywhere, the thread-per-(vertex, case) form up to 128^3, the
- * cluster forms up to 64^3 and where the device launches them), then sets the three sizes
+ * per-colour form for all cases everywhere, the thread-per-(vertex, case) form up to 128^3,
+ * the cluster forms up to 64^3 and where the device launches them), then sets the three sizes
  * of homo_set_coarse_smoother (each 0 or a level size) whose forms give the smallest sum
  * of those times, and caches them per (grid size, precision, sweep schedule) for the
  * process; flags HOMO_TUNE_RETIME ignores the cache. Needs a density; uses the coarse
  * levels' vectors, so call it between solves. The forms give bitwise the same iterates,
  * so the choice changes only the time. Outputs (host, nullable): the chosen sizes; ms:
- * 64 doubles, ms[4 l + k] the time of level l's two phases in form k (0 thread per
- * vertex, 1 thread per (vertex, case), 2 cluster through L2, 3 resident cluster), -1 where
+ * 64 doubles, ms[4 l + k] the time of level l's two phases in form k (0 per colour for all
+ * cases: staged above 16 cells per axis, thread per vertex at or below; 1 thread per (vertex,
+ * case), 2 cluster through L2, 3 resident cluster), -1 where
  * not timed (all -1 when the choice came from the cache). (The paper has no counterpart.) */
 int homo_autotune_coarse(homo_ctx* ctx, int flags, int* resident_max_n, int* cluster_max_n, int* split_max_n,
                          double* ms);

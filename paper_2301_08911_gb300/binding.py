@@ -354,11 +354,12 @@ class Homogenization:
 
     def set_coarse_smoother(self, resident_max_n: int, cluster_max_n: int, split_max_n: int):
         """Coarse Gauss-Seidel kernels by level size: at most resident_max_n cells per axis
-        smooth as one cluster launch per phase with the displacement in shared memory; larger
-        ones that are a multiple of 4 above 16 stage the stencil, a launch per colour; of the rest at
-        most cluster_max_n as one cluster launch through L2, at most split_max_n with a
-        thread per (vertex, case) per colour, larger levels with a thread per vertex
-        (0 disables a form)."""
+        smooth as one cluster launch per phase with the displacement in shared memory, of the
+        rest at most cluster_max_n as one cluster launch through L2, at most split_max_n with a
+        thread per (vertex, case) per colour, other levels in a launch per colour for all cases,
+        staged through shared memory above 16 (0 disables a form). With cluster_max_n and
+        split_max_n at their defaults (32, 32) all levels above 16 run staged. resident_max_n
+        also governs the finest level of a cell that small."""
         self._check(self.lib.homo_set_coarse_smoother(self.h, int(resident_max_n), int(cluster_max_n),
                                                       int(split_max_n)))
 
@@ -369,6 +370,7 @@ class Homogenization:
         self._check(self.lib.homo_coarse_smoother(self.h, *[ctypes.byref(x) for x in v]))
         return tuple(x.value for x in v)
 
+    # "vertex": the per-colour form for all cases (staged above 16 cells per axis)
     COARSE_FORMS = ("vertex", "item", "cluster", "resident")
 
     def autotune_coarse(self, retime: bool = False):

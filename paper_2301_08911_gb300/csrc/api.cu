@@ -215,10 +215,23 @@ int ensure_hierarchy(homo_ctx* c) {
   return HOMO_OK;
 }
 
-// A coarse level above the on-chip form's sizes smooths in the staged form (a launch per
-// colour, the stencil through shared memory) wherever its rows allow the 16-byte copies; the
-// sizes of homo_set_coarse_smoother choose among the other forms.
-bool coarse_staged(const homo::Level& lv) { return lv.n > kStagedMinN && coarse_tile_ok(lv); }
+// The form coarse level l >= 1 smooths in under the sizes (res, fuse, split) of
+// homo_set_coarse_smoother, for the dispatch and for the autotuner. A size that covers the level
+// asks for its form and gets it, but the default fuse and split say nothing about levels above
+// kStagedMinN: those, and every level there that no size covers, run the staged form (one sweep
+// of a 32^3 level with BF16 stencils: L2 clusters 75 us, staged 36 us).
+CoarseForm coarse_form(const homo_ctx* c, int l, int res, int fuse, int split) {
+  const homo::Level& lv = c->lev[l];
+  if (c->gs_resident > 0 && lv.n <= res && coarse_resident_ok(lv, c->gs_resident)) return kFormResident;
+  const bool large = lv.n > kStagedMinN && coarse_tile_ok(lv);
+  if (!large || fuse != kGsFuseDefault || split != kGsSplitDefault) {
+    if (c->gs_cluster > 0 && lv.n <= fuse) return kFormCluster;
+    if (lv.n <= split) return kFormItem;
+  }
+  return large ? kFormStaged : kFormVertex;
+}
+
+CoarseForm coarse_form(const homo_ctx* c, int l) { return coarse_form(c, l, c->gs_res_n, c->gs_fuse_n, c->gs_split_n); }
 
 // One 8-colour sweep. first: the sweep starts from x = 0 (x need not be cleared; only
 // valid with colours in increasing order).
@@ -236,13 +249,13 @@ int smooth_level(homo_ctx* c, int l, bool reverse, const float* f, float* x, boo
       KL(c, HOMO_KC_FINE_GS, 1, launch_fine_gs(c, reverse ? 3 - k : k, reverse, f, x, fz, fmean));
     return HOMO_OK;
   }
-  const bool staged = coarse_staged(c->lev[l]);
+  const CoarseForm form = coarse_form(c, l);
   for (int k = 0; k < 8; ++k) {
     const int col = reverse ? 7 - k : k;
-    if (staged)
+    if (form == kFormStaged)
       KL(c, HOMO_KC_COARSE_GS, 1,
          launch_coarse_gs_tile(c->lev[l], col, f, x, fz, chained || k > 0 ? 1 : 0, c->stream));
-    else if (c->lev[l].n <= c->gs_split_n)
+    else if (form == kFormItem)
       KL(c, HOMO_KC_COARSE_GS, 1, launch_coarse_gs_item(c->lev[l], col, f, x, fz, c->stream));
     else KL(c, HOMO_KC_COARSE_GS, 1, launch_coarse_gs(c->lev[l], col, f, x, fz, c->stream));
   }
@@ -251,19 +264,19 @@ int smooth_level(homo_ctx* c, int l, bool reverse, const float* f, float* x, boo
 
 // sweeps 8-colour sweeps on level l; first: the first sweep starts from x = 0. A small
 // coarse level runs them all as one launch of per-case clusters (displacement and stencil on
-// the chip up to gs_res_n cells per axis, read through L2 up to gs_fuse_n), larger
-// levels one launch per colour (the per-colour launches of the small levels are mostly
-// launch and load latency).
+// the chip, or read through L2), other levels one launch per colour (the per-colour launches
+// of the small levels are mostly launch and load latency).
 int smooth_level_sweeps(homo_ctx* c, int l, bool reverse, const float* f, float* x, int sweeps,
                         bool first = false) {
   if (sweeps < 1) return HOMO_OK;
-  if (l >= 1 && c->gs_resident > 0 && c->lev[l].n <= c->gs_res_n && coarse_resident_ok(c->lev[l], c->gs_resident)) {
+  const CoarseForm form = l >= 1 ? coarse_form(c, l) : kFormVertex;
+  if (form == kFormResident) {
     KL(c, HOMO_KC_COARSE_GS, 1,
        launch_coarse_gs_resident(c->lev[l], sweeps, reverse ? 1 : 0, first && !reverse ? 1 : 0, f, x,
                                  c->gs_resident, c->stream));
     return HOMO_OK;
   }
-  if (l >= 1 && c->gs_cluster > 0 && c->lev[l].n <= c->gs_fuse_n && !coarse_staged(c->lev[l])) {
+  if (form == kFormCluster) {
     KL(c, HOMO_KC_COARSE_GS, 1,
        launch_coarse_gs_sweeps(c->lev[l], sweeps, reverse ? 1 : 0, first && !reverse ? 1 : 0, f, x,
                                c->gs_cluster, c->stream));
@@ -1374,14 +1387,9 @@ std::mutex g_coarse_tune_mu;
 // (grid size, precision, level-1 sweeps, sweep growth, levels) -> (resident, cluster, split)
 std::map<std::array<int, 5>, std::array<int, 3>> g_coarse_tune_cache;
 
-// The coarse Gauss-Seidel form smooth_level_sweeps picks for level l under sizes (r, c, s):
-// 0 vertex, 1 item, 2 cluster, 3 resident.
-int coarse_form(const homo_ctx* ctx, int l, int r, int c, int s) {
-  const homo::Level& lv = ctx->lev[l];
-  if (ctx->gs_resident > 0 && lv.n <= r && homo::coarse_resident_ok(lv, ctx->gs_resident)) return 3;
-  if (ctx->gs_cluster > 0 && lv.n <= c) return 2;
-  return lv.n <= s ? 1 : 0;
-}
+// The slot of a form in the autotuner's times: 0 the form no size asks for (staged above
+// kStagedMinN, a thread per vertex at or below), 1 item, 2 cluster, 3 resident.
+int form_slot(CoarseForm f) { return f == kFormStaged ? kFormVertex : f; }
 }  // namespace
 
 int homo_autotune_coarse(homo_ctx* ctx, int flags, int* resident_max_n, int* cluster_max_n, int* split_max_n,
@@ -1430,7 +1438,7 @@ int homo_autotune_coarse(homo_ctx* ctx, int flags, int* resident_max_n, int* clu
         ctx->gs_res_n = kSizes[k][0];
         ctx->gs_fuse_n = kSizes[k][1];
         ctx->gs_split_n = kSizes[k][2];
-        if (coarse_form(ctx, l, ctx->gs_res_n, ctx->gs_fuse_n, ctx->gs_split_n) != k) continue;
+        if (form_slot(coarse_form(ctx, l)) != k) continue;
         const int reps = lv.n <= 32 ? 4 : 1;
         for (int rep = -1; rep < reps && rc == HOMO_OK; ++rep) {   // rep -1: warm-up
           if (rep == 0 && cudaEventRecord(a, ctx->stream) != cudaSuccess) rc = HOMO_ECUDA;
@@ -1463,7 +1471,7 @@ int homo_autotune_coarse(homo_ctx* ctx, int flags, int* resident_max_n, int* clu
         for (int sp : cand) {
           double tot = 0.0;
           for (int l = 1; l < last && tot >= 0.0; ++l) {
-            const double v = t[l][coarse_form(ctx, l, r, c, sp)];
+            const double v = t[l][form_slot(coarse_form(ctx, l, r, c, sp))];
             tot = v < 0.0 ? -1.0 : tot + v;
           }
           if (tot >= 0.0 && (best_t < 0.0 || tot < best_t)) {

@@ -27,6 +27,8 @@ constexpr int kPlanes = 18;
 constexpr int kStencil = 243;
 constexpr int kMaxLevels = 16;
 constexpr int kRedBlock = 256;          // threads per block of every reduction kernel
+constexpr int kGsFuseDefault = 32, kGsSplitDefault = 32;   // sizes of homo_set_coarse_smoother
+constexpr int kStagedMinN = 16;         // coarse levels above it have the staged smoother
 constexpr int kOcPasses = 8;            // OC multiplier search passes (15 candidates each)
 constexpr int kOcKernels = 2 + kOcPasses;   // kernels one OC update launches
 
@@ -118,6 +120,9 @@ enum SlotF : int {
   F_BETA = 60      // beta_c [6]
 };
 
+// Kernel forms of the coarse Gauss-Seidel sweeps.
+enum CoarseForm { kFormVertex = 0, kFormItem = 1, kFormCluster = 2, kFormResident = 3, kFormStaged = 4 };
+
 struct homo_ctx_impl;
 
 }  // namespace homo
@@ -184,15 +189,15 @@ struct homo_ctx {
   // fine Gauss-Seidel variant: load cases per thread (3 or 6) and threads per block
   // (128 or 256); set by homo_set_tuning / homo_autotune
   int gs_cases = 3, gs_block = 256;
-  // coarse Gauss-Seidel kernels (homo_set_coarse_smoother): levels with at most gs_fuse_n
-  // cells per axis run every sweep of a smoothing phase as one thread-block-cluster launch,
-  // levels with at most gs_split_n one launch per colour with a thread per (vertex, case),
-  // larger levels one launch per colour with a thread per vertex; gs_cluster: the largest
-  // cluster the device launches (-1: none, per-colour launches everywhere)
-  int gs_fuse_n = 32, gs_split_n = 32, gs_cluster = -1;
-  // levels with at most gs_res_n cells per axis (16 at most) keep each case's displacement
-  // in the clusters' shared memory and its stencil rows in their registers instead;
-  // gs_resident: the largest cluster of that form the device launches (-1: none)
+  // coarse Gauss-Seidel kernels (homo_set_coarse_smoother; coarse_form in api.cu decides): levels
+  // with at most gs_fuse_n cells per axis run every sweep of a smoothing phase as one
+  // thread-block-cluster launch, levels with at most gs_split_n one launch per colour with a
+  // thread per (vertex, case), other levels one launch per colour for all cases; gs_cluster: the
+  // largest cluster the device launches (-1: none, per-colour launches everywhere)
+  int gs_fuse_n = homo::kGsFuseDefault, gs_split_n = homo::kGsSplitDefault, gs_cluster = -1;
+  // levels with at most gs_res_n cells per axis (16 at most; the finest level too) keep each
+  // case's displacement in the clusters' shared memory and its stencil rows in their registers
+  // instead; gs_resident: the largest cluster of that form the device launches (-1: none)
   int gs_res_n = 16, gs_resident = -1;
 
   cudaGraphExec_t cg_graph[2] = {nullptr, nullptr};
@@ -281,7 +286,6 @@ cudaError_t launch_coarse_gs(const Level& L, int colour, const float* f, float* 
 // One colour pass of level L with the stencil staged in shared memory (coarse_tile_ok: rows are
 // 16-byte aligned); bitwise launch_coarse_gs. chained: the launch before on s was the colour
 // pass before of the same smoothing, whose end this one overlaps.
-constexpr int kStagedMinN = 16;   // levels above this many cells per axis take it
 bool coarse_tile_ok(const Level& L);
 cudaError_t launch_coarse_gs_tile(const Level& L, int colour, const float* f, float* x, int first, int chained,
                                   cudaStream_t s);
