@@ -369,9 +369,13 @@ int homo_prolong_add(homo_ctx* ctx, int level, const float* coarse, float* fine)
  * The finest-level Gauss-Seidel pass (Eq. 15-16) is compiled in four variants: 3 or 6
  * load cases per thread (3: the cases are split over two thread groups, each rebuilding
  * the coupling blocks; 6: blocks built once, more registers) times 128 or 256 threads
- * per block (more where a row has more x pairs). All four compute bitwise the same result;
- * which is fastest depends on the grid size. homo_set_tuning selects one (default 3, 256).
- * homo_autotune times one symmetric sweep pair of each on the context's own moduli and loads (needs a density;
+ * per block (a block holds whole rows of x pairs: above 256 cells per axis both are one row).
+ * All four compute bitwise the same result; which is fastest depends on the grid size.
+ * homo_set_tuning selects one (default 3, 256). It runs wherever the finest level is swept in
+ * launches of two colours; a cell of at most resident_max_n cells per axis
+ * (homo_set_coarse_smoother, default 16) takes its one-launch sweep instead.
+ * homo_autotune times one symmetric sweep pair of each variant, whatever that size, on the
+ * context's own moduli and loads (needs a density;
  * uses the solver's scratch, so call it between solves), selects the fastest and caches
  * the choice per grid size for the process; flags HOMO_TUNE_RETIME ignores the cache.
  * Outputs (host, nullable): the chosen variant; ms: 4 times per sweep of the variants

@@ -233,6 +233,14 @@ CoarseForm coarse_form(const homo_ctx* c, int l, int res, int fuse, int split) {
 
 CoarseForm coarse_form(const homo_ctx* c, int l) { return coarse_form(c, l, c->gs_res_n, c->gs_fuse_n, c->gs_split_n); }
 
+// One 8-colour sweep of the finest level in its four launches of two colours, in the variant of
+// homo_set_tuning.
+int fine_sweep(homo_ctx* c, bool reverse, const float* f, float* x, int first, const float* fmean) {
+  for (int k = 0; k < 4; ++k)
+    KL(c, HOMO_KC_FINE_GS, 1, launch_fine_gs(c, reverse ? 3 - k : k, reverse, f, x, first, fmean));
+  return HOMO_OK;
+}
+
 // One 8-colour sweep. first: the sweep starts from x = 0 (x need not be cleared; only
 // valid with colours in increasing order).
 // fmean (finest level only): plane means subtracted from f, or null. chained: the launch before
@@ -245,9 +253,7 @@ int smooth_level(homo_ctx* c, int l, bool reverse, const float* f, float* x, boo
       KL(c, HOMO_KC_FINE_GS, 1, launch_fine_gs_resident(c, reverse, f, x, fz, fmean));
       return HOMO_OK;
     }
-    for (int k = 0; k < 4; ++k)
-      KL(c, HOMO_KC_FINE_GS, 1, launch_fine_gs(c, reverse ? 3 - k : k, reverse, f, x, fz, fmean));
-    return HOMO_OK;
+    return fine_sweep(c, reverse, f, x, fz, fmean);
   }
   const CoarseForm form = coarse_form(c, l);
   for (int k = 0; k < 8; ++k) {
@@ -1309,7 +1315,8 @@ int homo_autotune(homo_ctx* ctx, int flags, int* gs_cases, int* gs_block, double
   }
   if (best < 0) {
     // time one symmetric sweep pair (8 launches of two colours) of each variant on the context's
-    // own moduli and loads, into the CG scratch vector z (free between solves)
+    // own moduli and loads, into the CG scratch vector z (free between solves); never the
+    // one-launch sweep of a small cell, which has no variants
     RET(ensure_loads(ctx));
     cudaEvent_t a = nullptr, b = nullptr;
     if (cudaEventCreate(&a) != cudaSuccess || cudaEventCreate(&b) != cudaSuccess) {
@@ -1322,12 +1329,12 @@ int homo_autotune(homo_ctx* ctx, int flags, int* gs_cases, int* gs_block, double
     for (int k = 0; k < 4 && rc == HOMO_OK; ++k) {
       ctx->gs_cases = kVar[k][0];
       ctx->gs_block = kVar[k][1];
-      rc = smooth_level(ctx, 0, false, ctx->f, ctx->z, true);            // warm-up, from zero
+      rc = fine_sweep(ctx, false, ctx->f, ctx->z, 1, nullptr);            // warm-up, from zero
       if (rc != HOMO_OK) break;
       if (cudaEventRecord(a, ctx->stream) != cudaSuccess) { rc = HOMO_ECUDA; break; }
       for (int rep = 0; rep < 2 && rc == HOMO_OK; ++rep) {
-        rc = smooth_level(ctx, 0, false, ctx->f, ctx->z);
-        if (rc == HOMO_OK) rc = smooth_level(ctx, 0, true, ctx->f, ctx->z);
+        rc = fine_sweep(ctx, false, ctx->f, ctx->z, 0, nullptr);
+        if (rc == HOMO_OK) rc = fine_sweep(ctx, true, ctx->f, ctx->z, 0, nullptr);
       }
       if (rc != HOMO_OK) break;
       float t = 0.f;

@@ -102,3 +102,15 @@ def test_autotuner_times_the_forms_it_names(B):
         for form in row:
             want += reps * 2 * (1 if form in ("cluster", "resident") else 8 * sweeps)
     assert sorted(times) == [1, 2, 3, 4] and got == want
+
+
+@pytest.mark.parametrize("n", [8, 16, 24])
+def test_fine_autotuner_times_its_variants_on_small_cells_too(B, n):
+    """Per variant five sweeps of four launches; a cell of at most 16 would take one launch a sweep."""
+    hom = B.Homogenization(n)
+    hom.set_density(cuda(uniform_density(n, 970, 0.05, 1.0)))
+    hom.autotune(retime=True)
+    before = hom.launch_count
+    choice, times = hom.autotune(retime=True)
+    assert hom.launch_count - before == 4 * 5 * 4
+    assert len(times) == 4 and times[choice] == min(times.values())
