@@ -214,10 +214,11 @@ SOLVE_FLOP = 6 * 15 + 30                # 3x3 LDL^T and 6 solves
 def algorithmic_work(kc: str, n: int, sweeps: int = 1):
     N = n ** 3
     if kc == "fine_gs":
-        # pass of two colours (the x pairs of the rows of one parity): E 4N, u 72N, f 18N and
-        # 18N written (112N); in the first sweep from zero only the rows of earlier passes are
-        # read (27N on average: 67N). 1 of 2*sweeps sweeps.
-        full_b, first_b = 112 * N, 67 * N
+        # pass of two colours (the x pairs of the rows of one parity): E 4N, u of the other three
+        # parities 54N and of the second colour 9N (the first one's is overwritten unread), f 18N
+        # and 18N written (103N); in the first sweep from zero only the rows of earlier passes
+        # are read (27N on average: 67N). 1 of 2*sweeps sweeps.
+        full_b, first_b = 103 * N, 67 * N
         full_f = (576 + 26 * 54 + SOLVE_FLOP) * 2 * N / 4
         first_f = (288 + 13 * 54 + SOLVE_FLOP) * 2 * N / 4
         w = 1.0 / (2 * sweeps)
