@@ -280,7 +280,8 @@ int tiled_zchunk(int n) {
   return chunk;
 }
 
-// Planes per block where nothing is summed (the chunks of the dots are part of their rounding).
+// Planes per block of the product where nothing is summed (the chunks of the dots are part of
+// their rounding).
 // A block's first planes cost little (its neighbour's last ones, from L2), so short chunks
 // that even the SMs out win until there are some ten rounds of long ones. Product with 1 / 2 /
 // 8 / 16 planes: 16^3 9 / 13 / 33 / 60 us, 128^3 250 / 228 / 238 / 267, 160^3 - / 446 / 479 / 478,
@@ -291,6 +292,19 @@ int tiled_zchunk_free(int n) {
   const long xy = static_cast<long>((n + TX - 1) / TX) * ((n + TY - 1) / TY);
   if (xy * ((n + 15) / 16) >= 4096) return 16;
   return xy * ((n + 1) / 2) >= 1216 ? 2 : 1;
+}
+
+// Planes per block of the residual and the Chebyshev steps. They also read b (and the iterates) and
+// gain less from short chunks than the product: those win while the cell has fewer than some
+// 1000 tile planes; from there on the chunks of the dots, at most 16. V-cycle residual with
+// the product's chunk / the dots' chunk: 16^3 10.4 / 21, 32^3 10.3 / 21, 48^3 23 / 29, 64^3 37.2 /
+// 36.9, 80^3 82.8 / 77.0, 112^3 194.6 / 194.7, 160^3 486.6 / 486.3, 192^3 830 / 807, 224^3 1327 /
+// 1271 us; 320^3 with 16 / 40 planes 3646 / 3712 us. Chebyshev step: 32^3 10.3 / 21.6, 64^3
+// 35.3 / 33.9, 112^3 199.9 / 203.5, 224^3 1360 / 1327 us.
+int tiled_zchunk_residual(int n) {
+  const long xy = static_cast<long>((n + TX - 1) / TX) * ((n + TY - 1) / TY);
+  const int dots = tiled_zchunk(n);
+  return xy * n < 1000 ? tiled_zchunk_free(n) : (dots < 16 ? dots : 16);
 }
 
 }  // namespace
@@ -336,7 +350,7 @@ cudaError_t launch_fine_tiled(const homo_ctx* c, int mode, const float* u, const
                               double* part, int* grid_out, const float* bmean, float c0, float c1,
                               const float* ulo) {
   const int n = c->n;
-  const int zc = mode == 1 || mode == 2 ? tiled_zchunk(n) : tiled_zchunk_free(n);
+  const int zc = mode == 1 || mode == 2 ? tiled_zchunk(n) : mode == 7 ? tiled_zchunk_free(n) : tiled_zchunk_residual(n);
   dim3 grid((n + TX - 1) / TX, (n + TY - 1) / TY, (n + zc - 1) / zc);
   if (grid_out) *grid_out = static_cast<int>(grid.x * grid.y * grid.z);
   switch (mode) {
