@@ -16,10 +16,12 @@ namespace {
 // 8-byte load, a warp's loads are whole lines) and one value beside it, so a sweep moves
 // 4 x 112 B per vertex of u, f and E in whole sectors; a launch per colour read all of u
 // eight times and touched half of every sector of f and of the written u (8 x 109 B measured).
-// The bound is the FMA pipe (per vertex and sweep 1404 FMA and about 350 for the blocks A_d)
-// shared with the load pipe (26 x 18 values per vertex at 4 B, twice through L1 for the
-// stride-2 side values); ncu at 128^3: issue active 71 %, about 1.7 integer instructions per
-// load for the addresses, DRAM 30 %. One sweep, against a launch per colour: 24^3 82 -> 43 us,
+// Of those 112 B, 9 are the first colour's old values, which are overwritten unread but share
+// their sectors with the second colour's. A neighbour row's pair is loaded once per vertex of
+// the pair, the second time from L1. The bound is instruction issue: about 4,260 per vertex and
+// sweep, of which 1404 are the scalar FMAs, 350 per case group build the blocks A_d and about 1.7
+// integer instructions go with each load; ncu at 160^3, full pass: issue active 74 %, shared/L1
+// data pipe 52 %, FMA pipe 42 %, DRAM 36 %, 23 warps an SM (80 registers). One sweep, against a launch per colour: 24^3 82 -> 43 us,
 // 64^3 98 -> 58 us, 256^3 3350 -> 2460 us. Measured and not adopted: plane pointers as kernel
 // parameters (fewer integer instructions, 2570 us: the loads come later).
 //
