@@ -296,15 +296,15 @@ int tiled_zchunk_free(int n) {
 
 // Planes per block of the residual and the Chebyshev steps. They also read b (and the iterates) and
 // gain less from short chunks than the product: those win while the cell has fewer than some
-// 1000 tile planes; from there on the chunks of the dots, at most 16. V-cycle residual with
+// 2000 tile planes; from there on the chunks of the dots, at most 16. V-cycle residual with
 // the product's chunk / the dots' chunk: 16^3 10.4 / 21, 32^3 10.3 / 21, 48^3 23 / 29, 64^3 37.2 /
-// 36.9, 80^3 82.8 / 77.0, 112^3 194.6 / 194.7, 160^3 486.6 / 486.3, 192^3 830 / 807, 224^3 1327 /
+// 36.9 (but a whole V-cycle 505.0 / 506.4), 80^3 82.8 / 77.0, 112^3 194.6 / 194.7, 160^3 486.6 / 486.3, 192^3 830 / 807, 224^3 1327 /
 // 1271 us; 320^3 with 16 / 40 planes 3646 / 3712 us. Chebyshev step: 32^3 10.3 / 21.6, 64^3
 // 35.3 / 33.9, 112^3 199.9 / 203.5, 224^3 1360 / 1327 us.
 int tiled_zchunk_residual(int n) {
   const long xy = static_cast<long>((n + TX - 1) / TX) * ((n + TY - 1) / TY);
   const int dots = tiled_zchunk(n);
-  return xy * n < 1000 ? tiled_zchunk_free(n) : (dots < 16 ? dots : 16);
+  return xy * n < 2000 ? tiled_zchunk_free(n) : (dots < 16 ? dots : 16);
 }
 
 }  // namespace
