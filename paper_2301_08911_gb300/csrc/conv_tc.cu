@@ -408,7 +408,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-// The bounded wait and the CTA's verdict on their own: in CTA b one warp, b mod 13, waits on an
+// The bounded wait and the CTA's closing vote on their own: in CTA b one warp, b mod 13, waits on an
 // mbarrier that no one arrives on and gives up after kWaitLimit polls, the others' waits complete
 // at once; the CTA counts one timeout whichever warp it was (no MMA is issued here, so nothing is
 // left in flight).
